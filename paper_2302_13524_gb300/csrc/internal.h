@@ -146,12 +146,35 @@ long long solver_dispatch_mixed(int N, int G, int what, const SolverParams *p, c
 cudaError_t launch_fill_synthetic(float *y, size_t n, unsigned seed, cudaStream_t s);
 
 // ---- BF16 tensor-core GEMM (gemm_tc.cu) ---------------------------------------
-// C[M][N] (FP32, row stride ldc) = A B^T with A [M][K], B [N][K] BF16, K-contiguous
-// rows of stride lda, ldb.  Needs M, N >= 128, K >= 64, K, lda, ldb multiples of 8
-// and 16-byte aligned A, B; *err (device) is raised when a barrier wait ran out.
-bool gemm_tc_supported(int M, int N, int K, const void *A, int lda, const void *B, int ldb);
-cudaError_t gemm_tc(int M, int N, int K, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
-                    float *C, int ldc, int *err, cudaStream_t s);
+// C[M][N] (FP32, row stride ldc) = sum_k A(m, k) B(n, k), then an elementwise
+// step.  An operand is BF16 with rows of stride ld elements: [M or N][K]
+// (k_contiguous) or [K][M or N].  Needs M, N >= 128, K >= 64, the contiguous
+// dimension and ld of each multiples of 8 and 16-byte aligned pointers; *err
+// (device) is raised when a barrier wait ran out.
+struct GemmOperand {
+    const __nv_bfloat16 *p;
+    int ld;
+    bool k_contiguous;
+};
+// What becomes of the product x at (row, col); every matrix has row stride ldc.
+//   GEMM_STORE      C = x
+//   GEMM_BIAS       C = x + bias[col]
+//   GEMM_BIAS_GELU  C = x + bias[col], H = GELU(C)
+//   GEMM_GELU_BACK  H = x GELU'(Z)
+//   GEMM_ADAM       one Adam update of w, m, v with gradient x, H = the new w
+enum { GEMM_STORE = 0, GEMM_BIAS, GEMM_BIAS_GELU, GEMM_GELU_BACK, GEMM_ADAM };
+struct GemmEpilogue {
+    int kind = GEMM_STORE;
+    float *C = nullptr;
+    const float *bias = nullptr, *Z = nullptr;
+    __nv_bfloat16 *H = nullptr;
+    float *w = nullptr, *m = nullptr, *v = nullptr;
+    float lr = 0.f, c1 = 1.f, c2 = 1.f;  // step size and bias corrections
+    bool wide = false;  // set by gemm_tc: 16-byte accesses are aligned
+};
+bool gemm_tc_supported(int M, int N, int K, const GemmOperand &A, const GemmOperand &B);
+cudaError_t gemm_tc(int M, int N, int K, const GemmOperand &A, const GemmOperand &B, int ldc, const GemmEpilogue &E,
+                    int *err, cudaStream_t s);
 
 // ---- learned initialiser (mlp.cu) --------------------------------------------
 // rows of y (B of them) -> features -> network -> starts T scaled to the

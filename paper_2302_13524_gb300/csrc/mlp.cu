@@ -6,9 +6,11 @@
 // that feed the products; activations enter the products in BF16; every
 // product accumulates in FP32 (mma.sync m16n8k16 BF16 tensor-core steps).  The
 // loss is the mean squared error over every output, or its phase-invariant
-// form (each target row rotated onto the output row first).  One GEMM kernel serves
-// the forward products X W^T, the input gradients dZ W and the weight
-// gradients dZ^T H through generic element strides.
+// form (each target row rotated onto the output row first).  The forward
+// products X W^T, the input gradients dZ W and the weight gradients dZ^T H run
+// on the tensor cores with the layer's elementwise step as their epilogue
+// (gemm_tc.cu); this file's mma.sync kernel, through generic element strides,
+// takes the shapes that does not.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -18,6 +20,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "mlp_math.cuh"
 #include "tmr.h"
 
 namespace tmr {
@@ -117,37 +120,6 @@ static void gemm_sync(int M, int N, int K, const __nv_bfloat16 *A, long long sam
     k_gemm_bf16<<<grid, 128, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, N);
 }
 
-// out[c][r] = in[r][c] for an rows x cols BF16 matrix (row strides ldi, ldo);
-// 32 x 32 tiles through shared memory, block (32, 8)
-__global__ void k_transpose_bf16(int rows, int cols, const __nv_bfloat16 *__restrict__ in, long long ldi,
-                                 __nv_bfloat16 *__restrict__ out, long long ldo)
-{
-    __shared__ __nv_bfloat16 t[32][34];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int r = r0 + j, c = c0 + threadIdx.x;
-        t[j][threadIdx.x] = (r < rows && c < cols) ? in[(size_t)r * ldi + c] : __float2bfloat16(0.f);
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int c = c0 + j, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) out[(size_t)c * ldo + r] = t[threadIdx.x][j];
-    }
-}
-
-static void transpose_bf16(int rows, int cols, const __nv_bfloat16 *in, long long ldi, __nv_bfloat16 *out,
-                           cudaStream_t s)
-{
-    dim3 grid((cols + 31) / 32, (rows + 31) / 32);
-    k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(rows, cols, in, ldi, out, rows);
-}
-
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float x)
-{
-    return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
-}
-
 // Z += b (per column); H = GELU(Z) in BF16 (gelu != 0) or Z itself copied to out.
 __global__ void k_bias_act(int B, int N, float *Z, const float *b, __nv_bfloat16 *H, int gelu)
 {
@@ -159,55 +131,65 @@ __global__ void k_bias_act(int B, int N, float *Z, const float *b, __nv_bfloat16
     }
 }
 
-// dY = 2 (Y - T) / (B n); per-block partial sums of (Y - T)^2 into part
-__global__ void k_mse(int B, int N, const float *Y, const float *T, __nv_bfloat16 *dY, float *part)
+// One block per row: dY = 2 (Y - T) / (B N) and the row's sum of (Y - T)^2
+// into part[row].  phase != 0 (the phase-invariant loss): the target row, read
+// as t = T[:n] + i T[n:], n = N / 2, is first rotated onto the output row
+// y = Y[:n] + i Y[n:]: t conj(c) / |c|, c = sum conj(y) t (unrotated where
+// c = 0).  Sums in block_sum order.
+__global__ void __launch_bounds__(256) k_loss_rows(int B, int N, int phase, const float *Y, const float *T,
+                                                   __nv_bfloat16 *dY, float *part)
 {
-    const size_t total = (size_t)B * N;
-    const float sc = 2.f / (float)total;
-    float acc = 0.f;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const float e = Y[i] - T[i];
-        acc = fmaf(e, e, acc);
-        dY[i] = __float2bfloat16(sc * e);
-    }
-    __shared__ float red[32], out[1];
-    float v[1] = {acc};
-    block_sum<1>(v, red, out);
-    if (threadIdx.x == 0) part[blockIdx.x] = out[0];
-}
-
-// Phase-invariant loss: row r of T, read as t = T[:n] + i T[n:], rotated onto
-// the output row y = Y[:n] + i Y[n:]: Ta = t conj(c) / |c|, c = sum conj(y) t
-// (unrotated where c = 0).  One block per row; the sum in block_sum order.
-__global__ void k_align_targets(int n, const float *Y, const float *T, float *Ta)
-{
-    const size_t o = (size_t)blockIdx.x * 2 * n;
+    const size_t o = (size_t)blockIdx.x * N;
     const float *y = Y + o, *t = T + o;
-    float cr = 0.f, ci = 0.f;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const float yr = y[k], yi = y[n + k], tr = t[k], ti = t[n + k];
-        cr = fmaf(yr, tr, fmaf(yi, ti, cr));
-        ci = fmaf(yr, ti, fmaf(-yi, tr, ci));
-    }
     __shared__ float red[64], res[2];
-    float v[2] = {cr, ci};
-    block_sum<2>(v, red, res);
-    const float ac = sqrtf(res[0] * res[0] + res[1] * res[1]);
-    const float rr = ac > 0.f ? res[0] / ac : 1.f, ri = ac > 0.f ? -res[1] / ac : 0.f;  // conj(c) / |c|
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const float tr = t[k], ti = t[n + k];
-        Ta[o + k] = tr * rr - ti * ri;
-        Ta[o + n + k] = tr * ri + ti * rr;
+    const float sc = 2.f / (float)((size_t)B * N);
+    float acc = 0.f;
+    if (phase) {
+        const int n = N / 2;
+        float cr = 0.f, ci = 0.f;
+#pragma unroll 4
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const float yr = y[k], yi = y[n + k], tr = t[k], ti = t[n + k];
+            cr = fmaf(yr, tr, fmaf(yi, ti, cr));
+            ci = fmaf(yr, ti, fmaf(-yi, tr, ci));
+        }
+        float v[2] = {cr, ci};
+        block_sum<2>(v, red, res);
+        const float ac = sqrtf(res[0] * res[0] + res[1] * res[1]);
+        const float rr = ac > 0.f ? res[0] / ac : 1.f, ri = ac > 0.f ? -res[1] / ac : 0.f;  // conj(c) / |c|
+#pragma unroll 4
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const float tr = t[k], ti = t[n + k];
+            const float e0 = y[k] - (tr * rr - ti * ri), e1 = y[n + k] - (tr * ri + ti * rr);
+            acc = fmaf(e0, e0, acc);
+            acc = fmaf(e1, e1, acc);
+            dY[o + k] = __float2bfloat16(sc * e0);
+            dY[o + n + k] = __float2bfloat16(sc * e1);
+        }
+    } else {
+#pragma unroll 4
+        for (int k = threadIdx.x; k < N; k += blockDim.x) {
+            const float e = y[k] - t[k];
+            acc = fmaf(e, e, acc);
+            dY[o + k] = __float2bfloat16(sc * e);
+        }
     }
+    __syncthreads();  // res is read before red and res are used again
+    float v[1] = {acc};
+    block_sum<1>(v, red, res);
+    if (threadIdx.x == 0) part[blockIdx.x] = res[0];
 }
 
-__global__ void k_loss_finish(int nparts, const float *part, float total, float *loss)
+// loss = sum of the parts / total, FP64, one block of 256 threads (one thread
+// walking the parts took longer than any product of the step)
+__global__ void __launch_bounds__(256) k_loss_finish(int nparts, const float *part, float total, float *loss)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nparts; i++) s += part[i];
-        *loss = (float)(s / total);
-    }
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 256) s += part[i];
+    __shared__ double red[8], out[1];
+    double v[1] = {s};
+    block_sum<1>(v, red, out);
+    if (threadIdx.x == 0) *loss = (float)(out[0] / total);
 }
 
 // dZ = dH .* GELU'(Z) -> BF16
@@ -217,32 +199,75 @@ __global__ void k_gelu_back(size_t n, const float *dH, const float *Z, __nv_bflo
         dZ[i] = __float2bfloat16(dH[i] * gelu_grad_f(Z[i]));
 }
 
-// db[c] = sum_r dZ[r][c] (dZ BF16 [B][N])
-__global__ void k_colsum(int B, int N, const __nv_bfloat16 *dZ, float *db)
+// Bias gradients of the three layers in one launch: g[c] = sum_r dZ[r][c] (dZ
+// BF16 [B][N]), and with adam != 0 the biases' Adam update instead of storing
+// it.  A block of 32 x 8 threads takes 32 columns of one layer, thread (c, r)
+// the rows r, r + 8, ...  (One thread per column, walking all rows, used 16
+// blocks of the chip for 20 us a layer.)
+struct BiasLayer {
+    const __nv_bfloat16 *dZ;
+    int N, block0;  // columns; first block of the layer
+    float *g, *w, *m, *v;
+    __nv_bfloat16 *wb;
+};
+struct BiasLayers {
+    BiasLayer l[3];
+};
+__global__ void __launch_bounds__(256) k_bias_grad(int B, const __grid_constant__ BiasLayers P, int adam, float lr,
+                                                   float c1, float c2)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
+    const BiasLayer &L = P.l[(int)blockIdx.x >= P.l[2].block0 ? 2 : (int)blockIdx.x >= P.l[1].block0 ? 1 : 0];
+    const int c = ((int)blockIdx.x - L.block0) * 32 + threadIdx.x;
+    __shared__ float red[8][33];
     float s = 0.f;
-    for (int r = 0; r < B; r++) s += __bfloat162float(dZ[(size_t)r * N + c]);
-    db[c] = s;
+    if (c < L.N) {
+#pragma unroll 8
+        for (int r = threadIdx.y; r < B; r += 8) s += __bfloat162float(L.dZ[(size_t)r * L.N + c]);
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y != 0 || c >= L.N) return;
+#pragma unroll
+    for (int r = 1; r < 8; r++) s += red[r][threadIdx.x];
+    if (!adam) {
+        L.g[c] = s;
+        return;
+    }
+    float w = L.w[c], m = L.m[c], v = L.v[c];
+    adam_update(w, s, m, v, lr, c1, c2);
+    L.w[c] = w;
+    L.m[c] = m;
+    L.v[c] = v;
+    L.wb[c] = __float2bfloat16(w);
 }
 
+// x -> BF16, four values a thread and step where both are aligned for it
 __global__ void k_to_bf16(size_t n, const float *x, __nv_bfloat16 *y)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16(x[i]);
+    const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    size_t done = 0;
+    if (((reinterpret_cast<uintptr_t>(x) & 15) | (reinterpret_cast<uintptr_t>(y) & 7)) == 0) {
+        const size_t n4 = n / 4;
+#pragma unroll 4
+        for (size_t i = t0; i < n4; i += step) {
+            const float4 v = reinterpret_cast<const float4 *>(x)[i];
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            reinterpret_cast<uint2 *>(y)[i] =
+                make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        }
+        done = 4 * n4;
+    }
+    for (size_t i = done + t0; i < n; i += step) y[i] = __float2bfloat16(x[i]);
 }
 
 __global__ void k_adam(size_t n, float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, float lr,
                        float c1, float c2)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = 0.9f * m[i] + 0.1f * gi;
-        const float vi = 0.999f * v[i] + 0.001f * gi * gi;
+        float wi = w[i], mi = m[i], vi = v[i];
+        adam_update(wi, g[i], mi, vi, lr, c1, c2);
         m[i] = mi;
         v[i] = vi;
-        const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
         w[i] = wi;
         wb[i] = __float2bfloat16(wi);
     }
@@ -296,12 +321,8 @@ struct tmr_mlp {
     int cap = 0;
     __nv_bfloat16 *xb = nullptr, *h1b = nullptr, *h2b = nullptr, *dzb = nullptr, *dz2b = nullptr, *dyb = nullptr;
     float *z1 = nullptr, *z2 = nullptr, *y = nullptr, *dh = nullptr, *part = nullptr, *lossd = nullptr;
-    float *ta = nullptr;  // aligned targets of the phase-invariant loss [B][out]
     int loss_kind = TMR_LOSS_MSE;
-    // tensor-core GEMM: transposed-operand scratch and the barrier-timeout flag
-    __nv_bfloat16 *tsa = nullptr, *tsb = nullptr;
-    size_t tsa_cap = 0, tsb_cap = 0;
-    int *tc_err = nullptr;
+    int *tc_err = nullptr;  // tensor-core GEMM: the barrier-timeout flag
 };
 
 namespace {
@@ -314,40 +335,30 @@ tmr_status mfail(tmr_status st, const char *msg)
 
 bool dev_ptr(const void *p) { return tmr::is_device_ptr(p); }
 
-// C[M][N] = sum_k A(m, k) B(k, n), A(m, k) = A[m sam + k sak], B(k, n) = B[k sbk + n sbn]:
-// on the tcgen05 tensor cores (gemm_tc.cu) when the shape allows, each operand
-// first made K-contiguous (a transpose into the network's scratch when it is
-// stored M- or N-contiguous); otherwise the mma.sync tile kernel above.
-void gemm(tmr_mlp *m, int M, int N, int K, const __nv_bfloat16 *A, long long sam, long long sak,
-          const __nv_bfloat16 *B, long long sbk, long long sbn, float *C)
+int ew_blocks(size_t n);
+
+// C[M][N] = sum_k A(m, k) B(n, k), then the elementwise step E (row stride N),
+// on the tcgen05 tensor cores (gemm_tc.cu) when the shape allows; otherwise the
+// mma.sync tile kernel above, the product into E.C (which the caller sets to
+// scratch where E itself does not store it) and the step as its own kernel.
+void gemm(tmr_mlp *m, int M, int N, int K, const GemmOperand &A, const GemmOperand &B, const GemmEpilogue &E)
 {
     cudaStream_t s = m->stream;
-    if (M >= 128 && N >= 128 && K >= 64 && K % 8 == 0 && m->tc_err) {
-        const __nv_bfloat16 *At = A, *Bt = B;
-        long long lda = sam, ldb = sbn;
-        bool ok = true;
-        if (sak != 1) {  // stored [K][M] (sam == 1): transpose to [M][K]
-            ok = sam == 1 && (size_t)M * K <= m->tsa_cap;
-            if (ok) {
-                transpose_bf16(K, M, A, sak, m->tsa, s);
-                At = m->tsa;
-                lda = K;
-            }
-        }
-        if (ok && sbk != 1) {  // stored [K][N] (sbn == 1): transpose to [N][K]
-            ok = sbn == 1 && (size_t)N * K <= m->tsb_cap;
-            if (ok) {
-                transpose_bf16(K, N, B, sbk, m->tsb, s);
-                Bt = m->tsb;
-                ldb = K;
-            }
-        }
-        if (ok && lda <= 0x7fffffff && ldb <= 0x7fffffff && gemm_tc_supported(M, N, K, At, (int)lda, Bt, (int)ldb) &&
-            gemm_tc(M, N, K, At, (int)lda, Bt, (int)ldb, C, N, m->tc_err, s) == cudaSuccess)
-            return;
+    if (m->tc_err && gemm_tc_supported(M, N, K, A, B)) {
+        if (gemm_tc(M, N, K, A, B, N, E, m->tc_err, s) == cudaSuccess) return;
         cudaGetLastError();
     }
-    gemm_sync(M, N, K, A, sam, sak, B, sbk, sbn, C, s);
+    gemm_sync(M, N, K, A.p, A.k_contiguous ? A.ld : 1, A.k_contiguous ? 1 : A.ld, B.p, B.k_contiguous ? 1 : B.ld,
+              B.k_contiguous ? B.ld : 1, E.C, s);
+    const size_t n = (size_t)M * N;
+    const int nb = ew_blocks(n);
+    switch (E.kind) {
+    case GEMM_BIAS:
+    case GEMM_BIAS_GELU: k_bias_act<<<nb, 256, 0, s>>>(M, N, E.C, E.bias, E.H, E.kind == GEMM_BIAS_GELU); break;
+    case GEMM_GELU_BACK: k_gelu_back<<<nb, 256, 0, s>>>(n, E.C, E.Z, E.H); break;
+    case GEMM_ADAM: k_adam<<<nb, 256, 0, s>>>(n, E.w, E.C, E.m, E.v, E.H, E.lr, E.c1, E.c2); break;
+    default: break;
+    }
 }
 
 int ew_blocks(size_t n)
@@ -361,7 +372,7 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
     if (B <= m->cap) return TMR_OK;
     void **bufs[] = {(void **)&m->xb, (void **)&m->h1b, (void **)&m->h2b, (void **)&m->dzb, (void **)&m->dz2b,
                      (void **)&m->dyb, (void **)&m->z1, (void **)&m->z2, (void **)&m->y, (void **)&m->dh,
-                     (void **)&m->ta, (void **)&m->tsa, (void **)&m->tsb};
+                     (void **)&m->part};
     for (void **b : bufs)
         if (*b) {
             cudaFree(*b);
@@ -380,19 +391,7 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
               cudaMalloc(&m->z2, sizeof(float) * (size_t)B * m->h2) == cudaSuccess &&
               cudaMalloc(&m->y, sizeof(float) * (size_t)B * m->n_out) == cudaSuccess &&
               cudaMalloc(&m->dh, sizeof(float) * hmax) == cudaSuccess &&
-              cudaMalloc(&m->ta, sizeof(float) * (size_t)B * m->n_out) == cudaSuccess;
-    // transposed operands of the tensor-core GEMM: A sides [max(out, h1, h2)][B],
-    // B sides W3^T, W2^T and [max(in, h1, h2)][B]
-    const size_t hmx = (size_t)(m->h1 > m->h2 ? m->h1 : m->h2);
-    const size_t amax = (size_t)B * ((size_t)m->n_out > hmx ? (size_t)m->n_out : hmx);
-    size_t bmax = (size_t)m->h2 * m->n_out;
-    if ((size_t)m->h1 * m->h2 > bmax) bmax = (size_t)m->h1 * m->h2;
-    const size_t bb = (size_t)B * ((size_t)m->n_in > hmx ? (size_t)m->n_in : hmx);
-    if (bb > bmax) bmax = bb;
-    ok = ok && cudaMalloc(&m->tsa, sizeof(__nv_bfloat16) * amax) == cudaSuccess &&
-         cudaMalloc(&m->tsb, sizeof(__nv_bfloat16) * bmax) == cudaSuccess;
-    m->tsa_cap = ok ? amax : 0;
-    m->tsb_cap = ok ? bmax : 0;
+              cudaMalloc(&m->part, sizeof(float) * (size_t)B) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         return mfail(TMR_ERR_OOM, "MLP batch buffers");
@@ -401,46 +400,81 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
     return TMR_OK;
 }
 
-// forward from BF16 features m->xb into m->y (FP32); keeps Z1, Z2, H1, H2
-void forward_core(tmr_mlp *m, int B)
+GemmEpilogue bias_step(float *z, const float *bias, __nv_bfloat16 *h)
 {
-    cudaStream_t s = m->stream;
-    const __nv_bfloat16 *W1 = m->wb + m->off[0], *W2 = m->wb + m->off[2], *W3 = m->wb + m->off[4];
-    const float *b1 = m->w + m->off[1], *b2 = m->w + m->off[3], *b3 = m->w + m->off[5];
-    // Z1 = X W1^T: A = X [B][n_in], B(k, n) = W1[n][k]
-    gemm(m, B, m->h1, m->n_in, m->xb, m->n_in, 1, W1, 1, m->n_in, m->z1);
-    k_bias_act<<<ew_blocks((size_t)B * m->h1), 256, 0, s>>>(B, m->h1, m->z1, b1, m->h1b, 1);
-    gemm(m, B, m->h2, m->h1, m->h1b, m->h1, 1, W2, 1, m->h1, m->z2);
-    k_bias_act<<<ew_blocks((size_t)B * m->h2), 256, 0, s>>>(B, m->h2, m->z2, b2, m->h2b, 1);
-    gemm(m, B, m->n_out, m->h2, m->h2b, m->h2, 1, W3, 1, m->h2, m->y);
-    k_bias_act<<<ew_blocks((size_t)B * m->n_out), 256, 0, s>>>(B, m->n_out, m->y, b3, nullptr, 0);
+    GemmEpilogue E;
+    E.kind = h ? GEMM_BIAS_GELU : GEMM_BIAS;
+    E.C = z;
+    E.bias = bias;
+    E.H = h;
+    return E;
 }
 
-// gradient of the MSE loss w.r.t. every parameter into m->g; loss (device scalar)
-void backward_core(tmr_mlp *m, int B, const float *T, float *loss)
+// forward from BF16 features m->xb into y (FP32 [B][out]); keeps Z1, Z2, H1, H2
+void forward_core(tmr_mlp *m, int B, float *y)
+{
+    const __nv_bfloat16 *W1 = m->wb + m->off[0], *W2 = m->wb + m->off[2], *W3 = m->wb + m->off[4];
+    const float *b1 = m->w + m->off[1], *b2 = m->w + m->off[3], *b3 = m->w + m->off[5];
+    gemm(m, B, m->h1, m->n_in, {m->xb, m->n_in, true}, {W1, m->n_in, true}, bias_step(m->z1, b1, m->h1b));
+    gemm(m, B, m->h2, m->h1, {m->h1b, m->h1, true}, {W2, m->h1, true}, bias_step(m->z2, b2, m->h2b));
+    gemm(m, B, m->n_out, m->h2, {m->h2b, m->h2, true}, {W3, m->h2, true}, bias_step(y, b3, nullptr));
+}
+
+// One Adam step's size and bias corrections
+struct AdamStep {
+    float lr, c1, c2;
+};
+
+// The loss (device scalar) and, from m->y, the gradient w.r.t. every parameter
+// into g; with `step`, every parameter is updated by it instead (g is scratch).
+void backward_core(tmr_mlp *m, int B, const float *T, float *loss, float *g, const AdamStep *step)
 {
     cudaStream_t s = m->stream;
     const __nv_bfloat16 *W2 = m->wb + m->off[2], *W3 = m->wb + m->off[4];
-    const int nb = ew_blocks((size_t)B * m->n_out);
-    if (m->loss_kind == TMR_LOSS_PHASE) {  // the loss against each row's aligned target
-        k_align_targets<<<B, 256, 0, s>>>(m->n_out / 2, m->y, T, m->ta);
-        T = m->ta;
+    k_loss_rows<<<B, 256, 0, s>>>(B, m->n_out, m->loss_kind == TMR_LOSS_PHASE, m->y, T, m->dyb, m->part);
+    k_loss_finish<<<1, 256, 0, s>>>(B, m->part, (float)((size_t)B * m->n_out), loss);
+    // dZ = (dZ_next W) .* GELU'(Z)
+    auto back = [&](const float *z, __nv_bfloat16 *dz) {
+        GemmEpilogue E;
+        E.kind = GEMM_GELU_BACK;
+        E.C = m->dh;
+        E.Z = z;
+        E.H = dz;
+        return E;
+    };
+    // dW = dZ^T H: the gradient, or the update of the weights at offset o
+    auto weights = [&](size_t o) {
+        GemmEpilogue E;
+        E.C = g + o;
+        if (step) {
+            E.kind = GEMM_ADAM;
+            E.w = m->w + o;
+            E.m = m->m + o;
+            E.v = m->v + o;
+            E.H = m->wb + o;
+            E.lr = step->lr;
+            E.c1 = step->c1;
+            E.c2 = step->c2;
+        }
+        return E;
+    };
+    // every dZ is made before the weights it was made with change
+    gemm(m, B, m->h2, m->n_out, {m->dyb, m->n_out, true}, {W3, m->h2, false}, back(m->z2, m->dz2b));
+    gemm(m, m->n_out, m->h2, B, {m->dyb, m->n_out, false}, {m->h2b, m->h2, false}, weights(m->off[4]));
+    gemm(m, B, m->h1, m->h2, {m->dz2b, m->h2, true}, {W2, m->h1, false}, back(m->z1, m->dzb));
+    gemm(m, m->h2, m->h1, B, {m->dz2b, m->h2, false}, {m->h1b, m->h1, false}, weights(m->off[2]));
+    gemm(m, m->h1, m->n_in, B, {m->dzb, m->h1, false}, {m->xb, m->n_in, false}, weights(m->off[0]));
+    BiasLayers L;
+    const __nv_bfloat16 *dz[3] = {m->dzb, m->dz2b, m->dyb};
+    const int width[3] = {m->h1, m->h2, m->n_out};
+    int blocks = 0;
+    for (int i = 0; i < 3; i++) {
+        const size_t o = m->off[2 * i + 1];
+        L.l[i] = {dz[i], width[i], blocks, g + o, m->w + o, m->m + o, m->v + o, m->wb + o};
+        blocks += (width[i] + 31) / 32;
     }
-    k_mse<<<nb, 256, 0, s>>>(B, m->n_out, m->y, T, m->dyb, m->part);
-    k_loss_finish<<<1, 32, 0, s>>>(nb, m->part, (float)((size_t)B * m->n_out), loss);
-    // layer 3: dW3 = dY^T H2 ([n_out][B] x [B][h2]); db3 = colsum(dY); dH2 = dY W3
-    gemm(m, m->n_out, m->h2, B, m->dyb, 1, m->n_out, m->h2b, m->h2, 1, m->g + m->off[4]);
-    k_colsum<<<(m->n_out + 255) / 256, 256, 0, s>>>(B, m->n_out, m->dyb, m->g + m->off[5]);
-    gemm(m, B, m->h2, m->n_out, m->dyb, m->n_out, 1, W3, m->h2, 1, m->dh);
-    k_gelu_back<<<ew_blocks((size_t)B * m->h2), 256, 0, s>>>((size_t)B * m->h2, m->dh, m->z2, m->dz2b);
-    // layer 2
-    gemm(m, m->h2, m->h1, B, m->dz2b, 1, m->h2, m->h1b, m->h1, 1, m->g + m->off[2]);
-    k_colsum<<<(m->h2 + 255) / 256, 256, 0, s>>>(B, m->h2, m->dz2b, m->g + m->off[3]);
-    gemm(m, B, m->h1, m->h2, m->dz2b, m->h2, 1, W2, m->h1, 1, m->dh);
-    k_gelu_back<<<ew_blocks((size_t)B * m->h1), 256, 0, s>>>((size_t)B * m->h1, m->dh, m->z1, m->dzb);
-    // layer 1
-    gemm(m, m->h1, m->n_in, B, m->dzb, 1, m->h1, m->xb, m->n_in, 1, m->g + m->off[0]);
-    k_colsum<<<(m->h1 + 255) / 256, 256, 0, s>>>(B, m->h1, m->dzb, m->g + m->off[1]);
+    k_bias_grad<<<blocks, dim3(32, 8), 0, s>>>(B, L, step != nullptr, step ? step->lr : 0.f, step ? step->c1 : 1.f,
+                                               step ? step->c2 : 1.f);
 }
 
 }  // namespace
@@ -454,7 +488,7 @@ cudaError_t mlp_propose(tmr_mlp *m, const float *y, int B, int N, int J, float2 
     cudaStream_t keep = m->stream;
     m->stream = s;
     k_features<<<B, 256, 0, s>>>(J * N, y, m->xb);
-    forward_core(m, B);
+    forward_core(m, B, m->y);
     k_candidate<<<B, 256, 0, s>>>(N, J * N, m->y, y, T);
     m->stream = keep;
     return cudaGetLastError();
@@ -489,7 +523,6 @@ tmr_status tmr_mlp_create(tmr_mlp **out, int n_in, int n_h1, int n_h2, int n_out
                     cudaMalloc(&m->v, sizeof(float) * o) == cudaSuccess &&
                     cudaMalloc(&m->g, sizeof(float) * o) == cudaSuccess &&
                     cudaMalloc(&m->wb, sizeof(__nv_bfloat16) * o) == cudaSuccess &&
-                    cudaMalloc(&m->part, sizeof(float) * 152 * 8) == cudaSuccess &&
                     cudaMalloc(&m->lossd, sizeof(float) * 4) == cudaSuccess &&
                     cudaMalloc(&m->tc_err, sizeof(int)) == cudaSuccess &&
                     cudaMemset(m->tc_err, 0, sizeof(int)) == cudaSuccess;
@@ -557,14 +590,14 @@ tmr_status tmr_mlp_forward(tmr_mlp *m, const float *X, int B, float *Y)
     tmr_status st = ensure_batch(m, B);
     if (st != TMR_OK) return st;
     k_to_bf16<<<ew_blocks((size_t)B * m->n_in), 256, 0, m->stream>>>((size_t)B * m->n_in, X, m->xb);
-    forward_core(m, B);
-    if (cudaMemcpyAsync(Y, m->y, sizeof(float) * (size_t)B * m->n_out, cudaMemcpyDeviceToDevice, m->stream) !=
-        cudaSuccess)
-        return mfail(TMR_ERR_CUDA, "forward copy");
+    forward_core(m, B, Y);
     return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "forward kernels");
 }
 
-tmr_status tmr_mlp_grad(tmr_mlp *m, const float *X, const float *T, int B, float *loss, float *grad)
+// the batch's loss and, without `step`, its gradient (into grad, or scratch when
+// NULL), with it one update
+static tmr_status mlp_batch(tmr_mlp *m, const float *X, const float *T, int B, float *loss, float *grad,
+                            const AdamStep *step)
 {
     set_last_error("");
     if (!m || !X || !T || B <= 0) return mfail(TMR_ERR_INVALID_ARG, "bad argument");
@@ -573,21 +606,24 @@ tmr_status tmr_mlp_grad(tmr_mlp *m, const float *X, const float *T, int B, float
     tmr_status st = ensure_batch(m, B);
     if (st != TMR_OK) return st;
     k_to_bf16<<<ew_blocks((size_t)B * m->n_in), 256, 0, m->stream>>>((size_t)B * m->n_in, X, m->xb);
-    forward_core(m, B);
-    backward_core(m, B, T, loss ? loss : m->lossd);
-    if (grad && cudaMemcpyAsync(grad, m->g, sizeof(float) * m->np, cudaMemcpyDeviceToDevice, m->stream) != cudaSuccess)
-        return mfail(TMR_ERR_CUDA, "grad copy");
-    return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "grad kernels");
+    forward_core(m, B, m->y);
+    backward_core(m, B, T, loss ? loss : m->lossd, grad ? grad : m->g, step);
+    return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "network kernels");
+}
+
+tmr_status tmr_mlp_grad(tmr_mlp *m, const float *X, const float *T, int B, float *loss, float *grad)
+{
+    return mlp_batch(m, X, T, B, loss, grad, nullptr);
 }
 
 tmr_status tmr_mlp_train_step(tmr_mlp *m, const float *X, const float *T, int B, float lr, float *loss)
 {
-    tmr_status st = tmr_mlp_grad(m, X, T, B, loss, nullptr);
-    if (st != TMR_OK) return st;
-    m->step++;
-    const float c1 = 1.f - powf(0.9f, (float)m->step), c2 = 1.f - powf(0.999f, (float)m->step);
-    k_adam<<<ew_blocks(m->np), 256, 0, m->stream>>>(m->np, m->w, m->g, m->m, m->v, m->wb, lr, c1, c2);
-    return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "adam kernel");
+    if (!m) return mlp_batch(m, X, T, B, loss, nullptr, nullptr);  // refused there
+    const float t = (float)(m->step + 1);
+    const AdamStep step = {lr, 1.f - powf(0.9f, t), 1.f - powf(0.999f, t)};
+    const tmr_status st = mlp_batch(m, X, T, B, loss, nullptr, &step);
+    if (st == TMR_OK) m->step++;
+    return st;
 }
 
 tmr_status tmr_mlp_set_loss(tmr_mlp *m, int kind)
@@ -607,7 +643,7 @@ void tmr_mlp_destroy(tmr_mlp *m)
     if (m->stream) cudaStreamSynchronize(m->stream);
     else cudaDeviceSynchronize();
     void *p[] = {m->w, m->m, m->v, m->g, m->wb, m->xb, m->h1b, m->h2b, m->dzb, m->dz2b, m->dyb,
-                 m->z1, m->z2, m->y, m->dh, m->part, m->lossd, m->ta, m->tsa, m->tsb, m->tc_err};
+                 m->z1, m->z2, m->y, m->dh, m->part, m->lossd, m->tc_err};
     for (void *q : p)
         if (q) cudaFree(q);
     delete m;
