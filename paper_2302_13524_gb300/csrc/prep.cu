@@ -8,8 +8,9 @@
 //                  energy partial per (frame chunk, pixel); HBM-bound
 //                  (reads the kept camera rows once, writes y once)
 //   k_prep_energy  E[p] = the partials of pixel p summed in chunk order
-//   k_prep_select  one CTA: the threshold tau = the c-th largest energy, found
-//                  by a bitwise search on the energy keys; mask and count
+//   k_prep_select  one cluster (FP64 energies: one CTA): the threshold tau = the
+//                  c-th largest energy, found by a bitwise search on the energy
+//                  keys; mask and count
 //   k_prep_zero    rows outside the mask set to zero (write-only)
 // Every sum runs in a fixed order, so repeated calls agree bitwise; uint16
 // frames are summed exactly in 64-bit integers, float32 frames in FP64.
@@ -17,9 +18,13 @@
 #include <cstdint>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "internal.h"
 #include "tmr.h"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -27,6 +32,7 @@ constexpr int kTile = 32;    // pixels (and frames) per transpose tile
 constexpr int kTy = 8;       // threadIdx.y extent of k_prep_rows
 constexpr int kChunk = 256;  // frames per CTA of k_prep_rows (one energy partial each)
 constexpr int kSelThreads = 1024;
+constexpr size_t kSelStage = 208 * 1024;  // keys staged in shared memory at most
 
 tmr_status fail(tmr_status st, const char *msg)
 {
@@ -135,11 +141,13 @@ __global__ void k_prep_energy(const unsigned long long *__restrict__ part, int C
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < M; p += gridDim.x * blockDim.x) {
         if constexpr (kInt) {
             unsigned long long s = 0;
+#pragma unroll 16
             for (int c = 0; c < C; c++) s += part[(size_t)c * M + p];
             key[p] = s;
             if (energy) energy[p] = (double)s;
         } else {
             double s = 0.0;
+#pragma unroll 16
             for (int c = 0; c < C; c++) s += __longlong_as_double((long long)part[(size_t)c * M + p]);
             s += 0.0;  // -0 -> +0
             if (!(s >= 0.0) || !isfinite(s)) {
@@ -152,144 +160,205 @@ __global__ void k_prep_energy(const unsigned long long *__restrict__ part, int C
     }
 }
 
-// Sum over the block of the energies whose key is >= lo, in a fixed order
+// Sum over the block of the FP64 energies whose key is >= lo, in a fixed order
 // (each thread its strided pixels in turn, then warp and block trees).
-// Integer energies are summed exactly and returned converted to FP64.
-template <bool kInt>
-__device__ double energy_at_or_above(const unsigned long long *__restrict__ key, int M,
-                                     unsigned long long lo, double *red_d,
-                                     unsigned long long *red_u)
+__device__ double energy_at_or_above(const unsigned long long *__restrict__ key, int M, unsigned long long lo,
+                                     double *red_d)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double out;
-    if constexpr (kInt) {
-        unsigned long long s = 0;
-        for (int p = threadIdx.x; p < M; p += blockDim.x) s += key[p] >= lo ? key[p] : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) red_u[warp] = s;
-        __syncthreads();
-        unsigned long long t = 0;
-        for (int w = 0; w < nw; w++) t += red_u[w];
-        out = (double)t;
-    } else {
-        double s = 0.0;
-        for (int p = threadIdx.x; p < M; p += blockDim.x)
-            s += key[p] >= lo ? __longlong_as_double((long long)key[p]) : 0.0;
-        s = tmr::warp_sum(s);
-        if (lane == 0) red_d[warp] = s;
-        __syncthreads();
-        if (warp == 0) {
-            double t = lane < nw ? red_d[lane] : 0.0;
-            t = tmr::warp_sum(t);
-            if (lane == 0) red_d[32] = t;
-        }
-        __syncthreads();
-        out = red_d[32];
+    double s = 0.0;
+#pragma unroll 4
+    for (int p = threadIdx.x; p < M; p += blockDim.x) s += key[p] >= lo ? __longlong_as_double((long long)key[p]) : 0.0;
+    s = tmr::warp_sum(s);
+    if (lane == 0) red_d[warp] = s;
+    __syncthreads();
+    if (warp == 0) {
+        double t = lane < nw ? red_d[lane] : 0.0;
+        t = tmr::warp_sum(t);
+        if (lane == 0) red_d[32] = t;
     }
+    __syncthreads();
+    const double out = red_d[32];
     __syncthreads();  // the scratch is reused by the next call
     return out;
 }
 
-// Integer energies: the threshold by 3-bit passes over the keys, from the
-// top set bit down.  A pass fixes the next digit of tau: with the bits above
-// already fixed (prefix), S(prefix | j << shift) for the eight digits j is
+// ---- the threshold ----
+// S(tau) = sum of the energies >= tau falls as tau grows; the mask threshold is
+// the largest key tau with S(tau) >= frac * S(0) (compared in FP64), built from
+// the top bit down.  That tau is the c-th largest energy for the smallest
+// brightest-first count c reaching the fraction, and E >= tau includes its ties.
+
+constexpr int kSelCtas = 8;  // CTAs (one portable cluster) of the integer search
+
+// Integer energies: one cluster, each CTA with an eighth of the pixels (in
+// shared memory where they fit), tau by 3-bit passes from the top set bit of
+// the largest key down.  A pass fixes the next digit of tau: with the bits
+// above already fixed (prefix), S(prefix | j << shift) for the eight digits j is
 // the sum of the keys whose upper bits exceed the prefix's, plus the keys
 // equal to it there whose digit is >= j; each thread accumulates all eight
-// sums in registers (no shared-memory atomics, which serialise when most
-// keys share their upper bits), the block adds them exactly, and the largest
-// j whose S reaches the target is taken (compared in FP64).
-__device__ unsigned long long select_tau_int(const unsigned long long *__restrict__ key, int M,
-                                             double target, unsigned long long mx,
-                                             unsigned long long (*red8)[8], unsigned long long *S8)
+// sums in registers (no shared-memory atomics, which serialise: the energies
+// of a lit core share their upper bits), and the CTAs' exact sums are added
+// through distributed shared memory.  One CTA alone took 84 us for the paper's
+// 8192 pixels: its 22 or so walks over the keys in L2 latencies, and FP64
+// comparisons (two lanes a cycle) in every thread; the cluster makes each walk
+// one key per thread and lets one lane per digit compare.
+template <bool kStaged>
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads)
+    k_prep_select_int(const unsigned long long *__restrict__ key_g, int M, double frac,
+                      unsigned char *__restrict__ mask_ws, unsigned char *__restrict__ mask, int *__restrict__ n_inside)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    unsigned long long prefix = 0;
-    for (int top = 63 - __clzll(mx); top >= 0;) {
-        const int shift = top >= 2 ? top - 2 : 0;
-        const int nd = 1 << (top - shift + 1);
-        const unsigned long long hi_mask = top >= 63 ? 0ull : (~0ull << (top + 1));
-        unsigned long long acc[8];
+    extern __shared__ unsigned long long key_s[];
+    __shared__ unsigned long long red8[kSelThreads / 32][8], part[2][kSelCtas][8], S8[8];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = (int)cluster.block_rank();
+    const int p0 = (int)((long long)rank * M / kSelCtas), n = (int)((long long)(rank + 1) * M / kSelCtas) - p0;
+    const unsigned long long *key = key_g + p0;
+    if constexpr (kStaged) {
+        for (int p = tid; p < n; p += kSelThreads) key_s[p] = key[p];
+        key = key_s;  // each thread reads back its own
+    }
+    // S8[j] <- the cluster's sum (or, with `largest`, maximum) of acc[j]; the two
+    // part buffers alternate, so that a slow CTA may still read the last one
+    int sel = 0;
+    auto reduce8 = [&](unsigned long long (&acc)[8], bool largest) {
+        auto join = [&](unsigned long long x, unsigned long long y) { return largest ? (x > y ? x : y) : x + y; };
+        // transposing tree: lane 4 q then holds the warp's result of value q
+        // (7 exchanges instead of 8 x 3), then two more over its four lanes
+#pragma unroll
+        for (int h = 4; h >= 1; h >>= 1) {
+            const bool upper = (lane & (4 * h)) != 0;
+#pragma unroll
+            for (int i = 0; i < h; i++) {
+                const unsigned long long send = upper ? acc[i] : acc[i + h], keep = upper ? acc[i + h] : acc[i];
+                acc[i] = join(keep, __shfl_xor_sync(0xffffffffu, send, 4 * h));
+            }
+        }
+        acc[0] = join(acc[0], __shfl_xor_sync(0xffffffffu, acc[0], 2));
+        acc[0] = join(acc[0], __shfl_xor_sync(0xffffffffu, acc[0], 1));
+        if ((lane & 3) == 0) red8[warp][lane >> 2] = acc[0];
+        __syncthreads();
+        if (warp < 8) {  // warp j joins value j over the warps and hands it to every CTA
+            unsigned long long v = red8[lane][warp];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v = join(v, __shfl_xor_sync(0xffffffffu, v, o));
+            if (lane < kSelCtas) *cluster.map_shared_rank(&part[sel][rank][warp], lane) = v;
+        }
+        cluster.sync();
+        if (tid < 8) {
+            unsigned long long v = part[sel][0][tid];
+            for (int r = 1; r < kSelCtas; r++) v = join(v, part[sel][r][tid]);
+            S8[tid] = v;
+        }
+        sel ^= 1;
+        __syncthreads();
+    };
+    unsigned long long acc[8] = {0ull};
+    for (int p = tid; p < n; p += kSelThreads) acc[0] += key[p];
+    reduce8(acc, false);
+    const unsigned long long total = S8[0];
+    unsigned long long prefix = ~0ull;  // above every key: empty mask
+    if (total > 0) {
 #pragma unroll
         for (int j = 0; j < 8; j++) acc[j] = 0ull;
-        for (int p = threadIdx.x; p < M; p += blockDim.x) {
-            const unsigned long long k = key[p], kh = k & hi_mask;
-            const int d = kh > prefix ? 7 : (kh == prefix ? (int)((k >> shift) & (unsigned long long)(nd - 1)) : -1);
+        for (int p = tid; p < n; p += kSelThreads) acc[0] = key[p] > acc[0] ? key[p] : acc[0];
+        __syncthreads();  // S8 is read before it is written again
+        reduce8(acc, true);
+        const unsigned long long mx = S8[0];
+        prefix = 0;
+        for (int top = 63 - __clzll(mx); top >= 0;) {
+            const int shift = top >= 2 ? top - 2 : 0;
+            const int nd = 1 << (top - shift + 1);
+            const unsigned long long hi_mask = top >= 63 ? 0ull : (~0ull << (top + 1));
 #pragma unroll
-            for (int j = 0; j < 8; j++) acc[j] += d >= j ? k : 0ull;
+            for (int j = 0; j < 8; j++) acc[j] = 0ull;
+            for (int p = tid; p < n; p += kSelThreads) {
+                const unsigned long long k = key[p], kh = k & hi_mask;
+                const int d = kh > prefix ? 7 : (kh == prefix ? (int)((k >> shift) & (unsigned long long)(nd - 1)) : -1);
+#pragma unroll
+                for (int j = 0; j < 8; j++) acc[j] += d >= j ? k : 0ull;
+            }
+            __syncthreads();  // S8 is read before it is written again
+            reduce8(acc, false);
+            // digit 0 always reaches the target (S of the prefix itself)
+            const bool reach = lane < nd && (lane == 0 || (double)S8[lane & 7] >= frac * (double)total);
+            prefix |= (unsigned long long)(31 - __clz(__ballot_sync(0xffffffffu, reach))) << shift;
+            top = shift - 1;
         }
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < 8; j++) red8[warp][j] = acc[j];
-        }
-        __syncthreads();
-        if (warp < 8) {  // warp j adds sum j over the warps
-            unsigned long long v = lane < nw ? red8[lane][warp] : 0ull;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) S8[warp] = v;
-        }
-        __syncthreads();
-        int best = 0;  // digit 0 always reaches the target (S of the prefix itself)
-        for (int j = 1; j < nd; j++)
-            if ((double)S8[j] >= target) best = j;
-        prefix |= (unsigned long long)best << shift;
-        top = shift - 1;
-        __syncthreads();  // S8 and red8 are rewritten by the next pass
     }
-    return prefix;
+#pragma unroll
+    for (int j = 0; j < 8; j++) acc[j] = 0ull;
+    for (int p = tid; p < n; p += kSelThreads) {
+        const unsigned char in = key[p] >= prefix ? 1 : 0;
+        mask_ws[p0 + p] = in;
+        if (mask) mask[p0 + p] = in;
+        acc[0] += in;
+    }
+    __syncthreads();
+    reduce8(acc, false);  // its last cluster barrier is the last access to another CTA's memory
+    if (rank == 0 && tid == 0 && n_inside) *n_inside = (int)S8[0];
 }
 
-// One CTA.  S(tau) = sum of the energies >= tau falls as tau grows; the mask
-// threshold is the largest key tau with S(tau) >= frac * S(0), built from the
-// top bit down (integer keys: 3 bits a pass; FP64 keys: one bit a pass, each
-// a fixed-order FP64 block sum).  That tau is the c-th largest energy for the smallest
-// brightest-first count c reaching the fraction, and E >= tau includes its ties.
-template <bool kInt>
-__global__ void __launch_bounds__(kSelThreads) k_prep_select(const unsigned long long *__restrict__ key,
-                                                             int M, double frac,
-                                                             const int *__restrict__ bad,
-                                                             unsigned char *__restrict__ mask_ws,
-                                                             unsigned char *__restrict__ mask,
-                                                             int *__restrict__ n_inside)
+// Bits in which the keys differ, as a mask, over the block (a key alone: 0);
+// the bits outside it are those of the largest key in every key.
+__device__ unsigned long long differing_bits(const unsigned long long *__restrict__ key, int M, unsigned long long *red_u)
+{
+    unsigned long long o = 0, a = ~0ull;
+#pragma unroll 4
+    for (int p = threadIdx.x; p < M; p += blockDim.x) o |= key[p], a &= key[p];
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        o |= __shfl_xor_sync(0xffffffffu, o, s);
+        a &= __shfl_xor_sync(0xffffffffu, a, s);
+    }
+    const int nw = blockDim.x >> 5;
+    if ((threadIdx.x & 31) == 0) red_u[threadIdx.x >> 5] = o;
+    __syncthreads();
+    for (int w = 0; w < nw; w++) o |= red_u[w];
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red_u[threadIdx.x >> 5] = a;
+    __syncthreads();
+    for (int w = 0; w < nw; w++) a &= red_u[w];
+    __syncthreads();
+    return o & ~a;
+}
+
+// FP64 energies (bit patterns): one CTA, one bit a pass, each a fixed-order FP64
+// block sum, over the keys in shared memory where they fit.  Only the bits in
+// which the keys differ take a pass: tau is a key, so it has the common ones
+// (the energies of counts, whole numbers below 2^27 or so, leave half of the
+// mantissa's bits zero in every key).
+template <bool kStaged>
+__global__ void __launch_bounds__(kSelThreads) k_prep_select_f64(const unsigned long long *__restrict__ key_g, int M,
+                                                                 double frac, const int *__restrict__ bad,
+                                                                 unsigned char *__restrict__ mask_ws,
+                                                                 unsigned char *__restrict__ mask,
+                                                                 int *__restrict__ n_inside)
 {
     __shared__ double red_d[kSelThreads / 32 + 1];
     __shared__ unsigned long long red_u[kSelThreads / 32];
     __shared__ int cnt[kSelThreads / 32];
-    __shared__ unsigned long long red8[kSelThreads / 32][8];
-    __shared__ unsigned long long S8[8];
+    extern __shared__ unsigned long long key_s[];
+    const unsigned long long *key = key_g;
+    if constexpr (kStaged) {
+        for (int p = threadIdx.x; p < M; p += blockDim.x) key_s[p] = key_g[p];
+        __syncthreads();
+        key = key_s;
+    }
     const bool invalid = *bad != 0;
     unsigned long long tau = ~0ull;  // above every key: empty mask
     if (!invalid) {
-        const double total = energy_at_or_above<kInt>(key, M, 0ull, red_d, red_u);
+        const double total = energy_at_or_above(key, M, 0ull, red_d);
         if (total > 0.0) {
             const double target = frac * total;
-            unsigned long long mx = 0;
-            for (int p = threadIdx.x; p < M; p += blockDim.x) mx = key[p] > mx ? key[p] : mx;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
-                mx = v > mx ? v : mx;
+            const unsigned long long diff = differing_bits(key, M, red_u);
+            unsigned long long t = key[0] & ~diff;
+            for (int bit = 63; bit >= 0; bit--) {
+                if (!(diff >> bit & 1ull)) continue;
+                const unsigned long long cand = t | (1ull << bit);
+                if (energy_at_or_above(key, M, cand, red_d) >= target) t = cand;
             }
-            if ((threadIdx.x & 31) == 0) red_u[threadIdx.x >> 5] = mx;
-            __syncthreads();
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) mx = red_u[w] > mx ? red_u[w] : mx;
-            __syncthreads();
-            if constexpr (kInt) {
-                tau = select_tau_int(key, M, target, mx, red8, S8);
-            } else {
-                unsigned long long t = 0;
-                for (int bit = 63 - __clzll(mx); bit >= 0; bit--) {
-                    const unsigned long long cand = t | (1ull << bit);
-                    if (energy_at_or_above<kInt>(key, M, cand, red_d, red_u) >= target) t = cand;
-                }
-                tau = t;
-            }
+            tau = t;
         }
     }
     int n = 0;
@@ -316,6 +385,12 @@ __global__ void k_prep_zero(const unsigned char *__restrict__ mask_ws, int K, fl
     const size_t p = blockIdx.x;
     if (mask_ws[p]) return;
     float *row = y + p * (size_t)K;
+    if (((reinterpret_cast<uintptr_t>(y) & 15) | (K & 3)) == 0) {
+        float4 *row4 = reinterpret_cast<float4 *>(row);
+#pragma unroll 4
+        for (int k = threadIdx.x; k < K / 4; k += blockDim.x) row4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
     for (int k = threadIdx.x; k < K; k += blockDim.x) row[k] = 0.f;
 }
 
@@ -371,9 +446,30 @@ cudaError_t launch_prep(const PT *frames, int K, int H, int W, int off, double f
     if (e != cudaSuccess) return e;
     k_prep_rows<PT><<<dim3((L.M + kTile - 1) / kTile, L.C), dim3(kTile, kTy), 0, s>>>(
         frames, K, H, W, off, L.nx, L.M, y, part);
-    const int eb = 256, eg = (int)std::min<long long>((L.M + eb - 1) / eb, 152LL * 8);
+    const int eb = 64, eg = (int)std::min<long long>((L.M + eb - 1) / eb, 152LL * 8);
     k_prep_energy<kInt><<<eg, eb, 0, s>>>(part, L.C, L.M, key, energy, bad);
-    k_prep_select<kInt><<<1, kSelThreads, 0, s>>>(key, L.M, frac, bad, mask_ws, mask, n_inside);
+    auto stage = [](const void *kernel, size_t bytes) {  // shared memory above the default needs asking for
+        return bytes > 40 * 1024
+                   ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelStage)
+                   : cudaSuccess;
+    };
+    if constexpr (kInt) {
+        const size_t ks = sizeof(unsigned long long) * (size_t)(L.M / kSelCtas + 1);
+        if (ks <= kSelStage) {
+            if ((e = stage((const void *)k_prep_select_int<true>, ks)) != cudaSuccess) return e;
+            k_prep_select_int<true><<<kSelCtas, kSelThreads, ks, s>>>(key, L.M, frac, mask_ws, mask, n_inside);
+        } else {
+            k_prep_select_int<false><<<kSelCtas, kSelThreads, 0, s>>>(key, L.M, frac, mask_ws, mask, n_inside);
+        }
+    } else {
+        const size_t ks = sizeof(unsigned long long) * (size_t)L.M;
+        if (ks <= kSelStage) {
+            if ((e = stage((const void *)k_prep_select_f64<true>, ks)) != cudaSuccess) return e;
+            k_prep_select_f64<true><<<1, kSelThreads, ks, s>>>(key, L.M, frac, bad, mask_ws, mask, n_inside);
+        } else {
+            k_prep_select_f64<false><<<1, kSelThreads, 0, s>>>(key, L.M, frac, bad, mask_ws, mask, n_inside);
+        }
+    }
     k_prep_zero<<<L.M, 256, 0, s>>>(mask_ws, K, y);
     return cudaGetLastError();
 }
