@@ -49,10 +49,10 @@ cudaError_t launch_make_quadratic_H(int ny, int nx, double coef, float2 *H, cuda
 // shared-memory 2D FFT, in place, radix-2 decimation in time after a
 // bit-reversal permutation along each axis.  grid pitch = nx + 1 float2.
 
-// tw[k] = exp(-2 pi i k / n), k < n/2 (twy for ny, twx for nx), made once per CTA.
+// tw[k] = exp(-2 pi i k / n), k < n (twy for ny, twx for nx), made once per CTA.
 __device__ void make_tw(float2 *tw, int n)
 {
-    for (int k = threadIdx.x; k < n / 2; k += blockDim.x) {
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
         double s, c;
         sincospi(-2.0 * k / n, &s, &c);
         tw[k] = make_float2((float)c, (float)s);
@@ -104,38 +104,34 @@ __device__ __forceinline__ int axis_freq(const AxisPlan &P, int pos)
     return f;
 }
 
-// W_n^idx from the half table tw[k] = exp(-2 pi i k / n), k < n / 2, idx < n
-__device__ __forceinline__ float2 tw_full(const float2 *tw, int n, int idx)
-{
-    if (idx < n / 2) return tw[idx];
-    const float2 w = tw[idx - n / 2];
-    return make_float2(-w.x, -w.y);
-}
-
-// One forward (FWD) or inverse stage of radix R and length L on every line
-// of one axis.  Along rows (ROWS): element e of line a at a * pitch + e,
-// nlines = ny; along columns: element e of line x at e * pitch + x.
+// One forward (FWD) or inverse stage of radix R and length L = 2^lL on every
+// line of one axis of length n = 2^ln.  Along rows (ROWS): element e of line a
+// at a * pitch + e, 2^ll lines; along columns: element e of line x at
+// e * pitch + x.  Every index is taken apart by shifts: with the integer
+// divisions that runtime sizes otherwise mean, the addressing of a butterfly
+// took more instructions than its arithmetic.
 template <int R, bool FWD, bool ROWS>
-__device__ void fft_stage(float2 *g, int n, int nlines, int pitch, int L, const float2 *tw)
+__device__ void fft_stage(float2 *g, int ln, int ll, int pitch, int lL, const float2 *tw)
 {
-    const int m = L / R, per = n / R, total = nlines * per;
+    constexpr int LR = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
+    const int lm = lL - LR, total = 1 << (ll + ln - LR);
     for (int i = threadIdx.x; i < total; i += blockDim.x) {
-        const int line = i % nlines, q = i / nlines;  // lines fastest
-        const int b = q / m, j = q - b * m;
-        const int e0 = b * L + j;
+        const int line = i & ((1 << ll) - 1), q = i >> ll;  // lines fastest
+        const int b = q >> lm, j = q & ((1 << lm) - 1);
+        const int e0 = (b << lL) + j;
         float2 *base = ROWS ? g + line * pitch + e0 : g + e0 * pitch + line;
-        const int es = ROWS ? m : m * pitch;
+        const int es = ROWS ? 1 << lm : pitch << lm;
         float2 x[R];
 #pragma unroll
         for (int k = 0; k < R; k++) x[k] = base[k * es];
-        const int step = j * (n / L);
+        const int step = j << (ln - lL);
         if (FWD) {
             dft_small<R, -1>(x);
 #pragma unroll
-            for (int k = 1; k < R; k++) x[k] = cmul(x[k], tw_full(tw, n, step * k));
+            for (int k = 1; k < R; k++) x[k] = cmul(x[k], tw[step * k]);
         } else {
 #pragma unroll
-            for (int k = 1; k < R; k++) x[k] = cmulc(x[k], tw_full(tw, n, step * k));
+            for (int k = 1; k < R; k++) x[k] = cmulc(x[k], tw[step * k]);
             dft_small<R, 1>(x);
         }
 #pragma unroll
@@ -147,17 +143,17 @@ __device__ void fft_stage(float2 *g, int n, int nlines, int pitch, int L, const 
 template <bool FWD, bool ROWS>
 __device__ void fft_axis(float2 *g, const AxisPlan &P, int nlines, int pitch, const float2 *tw)
 {
+    const int ll = __ffs(nlines) - 1;
     // forward: stages 0 .. ns-1 (span shrinking); inverse: the reverse order
     for (int t = 0; t < P.ns; t++) {
         const int s = FWD ? t : P.ns - 1 - t;
         int lL = P.ln;
         for (int u = 0; u < s; u++) lL -= P.lr(u);
-        const int L = 1 << lL;
-        switch (1 << P.lr(s)) {
-        case 2: fft_stage<2, FWD, ROWS>(g, P.n, nlines, pitch, L, tw); break;
-        case 4: fft_stage<4, FWD, ROWS>(g, P.n, nlines, pitch, L, tw); break;
-        case 8: fft_stage<8, FWD, ROWS>(g, P.n, nlines, pitch, L, tw); break;
-        default: fft_stage<16, FWD, ROWS>(g, P.n, nlines, pitch, L, tw); break;
+        switch (P.lr(s)) {
+        case 1: fft_stage<2, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        case 2: fft_stage<4, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        case 3: fft_stage<8, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        default: fft_stage<16, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
         }
     }
 }
@@ -178,6 +174,124 @@ __device__ void fft2_inv(float2 *g, int ny, int nx, const float2 *twy, const flo
     fft_axis<false, true>(g, Px, ny, nx + 1, twx);
 }
 
+// ---------------------------------------------------------------------------
+// Passes of the same-grid operator that fuse a transform's outer stage with what
+// stands next to it, so that the grid crosses shared memory 13 times for an
+// evaluation of the fit (D and D^H of one pattern) instead of 22.
+
+// The last forward column stage (length R: no twiddles), the product with H
+// and 1 / P (h(position)), and the first inverse column stage, on the R
+// elements that all three share.
+template <int R, class Hat>
+__device__ void col_mid_stage(float2 *g, int ln, int ll, int pitch, float inv, Hat &&h)
+{
+    constexpr int LR = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
+    const int total = 1 << (ll + ln - LR);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int col = i & ((1 << ll) - 1), row0 = (i >> ll) << LR;
+        float2 *base = g + row0 * pitch + col;
+        float2 x[R];
+#pragma unroll
+        for (int k = 0; k < R; k++) x[k] = base[k * pitch];
+        dft_small<R, -1>(x);
+#pragma unroll
+        for (int k = 0; k < R; k++) x[k] = cscale(cmul(x[k], h(row0 + k, col)), inv);
+        dft_small<R, 1>(x);
+#pragma unroll
+        for (int k = 0; k < R; k++) base[k * pitch] = x[k];
+    }
+    __syncthreads();
+}
+
+// The first forward row stage (FIRST) and / or the last inverse one, which share
+// their elements: LOAD: x = in(a, b) in place of the grid; otherwise the inverse
+// stage first.  Between the two, mid(a, b, x) on the natural-order values
+// (returning what goes on), and without FIRST nothing is stored.  Consecutive
+// threads take consecutive elements of a row, whole sectors of the arrays that
+// in and mid touch.
+template <int R, bool LOAD, bool FIRST, class In, class Mid>
+__device__ void row_outer_stage(float2 *g, int ln, int ll, int pitch, const float2 *tw, In &&in, Mid &&mid)
+{
+    constexpr int LR = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
+    const int lm = ln - LR, total = 1 << (ll + lm);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int j = i & ((1 << lm) - 1), a = i >> lm;
+        float2 *base = g + a * pitch + j;
+        float2 x[R];
+        if constexpr (LOAD) {
+#pragma unroll
+            for (int k = 0; k < R; k++) x[k] = in(a, j + (k << lm));
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; k++) x[k] = base[k << lm];
+#pragma unroll
+            for (int k = 1; k < R; k++) x[k] = cmulc(x[k], tw[j * k]);
+            dft_small<R, 1>(x);
+#pragma unroll
+            for (int k = 0; k < R; k++) x[k] = mid(a, j + (k << lm), x[k]);
+        }
+        if constexpr (FIRST) {
+            dft_small<R, -1>(x);
+#pragma unroll
+            for (int k = 1; k < R; k++) x[k] = cmul(x[k], tw[j * k]);
+#pragma unroll
+            for (int k = 0; k < R; k++) base[k << lm] = x[k];
+        }
+    }
+    __syncthreads();
+}
+
+// stages [s0, s1) of an axis in forward (FWD) or inverse order
+template <bool FWD, bool ROWS>
+__device__ void fft_axis_part(float2 *g, const AxisPlan &P, int nlines, int pitch, const float2 *tw, int s0, int s1)
+{
+    const int ll = __ffs(nlines) - 1;
+    for (int t = s0; t < s1; t++) {
+        const int s = FWD ? t : s1 - 1 - (t - s0);
+        int lL = P.ln;
+        for (int u = 0; u < s; u++) lL -= P.lr(u);
+        switch (P.lr(s)) {
+        case 1: fft_stage<2, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        case 2: fft_stage<4, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        case 3: fft_stage<8, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        default: fft_stage<16, FWD, ROWS>(g, P.ln, ll, pitch, lL, tw); break;
+        }
+    }
+}
+
+// Everything of D (or D^H) between the first row stage and the last: h(a, b) is
+// H (conjugated for the adjoint) at spectrum position (a, b).
+template <class Hat>
+__device__ void defocus_inner(float2 *g, int ny, int nx, const float2 *twy, const float2 *twx, Hat &&h)
+{
+    const AxisPlan Px = axis_plan(nx), Py = axis_plan(ny);
+    const int pitch = nx + 1, lx = __ffs(nx) - 1;
+    const float inv = 1.0f / (float)(ny * nx);
+    fft_axis_part<true, true>(g, Px, ny, pitch, twx, 1, Px.ns);
+    fft_axis_part<true, false>(g, Py, nx, pitch, twy, 0, Py.ns - 1);
+    switch (Py.lr(Py.ns - 1)) {
+    case 1: col_mid_stage<2>(g, Py.ln, lx, pitch, inv, h); break;
+    case 2: col_mid_stage<4>(g, Py.ln, lx, pitch, inv, h); break;
+    case 3: col_mid_stage<8>(g, Py.ln, lx, pitch, inv, h); break;
+    default: col_mid_stage<16>(g, Py.ln, lx, pitch, inv, h); break;
+    }
+    fft_axis_part<false, false>(g, Py, nx, pitch, twy, 0, Py.ns - 1);
+    fft_axis_part<false, true>(g, Px, ny, pitch, twx, 1, Px.ns);
+}
+
+template <bool LOAD, bool FIRST, class In, class Mid>
+__device__ void row_outer(float2 *g, int ny, int nx, const float2 *twx, In &&in, Mid &&mid)
+{
+    const AxisPlan Px = axis_plan(nx);
+    const int ly = __ffs(ny) - 1;
+    switch (Px.lr0) {
+    case 1: row_outer_stage<2, LOAD, FIRST>(g, Px.ln, ly, nx + 1, twx, in, mid); break;
+    case 2: row_outer_stage<4, LOAD, FIRST>(g, Px.ln, ly, nx + 1, twx, in, mid); break;
+    case 3: row_outer_stage<8, LOAD, FIRST>(g, Px.ln, ly, nx + 1, twx, in, mid); break;
+    default: row_outer_stage<16, LOAD, FIRST>(g, Px.ln, ly, nx + 1, twx, in, mid); break;
+    }
+}
+
 // natural frequencies (ky index, kx index) of the spectrum at grid position (a, b)
 struct SpecMap {
     AxisPlan py, px;
@@ -190,45 +304,35 @@ struct SpecMap {
     __device__ int fx(int b) const { return axis_freq(px, b); }
 };
 
-// g <- D g (adjoint: D^H g), including the 1/P of the inverse transform.
-__device__ void defocus_apply_smem(float2 *g, int ny, int nx, const float2 *__restrict__ H,
-                                   bool adjoint, const float2 *twy, const float2 *twx)
-{
-    const int pitch = nx + 1, P = ny * nx, lx = __ffs(nx) - 1;
-    SpecMap sm;
-    sm.init(ny, nx);
-    fft2_fwd(g, ny, nx, twy, twx);
-    const float inv = 1.0f / (float)P;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const int a = i >> lx, b = i & (nx - 1);
-        float2 h = H[sm.fy(a) * nx + sm.fx(b)];
-        if (adjoint) h.y = -h.y;
-        g[a * pitch + b] = cscale(cmul(g[a * pitch + b], h), inv);
-    }
-    __syncthreads();
-    fft2_inv(g, ny, nx, twy, twx);
-}
-
 static size_t defocus_smem(int ny, int nx)
 {
-    return sizeof(float2) * ((size_t)ny * (nx + 1) + ny / 2 + nx / 2) + 64 * sizeof(double);
+    return sizeof(float2) * ((size_t)ny * (nx + 1) + ny + nx) + 64 * sizeof(double);
 }
 
 __global__ void k_defocus_forward(int ny, int nx, int Nd, const float2 *__restrict__ Zd,
                                   const float2 *__restrict__ H, float *__restrict__ Ydef)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int P = ny * nx, pitch = nx + 1;
+    const int P = ny * nx, pitch = nx + 1, lx = __ffs(nx) - 1;
     float2 *g = reinterpret_cast<float2 *>(smem_raw);
-    float2 *twy = g + (size_t)ny * pitch, *twx = twy + ny / 2;
+    float2 *twy = g + (size_t)ny * pitch, *twx = twy + ny;
+    SpecMap sm;
+    sm.init(ny, nx);
     make_tw(twy, ny);
     make_tw(twx, nx);
+    __syncthreads();
     for (int n = blockIdx.x; n < Nd; n += gridDim.x) {
-        for (int i = threadIdx.x; i < P; i += blockDim.x) g[(i / nx) * pitch + i % nx] = Zd[(size_t)n * P + i];
-        __syncthreads();
-        defocus_apply_smem(g, ny, nx, H, false, twy, twx);
-        for (int i = threadIdx.x; i < P; i += blockDim.x) Ydef[(size_t)n * P + i] = cabs2(g[(i / nx) * pitch + i % nx]);
-        __syncthreads();
+        const float2 *cn = Zd + (size_t)n * P;
+        float *out = Ydef + (size_t)n * P;
+        row_outer<true, true>(
+            g, ny, nx, twx, [&](int a, int b) { return cn[(a << lx) + b]; }, [](int, int, float2 x) { return x; });
+        defocus_inner(g, ny, nx, twy, twx, [&](int a, int b) { return H[sm.fy(a) * nx + sm.fx(b)]; });
+        row_outer<false, false>(
+            g, ny, nx, twx, [](int, int) { return make_float2(0.f, 0.f); },
+            [&](int a, int b, float2 x) {
+                out[(a << lx) + b] = cabs2(x);
+                return x;
+            });
     }
 }
 
@@ -371,7 +475,7 @@ __device__ __forceinline__ float2 ramp_st(int st, int a, int b, const float2 *ry
 
 static size_t defocus2x_smem(int ny, int nx, int grids)
 {
-    return sizeof(float2) * ((size_t)grids * ny * (nx + 1) + ny / 2 + nx / 2 + ny + nx) + 64 * sizeof(double);
+    return sizeof(float2) * ((size_t)grids * ny * (nx + 1) + 2 * (ny + nx)) + 64 * sizeof(double);
 }
 
 bool phase_fit2x_fits(int ny, int nx);
@@ -390,7 +494,7 @@ __global__ void k_defocus_forward2x(int ny, int nx, int Nd, const float2 *__rest
     const int P = ny * nx, pitch = nx + 1, lx = __ffs(nx) - 1;
     float2 *g = reinterpret_cast<float2 *>(smem_raw);
     float2 *Xs = g + (size_t)ny * pitch;
-    float2 *twy = Xs + (size_t)ny * pitch, *twx = twy + ny / 2, *ry = twx + nx / 2, *rx = ry + ny;
+    float2 *twy = Xs + (size_t)ny * pitch, *twx = twy + ny, *ry = twx + nx, *rx = ry + ny;
     make_tw(twy, ny);
     make_tw(twx, nx);
     make_ramps(ry, rx, ny, nx);
@@ -537,8 +641,16 @@ __device__ void pf_part_sums(const float *part, int nb, int P, int k0, int k1, d
     for (int base = k0 + 4 * warp; base < k1; base += 4 * nw) {
         const int k = base + slot;
         double s = 0.0;
-        if (k < k1)
-            for (int b = sub; b < nb; b += 8) s += (double)__ldcg(part + (size_t)b * P + k);
+        if (k < k1) {
+            // eight loads in flight (one at a time, the walk was a chain of L2 latencies)
+            for (int b0 = sub; b0 < nb; b0 += 64) {
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; q++) v[q] = b0 + 8 * q < nb ? __ldcg(part + (size_t)(b0 + 8 * q) * P + k) : 0.f;
+#pragma unroll
+                for (int q = 0; q < 8; q++) s += (double)v[q];
+            }
+        }
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         s += __shfl_xor_sync(0xffffffffu, s, 4);
@@ -546,27 +658,32 @@ __device__ void pf_part_sums(const float *part, int nb, int P, int k0, int k1, d
     }
 }
 
-// Block sums of 32 values per thread (kPfDots): within each warp a
+// Block sums of 32 values per thread (kPfDots) of the first nw warps (the others
+// hold zeros: a CTA's chunk is a few hundred elements, and FP64 runs at two
+// lanes a cycle): within each warp a
 // transposing xor tree leaves value l's warp sum in lane l (31 additions per
 // lane instead of 32 x 5), then 32 threads add the warps' sums in order.
 static_assert(kPfDots == 32, "block_sum32 reduces 32 values");
-__device__ void block_sum32(double (&v)[32], double *red, double *out)
+__device__ void block_sum32(double (&v)[32], int nw, double *red, double *out)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < nw) {
 #pragma unroll
-    for (int h = 16; h >= 1; h >>= 1) {
-        const bool upper = (lane & h) != 0;
+        for (int h = 16; h >= 1; h >>= 1) {
+            const bool upper = (lane & h) != 0;
 #pragma unroll
-        for (int i = 0; i < h; i++) {
-            const double send = upper ? v[i] : v[i + h];
-            const double keep = upper ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+            for (int i = 0; i < h; i++) {
+                const double send = upper ? v[i] : v[i + h];
+                const double keep = upper ? v[i + h] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+            }
         }
+        red[lane * nw + warp] = v[0];
     }
-    red[lane * nw + warp] = v[0];
     __syncthreads();
     if (threadIdx.x < 32) {
         double s = 0.0;
+#pragma unroll 4
         for (int w = 0; w < nw; w++) s += red[threadIdx.x * nw + w];
         out[threadIdx.x] = s;
     }
@@ -594,42 +711,112 @@ struct PFGram {
     int floor_reached;  // the last accepted step lowered g by at most tol g (PhaseFitParams::tol)
 };
 
-// compact-form coefficients (one thread); restart = 1 selects p = -g / max|g|
-__device__ void pf_coefficients(PFGram &G)
+// Compact-form coefficients (one warp, every lane the same work, in registers);
+// restart = 1 selects p = -g / max|g|.  At most 6 x 6, the substitutions column
+// by column: a step of the chain is one multiplication and one FMA.
+__device__ void pf_coefficients(PFGram &G, int lane)
 {
     const int np = G.np;
-    for (int i = 0; i < kPfSlots; i++) G.c1[i] = G.c2[i] = 0.0;
-    G.restart = 1;
+    double c1[kMaxMem], c2[kMaxMem], acc[kMaxMem], rd[kMaxMem], gamma = 1.0, pg = 0.0;
+    bool ok = false;
     if (np > 0) {
-        const double gamma = G.SY[np - 1][np - 1] / G.YY[np - 1][np - 1];
-        double c1[kPfSlots], c2[kPfSlots];
-        for (int i = np - 1; i >= 0; i--) {
-            double s = -G.Sg[i];
-            for (int j = i + 1; j < np; j++) s -= G.SY[i][j] * c2[j];
-            c2[i] = s * G.rD[i];
+        gamma = G.SY[np - 1][np - 1] / G.YY[np - 1][np - 1];
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) {
+            acc[i] = i < np ? -G.Sg[i] : 0.0;
+            rd[i] = i < np ? G.rD[i] : 0.0;
         }
-        for (int i = 0; i < np; i++) {
-            double rhs = -G.SY[i][i] * c2[i] - gamma * G.Yg[i];
-            for (int j = 0; j < np; j++) rhs -= gamma * G.YY[i < j ? i : j][i < j ? j : i] * c2[j];
-            for (int j = 0; j < i; j++) rhs -= G.SY[j][i] * c1[j];
-            c1[i] = rhs * G.rD[i];
+#pragma unroll
+        for (int j = kMaxMem - 1; j >= 0; j--) {
+            c2[j] = acc[j] * rd[j];  // 0 for j >= np
+#pragma unroll
+            for (int i = 0; i < j; i++)
+                if (j < np) acc[i] -= G.SY[i][j] * c2[j];
         }
-        double pg = gamma * G.gg;
-        for (int i = 0; i < np; i++) pg += c1[i] * G.Sg[i] + gamma * c2[i] * G.Yg[i];
-        if (pg > 0.0 && isfinite(pg)) {
-            G.gamma = gamma;
-            for (int i = 0; i < np; i++) {
-                G.c1[i] = c1[i];
-                G.c2[i] = gamma * c2[i];
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) {
+            acc[i] = 0.0;
+            if (i < np) {
+                double yc = G.Yg[i];
+#pragma unroll
+                for (int j = 0; j < kMaxMem; j++)
+                    if (j < np) yc += G.YY[i < j ? i : j][i < j ? j : i] * c2[j];
+                acc[i] = -G.SY[i][i] * c2[i] - gamma * yc;
             }
-            G.gp = -pg;
-            G.restart = 0;
-            return;
         }
-        G.np = 0;
+        pg = gamma * G.gg;
+#pragma unroll
+        for (int j = 0; j < kMaxMem; j++) {
+            c1[j] = acc[j] * rd[j];
+            if (j < np) {
+#pragma unroll
+                for (int i = j + 1; i < kMaxMem; i++)
+                    if (i < np) acc[i] -= G.SY[j][i] * c1[j];
+                pg += c1[j] * G.Sg[j] + gamma * c2[j] * G.Yg[j];
+            }
+        }
+        ok = pg > 0.0 && isfinite(pg);
     }
-    G.gamma = 1.0;
-    G.gp = G.gmax > 0.0 ? -G.gg / G.gmax : 0.0;
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) {
+            G.c1[i] = ok ? c1[i] : 0.0;
+            G.c2[i] = ok ? gamma * c2[i] : 0.0;
+        }
+        G.restart = ok ? 0 : 1;
+        G.gamma = ok ? gamma : 1.0;
+        G.gp = ok ? -pg : (G.gmax > 0.0 ? -G.gg / G.gmax : 0.0);
+        if (!ok) G.np = 0;
+    }
+    __syncwarp();
+}
+
+// The pair bookkeeping after an accepted step (one warp; t: the batched dot
+// products, ft: the new loss), then the next direction's coefficients.
+__device__ void pf_gram_update(PFGram &G, int lane, int m, double ft, double tol)
+{
+    const double *t = G.red;
+    const int np = G.np;
+    if (lane <= np) {
+        G.SY[lane][np] = t[4 * lane + 0];
+        G.YY[lane][np] = t[4 * lane + 1];
+        G.Sg[lane] = t[4 * lane + 2];
+        G.Yg[lane] = t[4 * lane + 3];
+    }
+    const double sy = t[4 * np + 0], yy = t[4 * np + 1], ss = t[4 * kPfSlots + 0];
+    const bool accept = sy > 1e-10 * sqrt(ss) * sqrt(yy) && sy > 0.0;
+    if (accept && lane == 0) G.rD[np] = 1.0 / sy;
+    __syncwarp();
+    if (accept && np + 1 > m) {  // drop the oldest pair; its slot becomes the free one
+        double a[kPfSlots], b[kPfSlots], sg = 0.0, yg = 0.0, rd = 0.0;
+        int sl = 0;
+        const bool mine = lane < m;
+#pragma unroll
+        for (int j = 0; j < kPfSlots; j++) {
+            a[j] = mine && j < m ? G.SY[lane + 1][j + 1 < kPfSlots ? j + 1 : 0] : 0.0;
+            b[j] = mine && j < m ? G.YY[lane + 1][j + 1 < kPfSlots ? j + 1 : 0] : 0.0;
+        }
+        if (mine) sg = G.Sg[lane + 1], yg = G.Yg[lane + 1], rd = G.rD[lane + 1], sl = G.slot[lane + 1];
+        else if (lane == m) sl = G.slot[0];
+        __syncwarp();
+        if (mine) {
+#pragma unroll
+            for (int j = 0; j < kPfSlots; j++)
+                if (j < m) G.SY[lane][j] = a[j], G.YY[lane][j] = b[j];
+            G.Sg[lane] = sg, G.Yg[lane] = yg, G.rD[lane] = rd;
+        }
+        if (lane <= m) G.slot[lane] = sl;
+    }
+    if (lane == 0) {
+        G.gg = t[4 * kPfSlots + 1];
+        G.gmax = t[kPfDots - 2];
+        G.floor_reached = tol > 0.0 && G.f - ft <= tol * G.f;
+        G.f = ft;
+        if (accept) G.np = np + 1 > m ? m : np + 1;
+    }
+    __syncwarp();
+    pf_coefficients(G, lane);
 }
 
 // The 2x-padded operator's share of pf_eval for pattern n: on return g holds
@@ -637,7 +824,7 @@ __device__ void pf_coefficients(PFGram &G)
 // G = I_n - |w|^2, and the loss of the pattern is added to fpl.  Xs and S are
 // two more grids: X h, and the accumulated cropped spectrum of w G.
 __device__ void pf_pattern2x(const PhaseFitParams &Pp, int n, float2 *g, float2 *Xs, float2 *S, const float2 *twy,
-                             const float2 *twx, const float2 *ry, const float2 *rx, float &fpl)
+                             const float2 *twx, const float2 *ry, const float2 *rx, const float2 *Hs, float &fpl)
 {
     const int ny = Pp.ny, nx = Pp.nx, P = ny * nx, pitch = nx + 1, lx = __ffs(nx) - 1;
     const float *In = Pp.Ydef + (size_t)n * 4 * P;
@@ -647,7 +834,7 @@ __device__ void pf_pattern2x(const PhaseFitParams &Pp, int n, float2 *g, float2 
     fft2_fwd(g, ny, nx, twy, twx);
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         const int a = i >> lx, b = i & (nx - 1), gi = a * pitch + b;
-        Xs[gi] = cmul(g[gi], Pp.H[sm.fy(a) * nx + sm.fx(b)]);
+        Xs[gi] = cmul(g[gi], Hs ? Hs[i] : Pp.H[sm.fy(a) * nx + sm.fx(b)]);
         S[gi] = make_float2(0.f, 0.f);
     }
     __syncthreads();
@@ -676,7 +863,7 @@ __device__ void pf_pattern2x(const PhaseFitParams &Pp, int n, float2 *g, float2 
     }
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         const int a = i >> lx, b = i & (nx - 1), gi = a * pitch + b;
-        g[gi] = cscale(cmulc(S[gi], Pp.H[sm.fy(a) * nx + sm.fx(b)]), inv);
+        g[gi] = cscale(cmulc(S[gi], Hs ? Hs[i] : Pp.H[sm.fy(a) * nx + sm.fx(b)]), inv);
     }
     __syncthreads();
     fft2_inv(g, ny, nx, twy, twx);
@@ -685,26 +872,29 @@ __device__ void pf_pattern2x(const PhaseFitParams &Pp, int n, float2 *g, float2 
 // Loss and gradient partials of this CTA's patterns for the phase table u:
 // part[blockIdx.x][:] (FP32, at most a few patterns per CTA) and fpart (FP64).
 // ex (kind 1 only): the grids Xs, S and the ramps ry, rx of pf_pattern2x.
+// Hs: H in spectrum order (both kinds), NULL where it does not fit.
 struct PFExtra {
     float2 *Xs, *S;
     const float2 *ry, *rx;
+    const float2 *Hs;
 };
 
+template <int KIND>
 __device__ void pf_eval(const PhaseFitParams &Pp, const PFWork &W, float2 *g, const float2 *twy,
                         const float2 *twx, double *red, double *out, const PFExtra &ex)
 {
     const int ny = Pp.ny, nx = Pp.nx, P = ny * nx, pitch = nx + 1, lx = __ffs(nx) - 1;
     auto at = [&](int k) { return (k >> lx) * pitch + (k & (nx - 1)); };
     float *part = W.part + (size_t)blockIdx.x * P;
-    for (int k = threadIdx.x; k < P; k += blockDim.x) part[k] = 0.f;
     double fl = 0.0;
-    if (Pp.kind == 1) {
+    if constexpr (KIND == 1) {
+        for (int k = threadIdx.x; k < P; k += blockDim.x) part[k] = 0.f;
         for (int n = blockIdx.x; n < Pp.Nd; n += gridDim.x) {
             const float2 *cn = Pp.Zd + (size_t)n * P;
             for (int k = threadIdx.x; k < P; k += blockDim.x) g[at(k)] = cmul(cn[k], __ldcg(W.u + k));
             __syncthreads();
             float fpl = 0.f;
-            pf_pattern2x(Pp, n, g, ex.Xs, ex.S, twy, twx, ex.ry, ex.rx, fpl);
+            pf_pattern2x(Pp, n, g, ex.Xs, ex.S, twy, twx, ex.ry, ex.rx, ex.Hs, fpl);
             fl += (double)fpl;
             for (int k = threadIdx.x; k < P; k += blockDim.x) {
                 const float2 v = cmulc(g[at(k)], cn[k]);  // conj(c_n) A^H(w G)
@@ -713,35 +903,41 @@ __device__ void pf_eval(const PhaseFitParams &Pp, const PFWork &W, float2 *g, co
             }
             __syncthreads();
         }
-        double fv[1] = {fl};
-        block_sum<1, double>(fv, red, out);
-        if (threadIdx.x == 0) W.fpart[blockIdx.x] = out[0];
-        return;
-    }
-    for (int n = blockIdx.x; n < Pp.Nd; n += gridDim.x) {
-        const float2 *cn = Pp.Zd + (size_t)n * P;
-        const float *In = Pp.Ydef + (size_t)n * P;
-        for (int k = threadIdx.x; k < P; k += blockDim.x)
-            g[at(k)] = cmul(cn[k], __ldcg(W.u + k));
-        __syncthreads();
-        defocus_apply_smem(g, ny, nx, Pp.H, false, twy, twx);
-        float fpl = 0.f;
-        for (int k = threadIdx.x; k < P; k += blockDim.x) {
-            const int gi = at(k);
-            const float2 w = g[gi];
-            const float Gv = In[k] - cabs2(w);
-            fpl = fmaf(Gv, Gv, fpl);
-            g[gi] = cscale(w, Gv);
+    } else {
+        SpecMap sm;
+        sm.init(ny, nx);
+        auto hat = [&](int a, int b) { return ex.Hs ? ex.Hs[(a << lx) + b] : Pp.H[sm.fy(a) * nx + sm.fx(b)]; };
+        auto none = [](int, int, float2 x) { return x; };
+        for (int n = blockIdx.x; n < Pp.Nd; n += gridDim.x) {
+            const float2 *cn = Pp.Zd + (size_t)n * P;
+            const float *In = Pp.Ydef + (size_t)n * P;
+            float fpl = 0.f;
+            // w = D(c_n u)
+            row_outer<true, true>(
+                g, ny, nx, twx, [&](int a, int b) { return cmul(cn[(a << lx) + b], __ldcg(W.u + (a << lx) + b)); }, none);
+            defocus_inner(g, ny, nx, twy, twx, hat);
+            // G = I_n - |w|^2, and D^H(w G)
+            row_outer<false, true>(
+                g, ny, nx, twx, [](int, int) { return make_float2(0.f, 0.f); },
+                [&](int a, int b, float2 w) {
+                    const float Gv = In[(a << lx) + b] - cabs2(w);
+                    fpl = fmaf(Gv, Gv, fpl);
+                    return cscale(w, Gv);
+                });
+            defocus_inner(g, ny, nx, twy, twx, [&](int a, int b) { return cconj(hat(a, b)); });
+            const bool first = n == (int)blockIdx.x;
+            row_outer<false, false>(
+                g, ny, nx, twx, [](int, int) { return make_float2(0.f, 0.f); },
+                [&](int a, int b, float2 x) {
+                    const int k = (a << lx) + b;
+                    const float2 v = cmulc(x, cn[k]);  // conj(c_n) D^H(w G)
+                    const float2 cu = __ldcg(W.u + k);
+                    const float d = -4.f * fmaf(cu.x, v.y, -cu.y * v.x);  // -4 Im(conj(u) v)
+                    part[k] = first ? d : part[k] + d;
+                    return x;
+                });
+            fl += (double)fpl;
         }
-        fl += (double)fpl;
-        __syncthreads();
-        defocus_apply_smem(g, ny, nx, Pp.H, true, twy, twx);
-        for (int k = threadIdx.x; k < P; k += blockDim.x) {
-            const float2 v = cmulc(g[at(k)], cn[k]);  // conj(c_n) D^H(w G)
-            const float2 cu = __ldcg(W.u + k);
-            part[k] += -4.f * fmaf(cu.x, v.y, -cu.y * v.x);  // -4 Im(conj(u) v)
-        }
-        __syncthreads();
     }
     double fv[1] = {fl};
     block_sum<1, double>(fv, red, out);
@@ -755,22 +951,39 @@ __device__ void pf_eval(const PhaseFitParams &Pp, const PFWork &W, float2 *g, co
 // batched FP64 reduction of dot products per accepted step.  Every CTA holds
 // the same FP64 L-BFGS scalars (identical sums in identical order), so all
 // take the same decisions.
+//
+// Bound by latency, not by a rate: a fit is a few evaluations in a row, each a
+// chain of about 60 FFT stages of one grid with a block barrier between them,
+// and the CTAs past the Nd patterns only help with the chunk-owned vectors.  So
+// what counts is each stage's instructions: index arithmetic by shifts, neighbouring
+// passes of the same axis (last inverse stage, the product, first forward
+// stage) in one, H and full-length twiddle tables in shared memory, and the
+// FP64 scalars, on a pipe of two lanes a cycle, by one warp in registers.
+// 128 x 64 pixels, 50 patterns: 1235 -> 901 us the fit (padded operator: 4402
+// -> 3750); 1024 threads a CTA spill and take 8 % longer than 512.
+template <int KIND>
 __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ny = Pp.ny, nx = Pp.nx, P = ny * nx, m = Pp.m, nb = gridDim.x;
-    const int ngrid = Pp.kind == 1 ? 3 : 1;
+    constexpr int ngrid = KIND == 1 ? 3 : 1;
     float2 *g = reinterpret_cast<float2 *>(smem_raw);
-    float2 *twy = g + (size_t)ngrid * ny * (nx + 1), *twx = twy + ny / 2;
-    float2 *ry = twx + nx / 2, *rx = ry + ny;
+    float2 *twy = g + (size_t)ngrid * ny * (nx + 1), *twx = twy + ny;
+    float2 *ry = twx + nx, *rx = ry + ny;
     double *red = reinterpret_cast<double *>(rx + nx + 1);
     double *out = red + 32 * kPfDots;
+    float2 *Hs = Pp.stage_H ? reinterpret_cast<float2 *>(out + kPfDots + 8) : nullptr;
     __shared__ PFGram G;
     PFWork W = pf_carve(Pp.ws, P, m, nb);
     make_tw(twy, ny);
     make_tw(twx, nx);
-    PFExtra ex{g + (size_t)ny * (nx + 1), g + (size_t)2 * ny * (nx + 1), ry, rx};
-    if (Pp.kind == 1) make_ramps(ry, rx, ny, nx);
+    PFExtra ex{g + (size_t)ny * (nx + 1), g + (size_t)2 * ny * (nx + 1), ry, rx, Hs};
+    if (Hs) {
+        SpecMap sm;
+        sm.init(ny, nx);
+        for (int i = threadIdx.x; i < P; i += blockDim.x) Hs[i] = Pp.H[sm.fy(i / nx) * nx + sm.fx(i % nx)];
+    }
+    if (KIND == 1) make_ramps(ry, rx, ny, nx);
     const int tid = threadIdx.x, nt = blockDim.x;
     const int chunk = (P + nb - 1) / nb, k0 = min(P, blockIdx.x * chunk), k1 = min(P, k0 + chunk);
     double *Sg_ = W.S, *Yg_ = W.Y;
@@ -778,7 +991,8 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
     // reduce kPfDots per-thread values over the grid: block sums to pdot[b], a
     // grid barrier, then every CTA adds the nb partials in order into G.red
     auto grid_dots = [&](double (&v)[kPfDots], double vmax) -> bool {
-        block_sum32(v, red, out);
+        const int nw = min(nt, k1 - k0 + 31) >> 5;  // warps with elements of the chunk
+        block_sum32(v, nw > 0 ? nw : 1, red, out);
         __shared__ double mx[32];
         double mv = vmax;
         for (int o = 16; o > 0; o >>= 1) mv = fmax(mv, __shfl_xor_sync(0xffffffffu, mv, o));
@@ -837,7 +1051,7 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
         bail();
         return;
     }
-    pf_eval(Pp, W, g, twy, twx, red, out, ex);
+    pf_eval<KIND>(Pp, W, g, twy, twx, red, out, ex);
     if (!grid_sync(Pp.sync, Pp.err, Pp.wait_spins, Pp.withhold_release)) {
         bail();
         return;
@@ -865,8 +1079,9 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
         G.gmax = G.red[kPfDots - 2];
         G.np = 0;
         for (int i = 0; i < kPfSlots; i++) G.slot[i] = i;
-        pf_coefficients(G);
     }
+    __syncwarp();
+    if (tid < 32) pf_coefficients(G, tid);
     __syncthreads();
 
     int done = 0;
@@ -901,7 +1116,7 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
         bail();
         return;
     }
-            pf_eval(Pp, W, g, twy, twx, red, out, ex);
+            pf_eval<KIND>(Pp, W, g, twy, twx, red, out, ex);
             if (!grid_sync(Pp.sync, Pp.err, Pp.wait_spins, Pp.withhold_release)) {
         bail();
         return;
@@ -944,40 +1159,7 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
             bail();
             return;
         }
-            if (tid == 0) {
-                const double *t = G.red;
-                for (int i = 0; i <= np; i++) {
-                    G.SY[i][np] = t[4 * i + 0];
-                    G.YY[i][np] = t[4 * i + 1];
-                    G.Sg[i] = t[4 * i + 2];
-                    G.Yg[i] = t[4 * i + 3];
-                }
-                const double sy = t[4 * np + 0], yy = t[4 * np + 1], ss = t[4 * kPfSlots + 0];
-                G.gg = t[4 * kPfSlots + 1];
-                G.gmax = t[kPfDots - 2];
-                G.floor_reached = Pp.tol > 0.0 && G.f - ft <= Pp.tol * G.f;
-                G.f = ft;
-                if (sy > 1e-10 * sqrt(ss) * sqrt(yy) && sy > 0.0) {
-                    G.rD[np] = 1.0 / sy;
-                    G.np = np + 1;
-                    if (G.np > m) {  // drop the oldest pair; its slot becomes the free one
-                        const int s0 = G.slot[0];
-                        for (int i = 0; i < m; i++) {
-                            for (int j = i; j < m; j++) {
-                                G.SY[i][j] = G.SY[i + 1][j + 1];
-                                G.YY[i][j] = G.YY[i + 1][j + 1];
-                            }
-                            G.Sg[i] = G.Sg[i + 1];
-                            G.Yg[i] = G.Yg[i + 1];
-                            G.rD[i] = G.rD[i + 1];
-                            G.slot[i] = G.slot[i + 1];
-                        }
-                        G.slot[m] = s0;
-                        G.np = m;
-                    }
-                }
-                pf_coefficients(G);
-            }
+            if (tid < 32) pf_gram_update(G, tid, m, ft, Pp.tol);
             __syncthreads();
         }
         done = it + 1;
@@ -1012,7 +1194,7 @@ __global__ void __launch_bounds__(512) k_phase_fit(PhaseFitParams Pp)
 static size_t phase_fit_smem(int ny, int nx, int kind)
 {
     const int ngrid = kind == 1 ? 3 : 1;
-    return sizeof(float2) * ((size_t)ngrid * ny * (nx + 1) + ny / 2 + nx / 2 + ny + nx + 1) +
+    return sizeof(float2) * ((size_t)ngrid * ny * (nx + 1) + 2 * (ny + nx) + 1) +
            sizeof(double) * (32 * kPfDots + kPfDots + 8) + 64;
 }
 
@@ -1022,17 +1204,20 @@ cudaError_t launch_phase_fit(const PhaseFitParams &p, cudaStream_t s)
 {
     const int grid = phase_fit_grid(p.ny, p.nx, p.Nd);
     const int P = p.ny * p.nx;
-    const size_t sm = phase_fit_smem(p.ny, p.nx, p.kind);
-    (void)P;
-    cudaError_t e = cudaFuncSetAttribute(k_phase_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    size_t sm = phase_fit_smem(p.ny, p.nx, p.kind);
+    PhaseFitParams pp = p;
+    // the kernel H beside the grids where it fits
+    pp.stage_H = sm + sizeof(float2) * P + sizeof(PFGram) + 1024 <= 227 * 1024;
+    if (pp.stage_H) sm += sizeof(float2) * P;
+    const void *kernel = p.kind == 1 ? (const void *)k_phase_fit<1> : (const void *)k_phase_fit<0>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_phase_fit, 512, sm);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 512, sm);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
-    PhaseFitParams pp = p;
     void *args[] = {&pp};
-    return cudaLaunchCooperativeKernel((const void *)k_phase_fit, dim3(grid), dim3(512), args, sm, s);
+    return cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(512), args, sm, s);
 }
 
 }  // namespace tmr

@@ -203,6 +203,7 @@ struct PhaseFitParams {
     bool withhold_release;  // test hook: the barrier is never released
     int kind;               // 0: same-grid operator; 1: angular spectrum with 2x padding (Ydef [Nd][4P])
     double tol;             // > 0: stop after an accepted step lowering g by at most tol g
+    bool stage_H = false;   // set by launch_phase_fit: H is staged in shared memory
 };
 size_t phase_fit_workspace_doubles(int P, int Nd, int m, int grid);
 int phase_fit_grid(int ny, int nx, int Nd);
