@@ -773,19 +773,21 @@ static size_t ydef_floats(const tmr_handle *h)
     return (size_t)h->Nd * h->M * (h->dkind == TMR_DEFOCUS_ANGULAR_2X ? 4 : 1);
 }
 
-// Zd <- the fields c_n of T: probe patterns (kind 0) or incident fields (kind 1)
+// Zd <- the fields c_n of T: probe patterns (kind 0) or incident fields (kind
+// 1); wts <- the rows' energies, the weights of the fit's constant phase
 static cudaError_t defocus_fields(tmr_handle *h, const float2 *dT)
 {
-    if (h->dkind == TMR_DEFOCUS_ANGULAR_2X)
-        return launch_incident_fields(h->M, h->N, h->Nd, dT, h->incident, h->Zd, h->stream);
-    return launch_fields(h->N, h->M, h->J, h->Nd, dT, h->masks, h->tw, h->Zd, h->stream, h->xk);
+    if (h->dkind == TMR_DEFOCUS_ANGULAR_2X) {
+        const cudaError_t e = launch_incident_fields(h->M, h->N, h->Nd, dT, h->incident, h->Zd, h->stream);
+        return e == cudaSuccess ? launch_row_energy(h->N, h->M, dT, h->wts, h->stream) : e;
+    }
+    return launch_fields(h->N, h->M, h->J, h->Nd, dT, h->masks, h->tw, h->Zd, h->wts, h->stream, h->xk);
 }
 
+// after defocus_fields(h, Tin)
 static tmr_status run_phase_fit(tmr_handle *h, const float2 *Tin, const float *dYdef, double *dphi,
                                 float2 *Tout)
 {
-    // weights of the constant-phase normalisation: row energies of T_est
-    TMR_CUDA(launch_row_energy(h->N, h->M, Tin, h->wts, h->stream), "row energy");
     TMR_CUDA(cudaMemsetAsync(h->pf_sync, 0, sizeof(unsigned) * 4, h->stream), "memset");
     TMR_CUDA(cudaMemsetAsync(h->pf_err, 0, sizeof(int) * 4, h->stream), "memset");
     PhaseFitParams p{};

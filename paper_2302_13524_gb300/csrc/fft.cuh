@@ -345,4 +345,53 @@ __device__ __forceinline__ void block_fft_pp(float2 (&v)[N / T], float2 *buf, co
     ph ^= (Pl::P - 1) & 1;
 }
 
+// ---------------------------------------------------------------------------
+// Radix-16 plans whose last pass takes its twiddles from four per-thread bases,
+// w, w^2, w^4 and w^8 with w = exp(-2 pi i tid / N), each rounded from FP64.
+// Every power is a product of at most four of them; from w alone the rounding
+// of w itself would grow fifteenfold in w^15 (gradient at N = 2048: 1.8e-6
+// relative error instead of 1.0e-6).
+template <int SIGN>
+__device__ __forceinline__ void twiddle_powers16(float2 (&x)[16], const float2 (&wb)[4])
+{
+    float2 w[16];
+    w[1] = wb[0], w[2] = wb[1], w[4] = wb[2], w[8] = wb[3];
+    if constexpr (SIGN > 0) {
+#pragma unroll
+        for (int k = 1; k < 16; k *= 2) w[k].y = -w[k].y;
+    }
+#pragma unroll
+    for (int k = 1; k < 16; k++) {
+        const int top = k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1;
+        if (k != top) w[k] = cmul(w[top], w[k - top]);
+        x[k] = cmul(x[k], w[k]);
+    }
+}
+
+// As block_fft_pp (ping-pong exchanges), 16 points and one butterfly per thread.
+template <int N, int T, int SIGN, int p>
+__device__ __forceinline__ void fft_passes_pp16(float2 (&v)[16], float2 *b0, float2 *b1, const float2 *tw,
+                                                const float2 (&wb)[4], int tid)
+{
+    using Pl = FftPlan<N, 16>;
+    static_assert(N / T == 16, "16 points per thread");
+    if constexpr (p < Pl::P - 1) {
+        fft_pass<N, T, Pl::radix(p), Pl::ns(p), Pl::tw_off(p), SIGN, false, false>(v, (p & 1) ? b1 : b0, tw, tid);
+        fft_passes_pp16<N, T, SIGN, p + 1>(v, b0, b1, tw, wb, tid);
+    } else {
+        twiddle_powers16<SIGN>(v, wb);
+        dft_small<16, SIGN>(v);
+    }
+}
+
+template <int N, int T, int SIGN>
+__device__ __forceinline__ void block_fft_pp16(float2 (&v)[16], float2 *buf, const float2 *tw, const float2 (&wb)[4],
+                                               int tid, int &ph)
+{
+    using Pl = FftPlan<N, 16>;
+    float2 *b0 = buf + (ph ? fft_buf_len(N) : 0), *b1 = buf + (ph ? 0 : fft_buf_len(N));
+    fft_passes_pp16<N, T, SIGN, 0>(v, b0, b1, tw, wb, tid);
+    ph ^= (Pl::P - 1) & 1;
+}
+
 }  // namespace tmr

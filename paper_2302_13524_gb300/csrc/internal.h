@@ -58,9 +58,10 @@ cudaError_t launch_forward(int N, int M, int J, const float2 *T, const float2 *m
 cudaError_t launch_grad(int N, int M, int J, const float2 *T, const float2 *masks,
                         const float2 *tw, const float *Y, float *loss, float2 *G, cudaStream_t s,
                         int prec = 0, int cost = 0);
-// c_n[r] = (Q T[r])[n] for n < Nd, written as Zd[n][r] (the defocus fields).
+// c_n[r] = (Q T[r])[n] for n < Nd, written as Zd[n][r] (the defocus fields);
+// w non-NULL: also w[r] = ||T[r]||^2.
 cudaError_t launch_fields(int N, int M, int J, int Nd, const float2 *T, const float2 *masks,
-                          const float2 *tw, float2 *Zd, cudaStream_t s, int prec = 0);
+                          const float2 *tw, float2 *Zd, float *w, cudaStream_t s, int prec = 0);
 // y (float32 [M][K]) -> y16 (FP16, each row divided by its largest |y|) and the row scales
 cudaError_t launch_pack_f16(int M, size_t K, const float *y, void *y16, float *ysc, cudaStream_t s);
 // T[r] *= exp(i phi[r])

@@ -1,9 +1,9 @@
 // kernels.cu -- fused forward-model and gradient kernels, defocus fields,
 // phase application, and the host-side FFT twiddle tables.
 //
-// Forward model (Eq. optTMsmall2): one CTA per (row, mask) computes
-// z = F(d_j .* t) in registers and writes |z|^2.  Gradient (Eq. derivative,
-// App. A): one CTA per row loops over the J masks, keeping the accumulated
+// Forward model (Eq. optTMsmall2): a CTA keeps one mask and, row by row,
+// computes z = F(d_j .* t) in registers and writes |z|^2.  Gradient (Eq.
+// derivative, App. A): a CTA takes whole rows and loops over the J masks, keeping the accumulated
 // Q^H(z .* r) in registers: forward FFT, residual r = y - |z|^2 and its square
 // sum, inverse FFT of z .* r, multiply by conj(d_j), accumulate; g = -4 * acc.
 #include <cmath>
@@ -111,12 +111,22 @@ static void host_fft(std::vector<std::complex<double>> &x)
     }
 }
 
+// out[b] = exp(-2 pi i b / L), b < n
+static void last_pass_bases(int L, int n, float2 *out)
+{
+    for (int b = 0; b < n; b++) {
+        const double a = -2.0 * M_PI * (double)b / (double)L;
+        out[b] = make_float2((float)std::cos(a), (float)std::sin(a));
+    }
+}
+
 template <int L, int NE>
 static int blue_table(int N, float2 *out)
 {
     using X = XfBlue<L, NE>;
-    const int len = X::NCONST + N;
+    const int len = X::NCONST + N + X::NBASE;
     if (!out) return len;
+    last_pass_bases(L, X::NBASE, out + X::NCONST + N);
     plan_table<typename X::Plan>(out, X::Plan::P - 1);
     // exp(i pi s m^2 / N) with m^2 reduced mod 2N (exact)
     auto chirp = [N](long long m, double s) {
@@ -140,14 +150,15 @@ static int blue_table(int N, float2 *out)
     return len;
 }
 
-// [twiddles | B_1 | B_2 | chirp] of the split-output transform (XfBlueSplit)
+// [twiddles | B_1 | B_2 | chirp | bases] of the split-output transform (XfBlueSplit)
 template <int NE>
 static int blue_split_table(int N, float2 *out)
 {
     using X = XfBlueSplit<NE>;
     constexpr int L = X::L;
-    const int len = X::NCONST + N;
+    const int len = X::NCONST + N + X::NBASE;
     if (!out) return len;
+    last_pass_bases(L, X::NBASE, out + X::NCONST + N);
     std::vector<float2> full(fft_table_len(L));
     fft_table(L, full.data());
     for (int i = 0; i < X::NCONST_TW; i++) out[i] = full[i];
@@ -175,8 +186,32 @@ static int blue_split_table(int N, float2 *out)
     return len;
 }
 
+// XfPow2's table, then XfPow2W's
+template <int N>
+static int pow2_table(float2 *out)
+{
+    using W = XfPow2W<N>;
+    if (out) {
+        fft_table(N, out);
+        plan_table<typename W::Plan>(out + W::TABLE_OFF, W::Plan::P - 1);
+        for (int i = 0; i < 4; i++)
+            for (int t = 0; t < W::NT; t++) {
+                const double a = -2.0 * M_PI * (double)(t << i) / (double)N;
+                out[W::TABLE_OFF + W::NCONST + i * W::NT + t] = make_float2((float)std::cos(a), (float)std::sin(a));
+            }
+    }
+    return W::TABLE_OFF + W::NCONST + 4 * W::NT;
+}
+
 int xform_table(int N, float2 *out)
 {
+    switch (N) {
+    case 512: return pow2_table<512>(out);
+    case 1024: return pow2_table<1024>(out);
+    case 2048: return pow2_table<2048>(out);
+    case 4096: return pow2_table<4096>(out);
+    default: break;
+    }
     if (fft_supported(N)) return fft_table(N, out);
     int L, ne;
     if (!xform_blue_shape(N, &L, &ne)) return -1;
@@ -327,8 +362,9 @@ int xform_table_prec(int N, int prec, float2 *out)
 
 // Calls f(Xf{}) with the transform policy of length N and kind prec (0: FP32
 // with the 1D probing DFT, 1: mixed precision, 2: FP32 with the 2D probing DFT).
+// wide: 16 points per thread for the FP32 powers of two from 512 (XfPow2W).
 template <class F>
-static cudaError_t dispatch_xf(int N, int prec, F &&f)
+static cudaError_t dispatch_xf(int N, int prec, bool wide, F &&f)
 {
     if (prec == 2) {  // the 2D probing DFT
         switch (N) {
@@ -350,11 +386,24 @@ static cudaError_t dispatch_xf(int N, int prec, F &&f)
     case 64: return f(XfPow2<64>{});
     case 128: return f(XfPow2<128>{});
     case 256: return f(XfPow2<256>{});
-    case 512: return f(XfPow2<512>{});
-    case 1024: return f(XfPow2<1024>{});
-    case 2048: return f(XfPow2<2048>{});
-    case 4096: return f(XfPow2<4096>{});
     default: break;
+    }
+    if (wide) {
+        switch (N) {
+        case 512: return f(XfPow2W<512>{});
+        case 1024: return f(XfPow2W<1024>{});
+        case 2048: return f(XfPow2W<2048>{});
+        case 4096: return f(XfPow2W<4096>{});
+        default: break;
+        }
+    } else {
+        switch (N) {
+        case 512: return f(XfPow2<512>{});
+        case 1024: return f(XfPow2<1024>{});
+        case 2048: return f(XfPow2<2048>{});
+        case 4096: return f(XfPow2<4096>{});
+        default: break;
+        }
     }
     int L, ne;
     if (!xform_blue_shape(N, &L, &ne)) return cudaErrorInvalidValue;
@@ -376,8 +425,49 @@ static cudaError_t dispatch_xf(int N, int prec, F &&f)
 // ---------------------------------------------------------------------------
 // Kernels over a transform policy Xf (xform.cuh); shared memory holds the
 // exchange buffer (Xf::LBUF) and the transform's shared constants.
+//
+// Each CTA walks several rows, so that the constants (up to 87 KB for
+// Bluestein, 3.6 KB for N = 4096) and, where the CTA keeps one mask, the mask
+// are fetched once per CTA instead of once per row; and no FP64 sincospi is left
+// in a transform's setup (two FP64 lanes a cycle and SM: it took most of a
+// short row), its bases come from the table.  Bound by shared-memory wavefronts
+// and issue slots of the transforms, not by HBM.  J = 4, one call before ->
+// after: forward N = 4096, M = 16384 1896 -> 628 us (1.7 GB moved: 2.6 TB/s);
+// gradient N = 2048, M = 8192 435 -> 288; forward N = 64, M = 128 5.1 -> 4.6
+// (launch).
+//
+// CTAs per SM aimed at, as threads per SM, swept for the two kernels (forward,
+// gradient): register FFTs of 8 points 1024 and 640 (64 and 96 registers a
+// thread), of 16 points 512 and 384 (128 and 168), the others (Bluestein's 16 points and more, the tensor-core passes) 512.
+// E.g. N = 2048 with 16 points, M = 8192, J = 4: gradient 324 us at 256 threads,
+// 285 at 384, 314 at 512 (spills).
+enum { XK_FORWARD = 0, XK_GRAD = 1 };
 template <class Xf>
-__global__ void __launch_bounds__(Xf::NT) k_forward(int N, const float2 *__restrict__ T,
+__host__ __device__ constexpr int xf_min_ctas(int kernel)
+{
+    const bool grad = kernel == XK_GRAD;
+    const bool mixed = Xf::kN > 0 && Xf::NCONST > Xf::kN;
+    const int t = Xf::kBlue || mixed           ? 512
+                  : Xf::kN >= 512 && Xf::NE == 16 ? (grad ? 384 : 512)
+                                                 : (grad ? 640 : 1024);
+    return t / Xf::NT > 32 ? 32 : (t / Xf::NT > 1 ? t / Xf::NT : 1);
+}
+
+// Starts the fetch of n values at p towards this SM, a line per thread: the
+// next row arrives while this one is transformed, without registers or shared
+// memory to hold it (N = 4096, forward: 633 us with it, 659 without).  Short
+// rows gain nothing (N = 256: 41 against 37).
+template <class Xf, class V>
+__device__ __forceinline__ void prefetch_row(const V *p, int n, int tid)
+{
+    if constexpr (Xf::kN == 0 || Xf::kN >= 512) {
+        constexpr int kLine = 128 / (int)sizeof(V);
+        for (int i = tid * kLine; i < n; i += Xf::NT * kLine) asm volatile("prefetch.global.L1 [%0];" ::"l"(p + i));
+    }
+}
+
+template <class Xf>
+__global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_FORWARD)) k_forward(int N, int M, const float2 *__restrict__ T,
                                                     const float2 *__restrict__ masks,
                                                     const float2 *__restrict__ cg,
                                                     float *__restrict__ Y, int J)
@@ -385,24 +475,27 @@ __global__ void __launch_bounds__(Xf::NT) k_forward(int N, const float2 *__restr
     constexpr int NT = Xf::NT, E = Xf::NE;
     extern __shared__ float2 smem[];
     float2 *buf = smem, *cst = smem + Xf::BUFS * Xf::LBUF;
-    const int tid = threadIdx.x, row = blockIdx.x, j = blockIdx.y;
+    const int tid = threadIdx.x, j = blockIdx.y;
     for (int i = tid; i < Xf::shared_consts(N); i += NT) cst[i] = cg[i];
     Xf xf;
     xf.setup(masks + (size_t)j * N, cg + Xf::NCONST, N, tid);
-    float2 v[E];
-#pragma unroll
-    for (int e = 0; e < E; e++)
-        v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
     __syncthreads();
-    xf.fwd(v, buf, cst, tid);
-    float *yr = Y + ((size_t)row * J + j) * N;
+    for (int row = blockIdx.x; row < M; row += gridDim.x) {
+        float2 v[E];
 #pragma unroll
-    for (int e = 0; e < E; e++)
-        if (Xf::valid(e, tid, N)) yr[tid + e * NT] = cabs2(v[e]);
+        for (int e = 0; e < E; e++)
+            v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+        if (row + (int)gridDim.x < M) prefetch_row<Xf>(T + (size_t)(row + gridDim.x) * N, N, tid);
+        xf.fwd(v, buf, cst, tid);
+        float *yr = Y + ((size_t)row * J + j) * N;
+#pragma unroll
+        for (int e = 0; e < E; e++)
+            if (Xf::valid(e, tid, N)) yr[tid + e * NT] = cabs2(v[e]);
+    }
 }
 
 template <class Xf>
-__global__ void __launch_bounds__(Xf::NT) k_grad(int N, const float2 *__restrict__ T,
+__global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_GRAD)) k_grad(int N, int M, const float2 *__restrict__ T,
                                                  const float2 *__restrict__ masks,
                                                  const float2 *__restrict__ cg,
                                                  const float *__restrict__ Y,
@@ -413,75 +506,102 @@ __global__ void __launch_bounds__(Xf::NT) k_grad(int N, const float2 *__restrict
     extern __shared__ float2 smem[];
     float2 *buf = smem, *cst = smem + Xf::BUFS * Xf::LBUF;
     __shared__ float red[NT / 32 > 0 ? NT / 32 : 1], fsum[1];
-    const int tid = threadIdx.x, row = blockIdx.x;
+    const int tid = threadIdx.x;
     for (int i = tid; i < Xf::shared_consts(N); i += NT) cst[i] = cg[i];
-    float2 t[E], acc[E];
-#pragma unroll
-    for (int e = 0; e < E; e++) {
-        t[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
-        acc[e] = make_float2(0.f, 0.f);
-    }
-    float f = 0.f;
+    Xf xf;
+    xf.setup(masks, cg + Xf::NCONST, N, tid);
     __syncthreads();
-    for (int j = 0; j < J; j++) {
-        Xf xf;
-        xf.setup(masks + (size_t)j * N, cg + Xf::NCONST, N, tid);
-        __syncthreads();  // a fresh policy restarts the exchange-buffer alternation
-        const float *y = Y + ((size_t)row * J + j) * N;
-        float2 v[E];
+    for (int row = blockIdx.x; row < M; row += gridDim.x) {
+        float2 acc[E];
 #pragma unroll
-        for (int e = 0; e < E; e++) v[e] = t[e];
-        xf.fwd(v, buf, cst, tid);
+        for (int e = 0; e < E; e++) acc[e] = make_float2(0.f, 0.f);
+        float f = 0.f;
+        for (int j = 0; j < J; j++) {
+            if (J > 1) xf.load_mask(masks + (size_t)j * N, cst, N, tid);
+            const float *y = Y + ((size_t)row * J + j) * N;
+            float2 v[E];
+            // the row's intensities are in flight during the transform, where
+            // the registers allow (not beside Bluestein's 16 points)
+            float yv[E];
 #pragma unroll
-        for (int e = 0; e < E; e++) {
-            if (cost == COST_AMPLITUDE) {
-                const float c = Xf::valid(e, tid, N) ? cost_coef(cost, v[e], y[tid + e * NT], f) : 0.f;
-                v[e] = cscale(v[e], c);
-            } else {
-                const float r = Xf::valid(e, tid, N) ? y[tid + e * NT] - cabs2(v[e]) : 0.f;
-                f = fmaf(r, r, f);
-                v[e] = cscale(v[e], r);
+            for (int e = 0; e < E; e++) {
+                v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+                if constexpr (!Xf::kBlue) yv[e] = y[tid + e * NT];
             }
+            if (j + 1 < J) {
+                prefetch_row<Xf>(y + N, N, tid);
+            } else if (row + (int)gridDim.x < M) {
+                prefetch_row<Xf>(Y + (size_t)(row + gridDim.x) * J * N, N, tid);
+                prefetch_row<Xf>(T + (size_t)(row + gridDim.x) * N, N, tid);
+            }
+            xf.fwd(v, buf, cst, tid);
+            if constexpr (Xf::kBlue) {
+#pragma unroll
+                for (int e = 0; e < E; e++) yv[e] = Xf::valid(e, tid, N) ? y[tid + e * NT] : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                if (cost == COST_AMPLITUDE) {
+                    const float c = Xf::valid(e, tid, N) ? cost_coef(cost, v[e], yv[e], f) : 0.f;
+                    v[e] = cscale(v[e], c);
+                } else {
+                    const float r = Xf::valid(e, tid, N) ? yv[e] - cabs2(v[e]) : 0.f;
+                    f = fmaf(r, r, f);
+                    v[e] = cscale(v[e], r);
+                }
+            }
+            xf.adj(v, buf, cst, tid);
+#pragma unroll
+            for (int e = 0; e < E; e++) acc[e] = cadd(acc[e], v[e]);
         }
-        xf.adj(v, buf, cst, tid);
+        if (G) {
 #pragma unroll
-        for (int e = 0; e < E; e++) acc[e] = cadd(acc[e], v[e]);
+            for (int e = 0; e < E; e++)
+                if (Xf::valid(e, tid, N)) G[(size_t)row * N + tid + e * NT] = cscale(acc[e], cost_grad_scale(cost));
+        }
+        float fv[1] = {f};
+        block_sum<1>(fv, red, fsum);
+        if (loss && tid == 0) loss[row] = fsum[0];
     }
-    if (G) {
-#pragma unroll
-        for (int e = 0; e < E; e++)
-            if (Xf::valid(e, tid, N)) G[(size_t)row * N + tid + e * NT] = cscale(acc[e], cost_grad_scale(cost));
-    }
-    float fv[1] = {f};
-    block_sum<1>(fv, red, fsum);
-    if (loss && tid == 0) loss[row] = fsum[0];
 }
 
 // Defocus fields: CTA (row, j) computes z_j = F(d_j .* t) and keeps the
-// entries whose pattern index j*N + k is below Nd.
+// entries whose pattern index j*N + k is below Nd.  w (may be NULL): the rows'
+// energies ||t||^2, the fit's weights, from the same read of T.
 template <class Xf>
-__global__ void __launch_bounds__(Xf::NT) k_fields(int N, const float2 *__restrict__ T,
+__global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_FORWARD)) k_fields(int N, const float2 *__restrict__ T,
                                                    const float2 *__restrict__ masks,
                                                    const float2 *__restrict__ cg,
-                                                   float2 *__restrict__ Zd, int M, int Nd)
+                                                   float2 *__restrict__ Zd, int M, int Nd,
+                                                   float *__restrict__ w)
 {
     constexpr int NT = Xf::NT, E = Xf::NE;
     extern __shared__ float2 smem[];
     float2 *buf = smem, *cst = smem + Xf::BUFS * Xf::LBUF;
-    const int tid = threadIdx.x, row = blockIdx.x, j = blockIdx.y;
+    __shared__ float red[NT / 32], esum[1];
+    const int tid = threadIdx.x, j = blockIdx.y;
     for (int i = tid; i < Xf::shared_consts(N); i += NT) cst[i] = cg[i];
     Xf xf;
     xf.setup(masks + (size_t)j * N, cg + Xf::NCONST, N, tid);
-    float2 v[E];
-#pragma unroll
-    for (int e = 0; e < E; e++)
-        v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
     __syncthreads();
-    xf.fwd(v, buf, cst, tid);
+    for (int row = blockIdx.x; row < M; row += gridDim.x) {
+        float2 v[E];
 #pragma unroll
-    for (int e = 0; e < E; e++) {
-        const int pat = j * N + tid + e * NT;
-        if (Xf::valid(e, tid, N) && pat < Nd) Zd[(size_t)pat * M + row] = v[e];
+        for (int e = 0; e < E; e++)
+            v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+        if (w && j == 0) {
+            float en[1] = {0.f};
+#pragma unroll
+            for (int e = 0; e < E; e++) en[0] += cabs2(v[e]);
+            block_sum<1>(en, red, esum);
+            if (tid == 0) w[row] = esum[0];
+        }
+        xf.fwd(v, buf, cst, tid);
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+            const int pat = j * N + tid + e * NT;
+            if (Xf::valid(e, tid, N) && pat < Nd) Zd[(size_t)pat * M + row] = v[e];
+        }
     }
 }
 
@@ -519,15 +639,43 @@ __global__ void k_row_energy(int N, int M, const float2 *__restrict__ T, float *
 template <class Xf>
 static size_t xf_kernel_smem(int N) { return sizeof(float2) * (Xf::BUFS * Xf::LBUF + Xf::shared_consts(N)); }
 
+// (the default limit of 48 KB needs no call, and the smallest problems are all
+// launch latency)
+template <class K>
+static void xf_allow_smem(K kernel, size_t bytes)
+{
+    if (bytes > 47 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// CTAs along the rows when `per` CTAs share a row: about four times what the
+// SMs hold, so that the last wave is short, and no more than there are rows.
+template <class Xf>
+static int xf_row_ctas(int M, int per, int kernel)
+{
+    const int want = (4 * 152 * xf_min_ctas<Xf>(kernel) + per - 1) / per;
+    return want < M ? want : M;
+}
+
+// Whether the transform with 16 points per thread is the faster one: it moves
+// less through shared memory but has half the threads to cover a row's
+// latencies, so the rows (`transforms` of them side by side) have to fill the
+// SMs about four deep, and the gradient, whose short rows leave it few warps,
+// wants N >= 1024 (M = 16384, J = 4: N = 512 74 us against 66; N = 1024, 150
+// rows: 12 us against 8; N = 1024, 16384 rows: 139 us against 163).
+static bool xf_wide(int N, long long transforms, int kernel)
+{
+    return N >= (kernel == XK_GRAD ? 1024 : 512) && transforms >= 608;
+}
+
 cudaError_t launch_forward(int N, int M, int J, const float2 *T, const float2 *masks,
                            const float2 *tw, float *Y, cudaStream_t s, int prec)
 {
     if (M == 0) return cudaSuccess;
-    return dispatch_xf(N, prec, [&](auto xf) {
+    return dispatch_xf(N, prec, xf_wide(N, (long long)M * J, XK_FORWARD), [&](auto xf) {
         using XF = decltype(xf);
         const size_t sm = xf_kernel_smem<XF>(N);
-        cudaFuncSetAttribute(k_forward<XF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_forward<XF><<<dim3(M, J), XF::NT, sm, s>>>(N, T, masks, tw, Y, J);
+        xf_allow_smem(k_forward<XF>, sm);
+        k_forward<XF><<<dim3(xf_row_ctas<XF>(M, J, XK_FORWARD), J), XF::NT, sm, s>>>(N, M, T, masks, tw + TableOff<XF>::value, Y, J);
         return cudaGetLastError();
     });
 }
@@ -537,25 +685,27 @@ cudaError_t launch_grad(int N, int M, int J, const float2 *T, const float2 *mask
                         int prec, int cost)
 {
     if (M == 0) return cudaSuccess;
-    return dispatch_xf(N, prec, [&](auto xf) {
+    return dispatch_xf(N, prec, xf_wide(N, M, XK_GRAD), [&](auto xf) {
         using XF = decltype(xf);
         const size_t sm = xf_kernel_smem<XF>(N);
-        cudaFuncSetAttribute(k_grad<XF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_grad<XF><<<M, XF::NT, sm, s>>>(N, T, masks, tw, Y, loss, G, J, cost);
+        xf_allow_smem(k_grad<XF>, sm);
+        k_grad<XF><<<xf_row_ctas<XF>(M, 1, XK_GRAD), XF::NT, sm, s>>>(N, M, T, masks, tw + TableOff<XF>::value, Y, loss,
+                                                                                       G, J, cost);
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_fields(int N, int M, int J, int Nd, const float2 *T, const float2 *masks,
-                          const float2 *tw, float2 *Zd, cudaStream_t s, int prec)
+                          const float2 *tw, float2 *Zd, float *w, cudaStream_t s, int prec)
 {
     if (M == 0 || Nd == 0) return cudaSuccess;
     const int Jn = (Nd + N - 1) / N < J ? (Nd + N - 1) / N : J;
-    return dispatch_xf(N, prec, [&](auto xf) {
+    return dispatch_xf(N, prec, xf_wide(N, (long long)M * Jn, XK_FORWARD), [&](auto xf) {
         using XF = decltype(xf);
         const size_t sm = xf_kernel_smem<XF>(N);
-        cudaFuncSetAttribute(k_fields<XF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        k_fields<XF><<<dim3(M, Jn), XF::NT, sm, s>>>(N, T, masks, tw, Zd, M, Nd);
+        xf_allow_smem(k_fields<XF>, sm);
+        k_fields<XF><<<dim3(xf_row_ctas<XF>(M, Jn, XK_FORWARD), Jn), XF::NT, sm, s>>>(N, T, masks, tw + TableOff<XF>::value, Zd, M, Nd,
+                                                                                                        w);
         return cudaGetLastError();
     });
 }

@@ -23,8 +23,9 @@
 // Four length-L FFTs per forward/adjoint pair instead of two length-N ones.
 //
 // Constants (host-made in FP64, rounded to FP32), one table per N:
-//   [ FFT twiddles (NCONST_TW) | B half (L/2 + 1) | chirp c (N) ]
-// Every CTA copies the first shared_consts(N) entries (all of it for
+//   [ FFT twiddles (NCONST_TW) | B half (L/2 + 1) | chirp c (N) |
+//     last-pass twiddle bases exp(-2 pi i b / L) (NBASE) ]
+// Every CTA copies the first shared_consts(N) entries (all but the bases for
 // Bluestein, the twiddles of the non-final passes for powers of two) to shared
 // memory; dc is made once per thread in registers.
 #pragma once
@@ -56,15 +57,22 @@ struct XfPow2 {
 
     __device__ __forceinline__ static bool valid(int e, int tid, int n) { return true; }
 
+    // chirp: what follows the small twiddles in the table, here the last pass's
+    // block, whose first NT entries are the bases exp(-2 pi i tid / N).  (Made
+    // in the kernel by an FP64 sincospi they took longer than the transform:
+    // the FP64 pipe serves two lanes per SM and cycle.)
     __device__ __forceinline__ void setup(const float2 *__restrict__ mask, const float2 *__restrict__ chirp,
                                           int n, int tid)
     {
+        load_mask(mask, nullptr, n, tid);
+        wb[0] = chirp[tid];
+        ph = 0;
+    }
+    // another mask for the same policy; cst: the constants in shared memory
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
 #pragma unroll
         for (int e = 0; e < NE; e++) dm[e] = mask[tid + e * NT];
-        double s, c;
-        sincospi(-2.0 * (double)tid / (double)N_, &s, &c);
-        wb[0] = make_float2((float)c, (float)s);
-        ph = 0;
     }
     template <int SIGN>
     __device__ __forceinline__ void fft(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
@@ -85,6 +93,69 @@ struct XfPow2 {
 #pragma unroll
         for (int e = 0; e < NE; e++) x[e] = cmulc(x[e], dm[e]);
     }
+};
+
+// XfPow2W<N>: the same transform with 16 points per thread, N = 512 .. 4096, for
+// the streaming kernels: a first pass of the remaining radix and radix-16
+// passes, two exchanges (one for 512 and less) where XfPow2 has three.  What
+// bounds those kernels is the shared-memory traffic of the exchanges and the
+// instructions around them.  Its constants stand behind XfPow2's in the table:
+// [ twiddles of the middle pass | bases exp(-2 pi i k t / N), t < NT, for k = 1, 2,
+// 4, 8 ].
+template <int N_>
+struct XfPow2W {
+    static constexpr bool kBlue = false;
+    static constexpr int kN = N_;
+    static constexpr int NE = 16;
+    static constexpr int NT = N_ / NE;
+    using Plan = FftPlan<N_, NE>;
+    static constexpr int LBUF = fft_buf_len(N_);
+    static constexpr int BUFS = 2;
+    static constexpr int NCONST = Plan::TW_SMALL;
+    static constexpr int TABLE_OFF = FftPlan<N_, N_ / fft_threads(N_)>::TW_SIZE;
+    __host__ __device__ static constexpr int shared_consts(int n) { return NCONST; }
+
+    float2 dm[NE];
+    float2 wb[4];
+    int ph;
+
+    __device__ __forceinline__ static bool valid(int e, int tid, int n) { return true; }
+
+    __device__ __forceinline__ void setup(const float2 *__restrict__ mask, const float2 *__restrict__ after, int n,
+                                          int tid)
+    {
+        load_mask(mask, nullptr, n, tid);
+#pragma unroll
+        for (int i = 0; i < 4; i++) wb[i] = after[tid + i * NT];
+        ph = 0;
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+#pragma unroll
+        for (int e = 0; e < NE; e++) dm[e] = mask[tid + e * NT];
+    }
+    __device__ __forceinline__ void fwd(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
+    {
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = cmul(x[e], dm[e]);
+        block_fft_pp16<N_, NT, -1>(x, buf, cst, wb, tid, ph);
+    }
+    __device__ __forceinline__ void adj(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
+    {
+        block_fft_pp16<N_, NT, +1>(x, buf, cst, wb, tid, ph);
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = cmulc(x[e], dm[e]);
+    }
+};
+
+// Offset of a policy's constants in the table of its length.
+template <class Xf, class = void>
+struct TableOff {
+    static constexpr int value = 0;
+};
+template <class Xf>
+struct TableOff<Xf, decltype((void)Xf::TABLE_OFF)> {
+    static constexpr int value = Xf::TABLE_OFF;
 };
 
 // XfDenseMV<N>: the probing DFT as an explicit matrix-vector product, the
@@ -184,8 +255,7 @@ struct XfPow2D {
     __device__ __forceinline__ void setup(const float2 *__restrict__ mask, const float2 *__restrict__ chirp,
                                           int n, int tid)
     {
-#pragma unroll
-        for (int e = 0; e < NE; e++) dm[e] = mask[tid + e * NT];
+        load_mask(mask, nullptr, n, tid);
         const int n1 = (int)chirp[0].x, n2 = (int)chirp[0].y;
         // the last pass has stride N / NE >= n1, n2: twiddle base W_{N/B}^{tid div B}
         double s, c;
@@ -194,6 +264,11 @@ struct XfPow2D {
         sincospi(-2.0 * (double)(tid / n2) / (double)(N_ / n2), &s, &c);
         wba[0] = make_float2((float)c, (float)s);
         ph = 0;
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+#pragma unroll
+        for (int e = 0; e < NE; e++) dm[e] = mask[tid + e * NT];
     }
     __device__ __forceinline__ void fwd(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
     {
@@ -234,6 +309,7 @@ struct XfBlue {
     static constexpr int BUFS = 1;
     static constexpr int NCONST_TW = Plan::TW_SMALL;
     static constexpr int NCONST = NCONST_TW + L_ / 2 + 1;
+    static constexpr int NBASE = NT * BPT;  // last-pass twiddle bases
     __host__ __device__ static constexpr int shared_consts(int n) { return NCONST + n; }
 
     float2 dc[NE];
@@ -246,16 +322,20 @@ struct XfBlue {
                                           int n_, int tid)
     {
         n = n_;
+        load_mask_chirp(mask, chirp, tid);
+#pragma unroll
+        for (int i = 0; i < BPT; i++) wb[i] = chirp[n + tid + i * NT];
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+        load_mask_chirp(mask, cst + NCONST, tid);
+    }
+    __device__ __forceinline__ void load_mask_chirp(const float2 *__restrict__ mask, const float2 *chirp, int tid)
+    {
 #pragma unroll
         for (int e = 0; e < NE; e++) {
             const int i = tid + e * NT;
             dc[e] = i < n ? cmul(mask[i], chirp[i]) : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < BPT; i++) {
-            double s, co;
-            sincospi(-2.0 * (double)(tid + i * NT) / (double)L_, &s, &co);
-            wb[i] = make_float2((float)co, (float)s);
         }
     }
     // v <- F_L^{+}(F_L^{-}(v) .* B)
@@ -306,7 +386,7 @@ struct XfBlue {
 // One forward and two inverse length-4096 FFTs per transform (three, against
 // two of length 8192 above), 8 points per thread; the filters are not even,
 // so both are stored whole.
-// Constants: [ FFT twiddles | B_1 (L) | B_2 (L) | chirp c (N) ].
+// Constants: [ FFT twiddles | B_1 (L) | B_2 (L) | chirp c (N) | last-pass bases (NBASE) ].
 constexpr int kBlueSplitMaxN = 2731;  // N + ceil(N / 2) - 1 <= 4096
 
 template <int NE_>
@@ -321,6 +401,7 @@ struct XfBlueSplit {
     static constexpr int BUFS = 1;
     static constexpr int NCONST_TW = FftSmall<L, NT>::TW_SMALL;
     static constexpr int NCONST = NCONST_TW + 2 * L;
+    static constexpr int NBASE = NT;  // last-pass twiddle bases
     __host__ __device__ static constexpr int shared_consts(int n) { return NCONST + n; }
 
     float2 dc[NE];
@@ -334,14 +415,20 @@ struct XfBlueSplit {
     {
         n = n_;
         h = (n_ + 1) / 2;
+        load_mask_chirp(mask, chirp, tid);
+        wb = chirp[n + tid];
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+        load_mask_chirp(mask, cst + NCONST, tid);
+    }
+    __device__ __forceinline__ void load_mask_chirp(const float2 *__restrict__ mask, const float2 *chirp, int tid)
+    {
 #pragma unroll
         for (int e = 0; e < NE; e++) {
             const int i = tid + e * NT;
             dc[e] = i < n ? cmul(mask[i], chirp[i]) : make_float2(0.f, 0.f);
         }
-        double s, co;
-        sincospi(-2.0 * (double)tid / (double)L, &s, &co);
-        wb = make_float2((float)co, (float)s);
     }
     // out[e] (index k = tid + e NT < n) <- (c .* conv_h(a))_k, a given in v
     __device__ __forceinline__ void conv2(float2 (&v)[EL], float2 (&out)[NE], float2 *buf, const float2 *cst,
@@ -477,8 +564,12 @@ struct XfMixed {
     __device__ __forceinline__ void setup(const float2 *__restrict__ mask, const float2 *__restrict__ chirp,
                                           int n, int tid)
     {
-        f32.setup(mask, chirp, n, tid);
+        f32.setup(mask, chirp - N_, n, tid);  // the bases are the first of the roots W_N^k before it
         tc = true;
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+        f32.load_mask(mask, cst, n, tid);
     }
 
     // one radix-16 pass: 8-butterfly groups, lane (g, t) loads inputs
