@@ -76,19 +76,20 @@ constexpr int kIdxSS = 4 * kSlots, kIdxGG = 4 * kSlots + 1, kIdxF = 4 * kSlots +
 // them from identical sums added in the same order, so they agree bit for bit
 // and every CTA takes the same branches.  FP32 like the rest of the path (the
 // FP64 pipe of this part is a small fraction of its FP32 rate, and these
-// scalars sit on the critical path of every iteration).  Pairs are indexed by
-// age (0 = oldest); slot[] maps an age to its physical vector slot, and
-// slot[np] is the free slot that receives the next pair.
-struct Gram {
-    float SY[kSlots][kSlots];  // s_i^T y_j, ages i <= j
-    float YY[kSlots][kSlots];  // y_i^T y_j, ages i <= j
-    float rD[kSlots];          // 1 / s_i^T y_i
-    float Sg[kSlots], Yg[kSlots];
-    float c1[kSlots], c2[kSlots];  // direction coefficients by age (c2 includes gamma)
+// scalars sit on the critical path of every iteration).  Pairs have an age
+// (0 = oldest); slot[] maps an age to the physical slot of its vectors and of
+// its rows and columns of the Gram matrices (so that dropping the oldest pair
+// moves nothing), and slot[np] is the free slot that receives the next pair.
+constexpr int kGramPitch = 8;  // kSlots rounded up: rows and coefficient vectors are 16-byte aligned
+struct __align__(16) Gram {
+    float SY[kSlots][kGramPitch];  // s_i^T y_j at [slot of i][slot of j], i no younger than j
+    float YY[kSlots][kGramPitch];  // y_i^T y_j
+    float rD[kGramPitch];          // 1 / s_i^T y_i by slot
+    float c1[kGramPitch], c2[kGramPitch];  // direction coefficients by age (c2 includes gamma)
+    float red[kParts];  // the last cluster-wide sums
+    int slot[kGramPitch];
     float gamma, gg, f, sumy, alpha;
     float yscale, tsc;  // the row's intensity scale 4^-j and its t scale 2^j
-    float red[kParts];  // the last cluster-wide sums
-    int slot[kSlots];
     int np;
     int status, done, stop, early, row;
 };
@@ -192,70 +193,78 @@ static __device__ float quartic_argmin_safe(const float *c)
     return best;
 }
 
-// The same minimiser from the closed-form roots of the cubic phi'(a) = 0
-// (Cardano's formula for one real root, the trigonometric form for three),
-// each polished by Newton steps on phi' in FP32, the up to three polishings on
-// lanes 0..2 of a warp (every lane of the warp calls it and gets the same
-// result); among the real roots the one with the smallest phi wins (ties: the
-// smallest positive root).  The roots are found for the variable b = 2^-k a,
-// with k such that 2^(4k) c4 lies in [1/2, 8): an exact power-of-two
-// substitution that keeps the coefficients near 1 when the step's fields are
-// tiny (late iterations), where 1 / c4 and the cubic's coefficients would
-// leave FP32 range.  Falls back to the bracketing search when c4 <= 0 or a
-// root comes out non-finite.
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The same minimiser from the roots of the cubic phi'(a) = 0: closed-form
+// starting values (Cardano's formula for one real root, the trigonometric
+// form for three) from the approximate hardware functions, each polished by
+// Newton steps on phi' in FP32, which set the result's accuracy; the three
+// polishings run on lanes 0..2 of a warp (every lane of the warp calls it and
+// gets the same result; with one real root every lane does the same work and
+// nothing is exchanged).  Among the real roots the one with the smallest phi
+// wins (ties: the smallest positive root).  The roots are found for the
+// variable b = 2^-k a, with k such that 2^(4k) c4 lies in [1/2, 8): an exact
+// power-of-two substitution that keeps the coefficients near 1 when the
+// step's fields are tiny (late iterations), where 1 / c4 and the cubic's
+// coefficients would leave FP32 range.  Falls back to the bracketing search
+// when c4 <= 0 or a root comes out non-finite.
+//
+// One warp runs this between two block barriers of every iteration, so its
+// latency is all that counts, hence no IEEE divisions, cbrtf, acosf or ldexpf in
+// the chain.  With the bookkeeping below also in registers: 20 iterations of
+// 4096 rows at N = 4096, J = 4, one mask per CTA, 33.1 -> 29.0 ms.
 static __device__ float quartic_argmin_warp(const float *c, int lane)
 {
     if (!(c[4] > 0.f)) return quartic_argmin_safe(c);
-    int e;
-    frexpf(c[4], &e);  // c4 = f 2^e, f in [1/2, 1)
-    const int ks = -(e >> 2);  // -floor(e / 4)
-    const float c1 = ldexpf(c[1], ks), c2 = ldexpf(c[2], 2 * ks), c3 = ldexpf(c[3], 3 * ks),
-                c4 = ldexpf(c[4], 4 * ks);
-    auto g = [&](float a) { return fmaf(fmaf(fmaf(4.f * c4, a, 3.f * c3), a, 2.f * c2), a, c1); };
-    auto dg = [&](float a) { return fmaf(fmaf(12.f * c4, a, 6.f * c3), a, 2.f * c2); };
+    // c4 = f 2^e, f in [1/2, 1) (a denormal counts as 2^-126)
+    const int e = (__float_as_int(c[4]) >> 23) - 126;
+    const int ks = -(e >> 2);  // -floor(e / 4), in -32 .. 32
+    const float sc = __int_as_float((127 + ks) << 23);
+    const float c1 = c[1] * sc, c2 = c[2] * sc * sc, c3 = c[3] * sc * sc * sc, c4 = c[4] * sc * sc * sc * sc;
+    const float g3 = 4.f * c4, g2 = 3.f * c3, g1 = 2.f * c2;  // g = phi'
+    const float d2 = 12.f * c4, d1 = 6.f * c3;                // g' = (d2 a + d1) a + g1
     auto phi = [&](float a) { return a * fmaf(fmaf(fmaf(c4, a, c3), a, c2), a, c1); };
-    const float inv = 1.f / c4;
+    const float inv = __fdividef(1.f, c4);
     const float B3 = 0.25f * c3 * inv;
     const float C = 0.5f * c2 * inv, D = 0.25f * c1 * inv;
     const float p = fmaf(-3.f * B3, B3, C);
     const float q = fmaf(B3, fmaf(2.f * B3, B3, -C), D);
     const float hp = p * (1.f / 3.f), hq = 0.5f * q;
     const float disc = fmaf(hq, hq, hp * hp * hp);
-    float a = 0.f;
-    int nc;
-    if (disc > 0.f) {
-        nc = 1;
-        if (lane == 0) {
-            const float u = cbrtf(-hq - copysignf(sqrtf(disc), hq));
-            a = (u != 0.f ? u - hp / u : 0.f) - B3;
-        }
+    const bool one = disc > 0.f;
+    float a;
+    if (one) {
+        const float x = -hq - copysignf(sqrt_approx(disc), hq);
+        const float u = copysignf(exp2f(__log2f(fabsf(x)) * (1.f / 3.f)), x);  // cube root; 0 for x = 0
+        a = (u != 0.f ? u - __fdividef(hp, u) : 0.f) - B3;
     } else {
-        nc = 3;
-        if (lane < 3) {
-            const float r = sqrtf(fmaxf(-hp, 0.f));
-            const float r3 = r * r * r;
-            const float arg = r3 > 0.f ? fminf(fmaxf(-hq / r3, -1.f), 1.f) : 0.f;
-            const float th = acosf(arg) * (1.f / 3.f);
-            const float tr = 2.0943951023931955f;  // 2 pi / 3
-            a = 2.f * r * cosf(lane == 0 ? th : (lane == 1 ? th - tr : th + tr)) - B3;
-        }
+        const float r = sqrt_approx(fmaxf(-hp, 0.f));
+        const float r3 = r * r * r;
+        const float arg = r3 > 0.f ? fminf(fmaxf(__fdividef(-hq, r3), -1.f), 1.f) : 0.f;
+        const float th = acosf(arg) * (1.f / 3.f);
+        const float tr = 2.0943951023931955f;  // 2 pi / 3
+        a = 2.f * r * __cosf(lane == 0 ? th : (lane == 1 ? th - tr : th + tr)) - B3;
     }
-    if (lane < nc) {
-        for (int it = 0; it < 4; it++) {
-            const float d = dg(a);
-            if (!(d != 0.f)) break;
-            const float na = a - g(a) / d;
-            if (!isfinite(na) || na == a) break;
-            a = na;
-        }
-    }
-    const float v = phi(a);
-    float best = 0.f, bestv = 0.f;
-    bool bad = false;
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const float ak = __shfl_sync(0xffffffffu, a, k), vk = __shfl_sync(0xffffffffu, v, k);
-        if (k < nc) {
+    for (int it = 0; it < 4; it++) {
+        const float d = fmaf(fmaf(d2, a, d1), a, g1);
+        const float na = a - __fdividef(fmaf(fmaf(fmaf(g3, a, g2), a, g1), a, c1), d);
+        a = isfinite(na) ? na : a;  // d = 0: keep the point
+    }
+    float best = a;
+    bool bad = !isfinite(a);
+    if (!one) {
+        const float v = phi(a);
+        float bestv = 0.f;
+        bad = false;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const float ak = __shfl_sync(0xffffffffu, a, k), vk = __shfl_sync(0xffffffffu, v, k);
             bad = bad || !isfinite(ak);
             if (k == 0 || vk < bestv || (vk == bestv && ak > 0.f && (best <= 0.f || ak < best))) {
                 best = ak;
@@ -264,16 +273,9 @@ static __device__ float quartic_argmin_warp(const float *c, int lane)
         }
     }
     if (bad) return quartic_argmin_safe(c);
-    return ldexpf(best, ks);
+    return best * sc;
 }
 
-// Compact-form coefficients, run by one warp (lane i owns age i):
-// p = -(gamma g + sum_i c1_i s_i + sum_i c2_i y_i), c2 already scaled by gamma.
-// R c2 = -S^T g is solved by back substitution and R^T c1 =
-// -(D + gamma Y^T Y) c2 - gamma Y^T g by forward substitution, each step
-// broadcasting the new unknown with a shuffle.  Falls back to p = -g (and
-// clears the history) when there is no pair or the result is not a descent
-// direction.
 // Exponent j of a row's intensity scale: with the mean intensity ybar in
 // [2^(e-1), 2^e), j = floor(e / 2), so y 4^-j has a mean in [1/2, 2), rows
 // whose mean is already there keep j = 0, and scaling y by 4^k moves j by
@@ -287,116 +289,150 @@ static __device__ __forceinline__ int row_scale_exp(float sumy, int K)
     return e >> 1;  // floor(e / 2) for either sign
 }
 
-static __device__ void lbfgs_coefficients_warp(Gram &G, int lane)
+// The state before the first pair: p = -g.  One warp.
+static __device__ __forceinline__ void lbfgs_reset(Gram &G, int lane)
 {
-    const int np = G.np;
-    float c1 = 0.f, c2 = 0.f, gamma = 1.f;
-    bool ok = false;
-    if (np > 0) {
-        gamma = G.SY[np - 1][np - 1] / G.YY[np - 1][np - 1];
-        const bool mine = lane < np;
-        float acc = mine ? -G.Sg[lane] : 0.f;
-        for (int j = np - 1; j >= 0; j--) {
-            if (lane == j) c2 = acc * G.rD[j];
-            const float cj = __shfl_sync(0xffffffffu, c2, j);
-            if (lane < j) acc = fmaf(-G.SY[lane][j], cj, acc);
-        }
-        float yc = 0.f;
-        for (int j = 0; j < np; j++) {
-            const float cj = __shfl_sync(0xffffffffu, c2, j);
-            if (mine) yc = fmaf(G.YY[lane < j ? lane : j][lane < j ? j : lane], cj, yc);
-        }
-        float acc1 = mine ? -G.SY[lane][lane] * c2 - gamma * (G.Yg[lane] + yc) : 0.f;
-        for (int j = 0; j < np; j++) {
-            if (lane == j) c1 = acc1 * G.rD[j];
-            const float cj = __shfl_sync(0xffffffffu, c1, j);
-            if (mine && lane > j) acc1 = fmaf(-G.SY[j][lane], cj, acc1);
-        }
-        float t = mine ? fmaf(c1, G.Sg[lane], gamma * c2 * G.Yg[lane]) : 0.f;
-        const float pg = gamma * G.gg + warp_sum(t);  // <g, H g> = -<p, g>
-        ok = pg > 0.f && isfinite(pg);
-    }
-    __syncwarp();
-    if (lane < kSlots) {
-        G.c1[lane] = (ok && lane < np) ? c1 : 0.f;
-        G.c2[lane] = (ok && lane < np) ? gamma * c2 : 0.f;
+    if (lane < kGramPitch) {
+        G.c1[lane] = G.c2[lane] = 0.f;
+        G.slot[lane] = lane;
     }
     if (lane == 0) {
-        G.gamma = ok ? gamma : 1.f;
-        if (!ok) G.np = 0;
+        G.np = 0;
+        G.gamma = 1.f;
     }
     __syncwarp();
 }
 
-// Gram bookkeeping after the batched dot products of an iteration, run by one
-// warp (lane i owns age i): the new column of S^T Y and Y^T Y and the new
-// S^T g, Y^T g from Gm.red, the pair test s^T y > 1e-10 |s| |y|, the shift
-// that drops the oldest pair once m are held (its slot becomes the free one),
-// the loss and the stopping tests, then the next direction's coefficients.
+// The L-BFGS bookkeeping after the batched dot products of an iteration, run
+// by one warp: the new column of S^T Y and Y^T Y from Gm.red, the pair test
+// s^T y > 1e-10 |s| |y|, dropping the oldest pair once m are held (its slot
+// becomes the free one), the loss and the stopping tests, then the next
+// direction's compact-form coefficients: p = -(gamma g + sum_i c1_i s_i +
+// sum_i c2_i y_i), c2 already scaled by gamma.  R c2 = -S^T g is solved by back
+// substitution and R^T c1 = -(D + gamma Y^T Y) c2 - gamma Y^T g by forward
+// substitution.  Falls back to p = -g (and clears the history) when there is
+// no pair or the result is not a descent direction.
+//
+// The other warps wait for this, so only its latency counts.  Every lane does
+// the whole algebra (at most 6 x 6) in registers: the substitutions are then
+// chains of one multiplication and one FMA a step, where a lane per unknown
+// needed a shuffle and two shared-memory reads a step,
+// and the Gram matrices stay where they are when a pair is dropped.
 static __device__ void lbfgs_gram_update(Gram &Gm, int lane, int m, int it, int iters, double tol)
 {
-    const int np = Gm.np;
     const float *tot = Gm.red;
+    const int np = Gm.np;
+    int sl[kSlots + 1];  // slots by age; afterwards by age without a dropped pair
+    {
+        const int4 a = reinterpret_cast<const int4 *>(Gm.slot)[0], b = reinterpret_cast<const int4 *>(Gm.slot)[1];
+        sl[0] = a.x, sl[1] = a.y, sl[2] = a.z, sl[3] = a.w, sl[4] = b.x, sl[5] = b.y, sl[6] = b.z, sl[7] = 0;
+    }
+    const int ns = Gm.slot[np];
     if (lane <= np) {
-        Gm.SY[lane][np] = tot[4 * lane + 0];
-        Gm.YY[lane][np] = tot[4 * lane + 1];
-        Gm.Sg[lane] = tot[4 * lane + 2];
-        Gm.Yg[lane] = tot[4 * lane + 3];
+        const int si = Gm.slot[lane];
+        Gm.SY[si][ns] = tot[4 * lane + 0];
+        Gm.YY[si][ns] = tot[4 * lane + 1];
     }
     const float sy = tot[4 * np + 0], yy = tot[4 * np + 1];
-    const float fnew = tot[kIdxF];
+    const float fnew = tot[kIdxF], gg = tot[kIdxGG], fold = Gm.f;
     const bool accept = sy > 1e-10f * sqrtf(tot[kIdxSS]) * sqrtf(yy) && sy > 0.f;
-    int np2 = np + (accept ? 1 : 0);
-    __syncwarp();
-    if (accept && lane == 0) Gm.rD[np] = 1.f / sy;
-    __syncwarp();
-    if (np2 > m) {
-        // drop the oldest pair: age i + 1 becomes age i
-        float sy_r[kSlots], yy_r[kSlots], sg = 0.f, yg = 0.f, rd = 0.f;
-        int sl = 0;
-        const bool mine = lane < np2 - 1;
-        const int src = lane + 1;
+    const bool drop = accept && np + 1 > m;
+    const int np2 = np + (accept ? 1 : 0) - (drop ? 1 : 0);
+    if (accept && lane == 0) Gm.rD[ns] = 1.f / sy;
+    if (drop) {
+        const int s0 = sl[0];
 #pragma unroll
-        for (int j = 0; j < kSlots; j++) {
-            sy_r[j] = (mine && j + 1 < kSlots) ? Gm.SY[src][j + 1 < kSlots ? j + 1 : 0] : 0.f;
-            yy_r[j] = (mine && j + 1 < kSlots) ? Gm.YY[src][j + 1 < kSlots ? j + 1 : 0] : 0.f;
-        }
-        if (mine) {
-            sg = Gm.Sg[src];
-            yg = Gm.Yg[src];
-            rd = Gm.rD[src];
-        }
-        // the m + 1 allocated slots rotate: the oldest pair's slot
-        // becomes the free one at position m
-        const int sl_old0 = Gm.slot[0];
-        if (lane < m) sl = Gm.slot[lane + 1];
-        __syncwarp();
-        if (mine) {
-#pragma unroll
-            for (int j = 0; j < kSlots; j++) {
-                Gm.SY[lane][j] = sy_r[j];
-                Gm.YY[lane][j] = yy_r[j];
-            }
-            Gm.Sg[lane] = sg;
-            Gm.Yg[lane] = yg;
-            Gm.rD[lane] = rd;
-        }
-        if (lane < m) Gm.slot[lane] = sl;
-        if (lane == m) Gm.slot[lane] = sl_old0;
-        np2 = m;
+        for (int i = 0; i < kSlots; i++) sl[i] = i < m ? sl[i + 1] : s0;  // the m + 1 slots in use rotate
+        if (lane < kSlots && lane <= m) Gm.slot[lane] = lane < m ? Gm.slot[lane + 1] : s0;
     }
+    // status, when a row stops here: numeric trouble before convergence
+    const float rel = fabsf(fold - fnew) / fmaxf(fold, 1e-30f);
+    const bool numeric = !isfinite(fnew) || !isfinite(gg);
+    const bool conv = (tol > 0.0 && rel < (float)tol) || (it + 1 < iters && (fnew == 0.f || gg == 0.f));
+    __syncwarp();
     if (lane == 0) {
         Gm.np = np2;
-        Gm.gg = tot[kIdxGG];
-        const float rel = fabsf(Gm.f - fnew) / fmaxf(Gm.f, 1e-30f);
+        Gm.gg = gg;
         Gm.f = fnew;
         Gm.done = it + 1;
-        if (!isfinite(fnew) || !isfinite(Gm.gg)) { Gm.status = ROW_NUMERIC; Gm.stop = 1; }
-        else if (tol > 0.0 && rel < (float)tol) { Gm.status = ROW_CONVERGED; Gm.stop = 1; }
-        else if (it + 1 < iters && (fnew == 0.f || Gm.gg == 0.f)) { Gm.status = ROW_CONVERGED; Gm.stop = 1; }
+        if (numeric || conv) {
+            Gm.status = numeric ? ROW_NUMERIC : ROW_CONVERGED;
+            Gm.stop = 1;
+        }
+    }
+    if (numeric || conv || it + 1 >= iters) {
+        __syncwarp();
+        return;
+    }
+
+    // ---- coefficients ----
+    float c1[kMaxMem], c2[kMaxMem], gamma = 1.f;
+    bool ok = false;
+    if (np2 > 0) {
+        const int off = drop ? 1 : 0;
+        const int sn = Gm.slot[np2 - 1];  // the youngest pair
+        // three phases, each loading what it needs (a __syncwarp keeps the
+        // compiler from holding both matrices in registers at once)
+        float acc[kMaxMem], rd[kMaxMem], SY[kMaxMem][kMaxMem];
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) {
+            const bool in = i < np2;
+            acc[i] = in ? -tot[4 * (i + off) + 2] : 0.f;
+            rd[i] = in ? Gm.rD[sl[i]] : 0.f;
+#pragma unroll
+            for (int j = i; j < kMaxMem; j++) SY[i][j] = j < np2 ? Gm.SY[sl[i]][sl[j]] : 0.f;
+        }
+        gamma = Gm.SY[sn][sn] / Gm.YY[sn][sn];
+#pragma unroll
+        for (int j = kMaxMem - 1; j >= 0; j--) {
+            c2[j] = acc[j] * rd[j];  // 0 for j >= np2
+#pragma unroll
+            for (int i = 0; i < j; i++) acc[i] = fmaf(-SY[i][j], c2[j], acc[i]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) acc[i] = 0.f;  // Y^T Y c2, each sum in ascending order
+#pragma unroll
+        for (int j = 0; j < kMaxMem; j++) {
+#pragma unroll
+            for (int i = 0; i < kMaxMem; i++) {
+                const float v = (i < np2 && j < np2) ? Gm.YY[i < j ? sl[i] : sl[j]][i < j ? sl[j] : sl[i]] : 0.f;
+                acc[i] = fmaf(v, c2[j], acc[i]);
+            }
+        }
+        __syncwarp();
+        float t[kMaxMem], Yg[kMaxMem];
+#pragma unroll
+        for (int i = 0; i < kMaxMem; i++) {
+            Yg[i] = i < np2 ? tot[4 * (i + off) + 3] : 0.f;
+            acc[i] = -SY[i][i] * c2[i] - gamma * (Yg[i] + acc[i]);
+        }
+#pragma unroll
+        for (int j = 0; j < kMaxMem; j++) {
+            c1[j] = acc[j] * rd[j];
+#pragma unroll
+            for (int i = j + 1; i < kMaxMem; i++) acc[i] = fmaf(-SY[j][i], c1[j], acc[i]);
+            t[j] = fmaf(c1[j], j < np2 ? tot[4 * (j + off) + 2] : 0.f, gamma * c2[j] * Yg[j]);
+        }
+        const float pg = gamma * gg + (((t[0] + t[4]) + t[2]) + ((t[1] + t[5]) + t[3]));  // <g, H g> = -<p, g>
+        ok = pg > 0.f && isfinite(pg);
+    }
+    if (lane == 0) {
+        float4 *o1 = reinterpret_cast<float4 *>(Gm.c1), *o2 = reinterpret_cast<float4 *>(Gm.c2);
+        if (ok) {
+            o1[0] = make_float4(c1[0], c1[1], c1[2], c1[3]);
+            o1[1] = make_float4(c1[4], c1[5], 0.f, 0.f);
+            o2[0] = make_float4(gamma * c2[0], gamma * c2[1], gamma * c2[2], gamma * c2[3]);
+            o2[1] = make_float4(gamma * c2[4], gamma * c2[5], 0.f, 0.f);
+            Gm.gamma = gamma;
+        } else {
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            o1[0] = o1[1] = o2[0] = o2[1] = zero;
+            Gm.gamma = 1.f;
+            Gm.np = 0;
+        }
     }
     __syncwarp();
-    if (!Gm.stop && it + 1 < iters) lbfgs_coefficients_warp(Gm, lane);
 }
 
 // Sum of up to 32 values over a warp by recursive halving: after the call,
@@ -516,14 +552,19 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
         for (int e = 0; e < E; e++) x[e] = valid(e) ? X[ttid + e * NT] : make_float2(0.f, 0.f);
     };
     const int sl_shift = (even && (SL & (SL - 1)) == 0) ? __ffs(SL) - 1 : -1;
+    // the CTA that owns element n; for uneven slices by counting the slice
+    // starts at or below n (a 64-bit division here cost more than the
+    // exchange itself: 4000 cycles an iteration at N = 2286)
+    __shared__ int slice0[kMaxMasks];  // first element of each CTA's slice
     auto owner = [&](int n) {
         if (sl_shift >= 0) return n >> sl_shift;
-        if (even) return n / SL;
-        int o = (int)(((long long)n * JC) / N);
-        while (o + 1 < JC && ((o + 1) * N) / JC <= n) o++;
-        while (o > 0 && (o * N) / JC > n) o--;
+        int o = 0;
+#pragma unroll
+        for (int r = 1; r < kMaxMasks; r++) o += r < JC && n >= slice0[r];
         return o;
     };
+    if (tid < JC) slice0[tid] = (tid * N) / JC;
+    __syncthreads();
     cluster.sync();  // every CTA of the cluster runs before anyone touches its shared memory
 
     // Cluster-wide sums of nv <= 32 per-thread values (v padded with zeros):
@@ -562,7 +603,9 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
         cluster.sync();
         if (tid < nv) {
             float acc = 0.f;
-            for (int o = 0; o < JC; o++) acc += pb[o * kParts + tid];
+#pragma unroll
+            for (int o = 0; o < kMaxMasks; o++)  // the loads are in flight together
+                if (o < JC) acc += pb[o * kParts + tid];
             Gm.red[tid] = acc;
         }
         __syncthreads();
@@ -581,13 +624,15 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
             if (!valid(e)) continue;
             const int n = ttid + e * NT;
             const int o = owner(n);
-            cluster.map_shared_rank(Yr, o)[(size_t)jm * SL + (n - (o * N) / JC)] = v[e];
+            cluster.map_shared_rank(Yr, o)[jm * SL + (n - slice0[o])] = v[e];
         }
     };
     // element i of my slice of sum_j Y[j], times s
     auto slice_sum = [&](int i, float s) {
         float2 acc = Yr[i];
-        for (int o = 1; o < J; o++) acc = cadd(acc, Yr[(size_t)o * SL + i]);
+#pragma unroll
+        for (int o = 1; o < kMaxMasks; o++)
+            if (o < J) acc = cadd(acc, Yr[o * SL + i]);
         return cscale(acc, s);
     };
 
@@ -822,9 +867,7 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
                         if (!isfinite(Gm.f) || !isfinite(Gm.gg)) { Gm.status = ROW_NUMERIC; Gm.stop = 1; }
                         else if (P.iters > 0 && (Gm.f == 0.f || Gm.gg == 0.f)) { Gm.status = ROW_CONVERGED; Gm.stop = 1; }
                     }
-                    if (lane < kSlots) Gm.slot[lane] = lane;
-                    __syncwarp();
-                    if (!Gm.stop) lbfgs_coefficients_warp(Gm, lane);
+                    lbfgs_reset(Gm, lane);
                 }
                 __syncthreads();
             };

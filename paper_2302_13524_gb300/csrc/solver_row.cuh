@@ -191,7 +191,9 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
     // sum over the masks of the parked results, element i, times s
     auto team_sum = [&](int i, float s) {
         float2 acc = bufs[i];
-        for (int j = 1; j < J; j++) acc = cadd(acc, bufs[(size_t)j * LBUF + i]);
+#pragma unroll
+        for (int j = 1; j < kMaxMasks; j++)
+            if (j < J) acc = cadd(acc, bufs[j * LBUF + i]);
         return cscale(acc, s);
     };
     auto load_team = [&](const float2 *src, float2 (&x)[E]) {
@@ -219,7 +221,9 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
         __syncthreads();
         if (tid < nv) {
             float acc = 0.f;
-            for (int w = 0; w < NW; w++) acc += red[tid * NW + w];
+#pragma unroll
+            for (int w = 0; w < 16; w++)  // at most 16 warps: the loads are in flight together
+                if (w < NW) acc += red[tid * NW + w];
             Gm.red[tid] = acc;
         }
         if (all) __syncthreads();
@@ -419,9 +423,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                         if (!isfinite(Gm.f) || !isfinite(Gm.gg)) { Gm.status = ROW_NUMERIC; Gm.stop = 1; }
                         else if (P.iters > 0 && (Gm.f == 0.f || Gm.gg == 0.f)) { Gm.status = ROW_CONVERGED; Gm.stop = 1; }
                     }
-                    if (lane < kSlots) Gm.slot[lane] = lane;
-                    __syncwarp();
-                    if (!Gm.stop) lbfgs_coefficients_warp(Gm, lane);
+                    lbfgs_reset(Gm, lane);
                 }
                 __syncthreads();
             }
