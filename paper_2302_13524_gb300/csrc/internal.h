@@ -37,6 +37,7 @@ bool xform_supported(int N);
 // thread (the instantiated variant); false when N has none.
 bool xform_blue_shape(int N, int *L, int *ne);
 int xform_table(int N, float2 *out);  // length in float2; writes when out != NULL
+bool xform_comp(int N);  // lengths the composite transform takes (XfComp) in place of plain Bluestein
 // For 2048 < N <= 2731 the other Bluestein plan: the full convolution at
 // L = 8192 (XfBlue<8192, 6>) instead of the split outputs at L = 4096; the
 // table of the solver schedule kBlueFullSchedule.
@@ -135,6 +136,10 @@ int solver_row_max_ctas(int N, int J, int m);
 size_t solver_row_pair_stride(int N, int m);  // float2 per CTA region
 size_t solver_smem_bytes(int N, int J, int m, int G, int prec = 0);
 cudaError_t launch_solver(int N, int G, const SolverParams &p, cudaStream_t s, int *clusters_out);
+// the composite lengths (solver_comp.cu, solver_comp_amp.cu)
+size_t solver_comp_smem(int N, int J, int m);
+cudaError_t launch_solver_comp(int N, const SolverParams &p, cudaStream_t s, int *clusters_out);
+cudaError_t launch_solver_comp_amp(int N, const SolverParams &p, cudaStream_t s, int *clusters_out);
 // the Bluestein variants (solver_bs.cu); what == 0: shared bytes, 1: launch
 long long solver_dispatch_blue(int N, int G, int what, const SolverParams *p, cudaStream_t s, int *clusters_out);
 // the one-CTA-per-row variants (solver_row.cu)

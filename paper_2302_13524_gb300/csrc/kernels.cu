@@ -186,6 +186,43 @@ static int blue_split_table(int N, float2 *out)
     return len;
 }
 
+// The table of the composite-length transform (XfComp).
+static int comp_table(int N, float2 *out)
+{
+    using X = XfComp<4>;  // the layout does not depend on the team count
+    const int len = X::NCONST + N + 1;
+    if (!out) return len;
+    int A = 0, B = 0;
+    if (!comp_shape(N, &A, &B)) return -1;
+    auto root = [](long long num, long long den) {  // exp(-2 pi i num / den)
+        const double a = -2.0 * M_PI * (double)(num % den) / (double)den;
+        return std::complex<double>(std::cos(a), std::sin(a));
+    };
+    auto f2 = [](std::complex<double> v) { return make_float2((float)v.real(), (float)v.imag()); };
+    for (int r = 1; r < 16; r++)
+        for (int j = 0; j < 16; j++) out[(r - 1) * 16 + j] = f2(root(r * j, 256));
+    std::vector<std::complex<double>> b(X::L, 0.0);
+    for (int m = 0; m < B; m++) {
+        b[m] = std::conj(root((long long)m * m, 2LL * B));
+        if (m > 0) b[X::L - m] = b[m];
+    }
+    host_fft(b);
+    for (int k = 0; k < X::L; k++) out[X::OFF_FILT + k] = f2(b[k] / (double)X::L);
+    for (int n = 0; n < kCompB; n++) out[X::OFF_CHIRP + n] = n < B ? f2(root((long long)n * n, 2LL * B)) : make_float2(0.f, 0.f);
+    for (int m = 0; m < kCompA; m++) out[X::OFF_WA + m] = m < A ? f2(root(m, A)) : make_float2(0.f, 0.f);
+    for (int k1 = 0; k1 < A; k1++)
+        for (int n2 = 0; n2 < B; n2++)
+            out[X::NCONST + k1 * B + n2] = f2(root((long long)n2 * k1, N) * root((long long)n2 * n2, 2LL * B));
+    out[X::NCONST + N] = make_float2((float)A, (float)B);
+    return len;
+}
+
+bool xform_comp(int N)
+{
+    int A = 0, B = 0;
+    return N >= 16 && N <= 4096 && !fft_supported(N) && comp_shape(N, &A, &B);
+}
+
 // XfPow2's table, then XfPow2W's
 template <int N>
 static int pow2_table(float2 *out)
@@ -213,6 +250,7 @@ int xform_table(int N, float2 *out)
     default: break;
     }
     if (fft_supported(N)) return fft_table(N, out);
+    if (xform_comp(N)) return comp_table(N, out);
     int L, ne;
     if (!xform_blue_shape(N, &L, &ne)) return -1;
     if (N > 2048 && L == 4096) return ne == 5 ? blue_split_table<5>(N, out) : blue_split_table<6>(N, out);
@@ -407,6 +445,18 @@ static cudaError_t dispatch_xf(int N, int prec, bool wide, F &&f)
     }
     int L, ne;
     if (!xform_blue_shape(N, &L, &ne)) return cudaErrorInvalidValue;
+    int A = 0, B = 0;
+    if (xform_comp(N) && comp_shape(N, &A, &B)) {
+        switch (comp_teams(A)) {
+        case 2: return f(XfComp<2>{});
+        case 4: return f(XfComp<4>{});
+        case 8: return f(XfComp<8>{});
+        case 12: return f(XfComp<12>{});
+        case 18: return f(XfComp<18>{});
+        case 24: return f(XfComp<24>{});
+        default: return f(XfComp<32>{});
+        }
+    }
     if (N > 2048 && L == 4096) return ne == 5 ? f(XfBlueSplit<5>{}) : f(XfBlueSplit<6>{});
     switch (L) {
     case 512: return f(XfBlue<512, 8>{});
@@ -438,7 +488,8 @@ static cudaError_t dispatch_xf(int N, int prec, bool wide, F &&f)
 //
 // CTAs per SM aimed at, as threads per SM, swept for the two kernels (forward,
 // gradient): register FFTs of 8 points 1024 and 640 (64 and 96 registers a
-// thread), of 16 points 512 and 384 (128 and 168), the others (Bluestein's 16 points and more, the tensor-core passes) 512.
+// thread), of 16 points 512 and 384 (128 and 168), composite lengths 960 and
+// 640, the others (Bluestein's 16 points and more, the tensor-core passes) 512.
 // E.g. N = 2048 with 16 points, M = 8192, J = 4: gradient 324 us at 256 threads,
 // 285 at 384, 314 at 512 (spills).
 enum { XK_FORWARD = 0, XK_GRAD = 1 };
@@ -447,7 +498,8 @@ __host__ __device__ constexpr int xf_min_ctas(int kernel)
 {
     const bool grad = kernel == XK_GRAD;
     const bool mixed = Xf::kN > 0 && Xf::NCONST > Xf::kN;
-    const int t = Xf::kBlue || mixed           ? 512
+    const int t = PermutedTrait<Xf>::value       ? (grad ? 640 : 960)
+                  : Xf::kBlue || mixed           ? 512
                   : Xf::kN >= 512 && Xf::NE == 16 ? (grad ? 384 : 512)
                                                  : (grad ? 640 : 1024);
     return t / Xf::NT > 32 ? 32 : (t / Xf::NT > 1 ? t / Xf::NT : 1);
@@ -484,13 +536,25 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_FORWARD)) k_forward
         float2 v[E];
 #pragma unroll
         for (int e = 0; e < E; e++)
-            v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+            v[e] = xf_valid(xf, e, tid, N) ? T[(size_t)row * N + xf_vidx(xf, e, tid)] : make_float2(0.f, 0.f);
         if (row + (int)gridDim.x < M) prefetch_row<Xf>(T + (size_t)(row + gridDim.x) * N, N, tid);
         xf.fwd(v, buf, cst, tid);
         float *yr = Y + ((size_t)row * J + j) * N;
+        if constexpr (PermutedTrait<Xf>::value) {
+            // the spectrum's order is strided over the threads: turned around
+            // in the (free) vector buffer, so that the stores are whole lines
+            float *st = reinterpret_cast<float *>(buf);
 #pragma unroll
-        for (int e = 0; e < E; e++)
-            if (Xf::valid(e, tid, N)) yr[tid + e * NT] = cabs2(v[e]);
+            for (int e = 0; e < E; e++)
+                if (xf.live(e, tid)) st[xf.kidx(e, tid)] = cabs2(v[e]);
+            __syncthreads();
+            for (int i = tid; i < N; i += NT) yr[i] = st[i];
+            __syncthreads();
+        } else {
+#pragma unroll
+            for (int e = 0; e < E; e++)
+                if (Xf::valid(e, tid, N)) yr[tid + e * NT] = cabs2(v[e]);
+        }
     }
 }
 
@@ -523,9 +587,17 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_GRAD)) k_grad(int N
             // the row's intensities are in flight during the transform, where
             // the registers allow (not beside Bluestein's 16 points)
             float yv[E];
+            if constexpr (PermutedTrait<Xf>::value) {  // whole lines into the free vector buffer, then this thread's
+                float *st = reinterpret_cast<float *>(buf);
+                for (int i = tid; i < N; i += NT) st[i] = y[i];
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; e++) yv[e] = xf.live(e, tid) ? st[xf.kidx(e, tid)] : 0.f;
+                __syncthreads();
+            }
 #pragma unroll
             for (int e = 0; e < E; e++) {
-                v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+                v[e] = xf_valid(xf, e, tid, N) ? T[(size_t)row * N + xf_vidx(xf, e, tid)] : make_float2(0.f, 0.f);
                 if constexpr (!Xf::kBlue) yv[e] = y[tid + e * NT];
             }
             if (j + 1 < J) {
@@ -535,17 +607,17 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_GRAD)) k_grad(int N
                 prefetch_row<Xf>(T + (size_t)(row + gridDim.x) * N, N, tid);
             }
             xf.fwd(v, buf, cst, tid);
-            if constexpr (Xf::kBlue) {
+            if constexpr (Xf::kBlue && !PermutedTrait<Xf>::value) {
 #pragma unroll
                 for (int e = 0; e < E; e++) yv[e] = Xf::valid(e, tid, N) ? y[tid + e * NT] : 0.f;
             }
 #pragma unroll
             for (int e = 0; e < E; e++) {
                 if (cost == COST_AMPLITUDE) {
-                    const float c = Xf::valid(e, tid, N) ? cost_coef(cost, v[e], yv[e], f) : 0.f;
+                    const float c = xf_valid(xf, e, tid, N) ? cost_coef(cost, v[e], yv[e], f) : 0.f;
                     v[e] = cscale(v[e], c);
                 } else {
-                    const float r = Xf::valid(e, tid, N) ? yv[e] - cabs2(v[e]) : 0.f;
+                    const float r = xf_valid(xf, e, tid, N) ? yv[e] - cabs2(v[e]) : 0.f;
                     f = fmaf(r, r, f);
                     v[e] = cscale(v[e], r);
                 }
@@ -557,7 +629,7 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_GRAD)) k_grad(int N
         if (G) {
 #pragma unroll
             for (int e = 0; e < E; e++)
-                if (Xf::valid(e, tid, N)) G[(size_t)row * N + tid + e * NT] = cscale(acc[e], cost_grad_scale(cost));
+                if (xf_valid(xf, e, tid, N)) G[(size_t)row * N + xf_vidx(xf, e, tid)] = cscale(acc[e], cost_grad_scale(cost));
         }
         float fv[1] = {f};
         block_sum<1>(fv, red, fsum);
@@ -588,7 +660,7 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_FORWARD)) k_fields(
         float2 v[E];
 #pragma unroll
         for (int e = 0; e < E; e++)
-            v[e] = Xf::valid(e, tid, N) ? T[(size_t)row * N + tid + e * NT] : make_float2(0.f, 0.f);
+            v[e] = xf_valid(xf, e, tid, N) ? T[(size_t)row * N + xf_vidx(xf, e, tid)] : make_float2(0.f, 0.f);
         if (w && j == 0) {
             float en[1] = {0.f};
 #pragma unroll
@@ -599,8 +671,8 @@ __global__ void __launch_bounds__(Xf::NT, xf_min_ctas<Xf>(XK_FORWARD)) k_fields(
         xf.fwd(v, buf, cst, tid);
 #pragma unroll
         for (int e = 0; e < E; e++) {
-            const int pat = j * N + tid + e * NT;
-            if (Xf::valid(e, tid, N) && pat < Nd) Zd[(size_t)pat * M + row] = v[e];
+            const int pat = j * N + xf_kidx(xf, e, tid);
+            if (xf_valid(xf, e, tid, N) && pat < Nd) Zd[(size_t)pat * M + row] = v[e];
         }
     }
 }

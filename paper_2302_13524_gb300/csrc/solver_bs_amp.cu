@@ -9,6 +9,7 @@ long long solver_launch_blue_amp(int N, const SolverParams &p, cudaStream_t s, i
 {
     int L = 0, ne = 0;
     if (!xform_blue_shape(N, &L, &ne)) return (long long)cudaErrorInvalidValue;
+    if (xform_comp(N)) return (long long)launch_solver_comp_amp(N, p, s, clusters_out);
     if (N > 2048 && L == 4096)
         return ne == 5 ? (long long)launch_solver_t<XfBlueSplit<5>, 1, COST_AMPLITUDE>(p, s, clusters_out)
                        : (long long)launch_solver_t<XfBlueSplit<6>, 1, COST_AMPLITUDE>(p, s, clusters_out);

@@ -499,8 +499,18 @@ __host__ __device__ size_t solver_smem(int N, int J, int m)
     return bytes + sizeof(Gram);
 }
 
+// CTAs per SM to leave registers for: 128 a thread for the composite lengths,
+// two of up to 256 threads for powers of two from 256
+template <class Xf, int G>
+__host__ __device__ constexpr int solver_min_ctas()
+{
+    constexpr int BT = SolverCfg<Xf, G>::BT;
+    if (PermutedTrait<Xf>::value) return BT <= 512 ? 512 / BT : 1;
+    return BT <= 256 && Xf::kN >= 256 ? 2 : 1;
+}
+
 template <class Xf, int G, int COST = COST_INTENSITY>
-__global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <= 256 && Xf::kN >= 256) ? 2 : 1)
+__global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, solver_min_ctas<Xf, G>())
     k_solver(SolverParams P)
 {
     using C = SolverCfg<Xf, G>;
@@ -544,12 +554,14 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
     for (int i = tid; i < NCS; i += BT) tws[i] = P.tw[i];
     Xf xf;
     xf.setup(P.masks + (size_t)jm * N, P.tw + Xf::NCONST, N, ttid);
-    auto valid = [&](int e) { return Xf::valid(e, ttid, N); };
+    auto valid = [&](int e) { return xf_valid(xf, e, ttid, N); };
+    auto vi = [&](int e) { return xf_vidx(xf, e, ttid); };  // register e's place in the vector
+    auto ki = [&](int e) { return xf_kidx(xf, e, ttid); };  // and in the spectrum
     const float gsc = cost_grad_scale(COST);  // the gradient's scale (-4 intensity, 2 amplitude)
     // x[e] = X[index of register e] (zero past the end)
     auto load_X = [&](float2 (&x)[E]) {
 #pragma unroll
-        for (int e = 0; e < E; e++) x[e] = valid(e) ? X[ttid + e * NT] : make_float2(0.f, 0.f);
+        for (int e = 0; e < E; e++) x[e] = valid(e) ? X[vi(e)] : make_float2(0.f, 0.f);
     };
     const int sl_shift = (even && (SL & (SL - 1)) == 0) ? __ffs(SL) - 1 : -1;
     // the CTA that owns element n; for uneven slices by counting the slice
@@ -617,12 +629,12 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
             for (int o = 0; o < JC; o++) cluster.map_shared_rank(X, o)[lo + i] = v;
         }
     };
-    // this team's thread-strided natural-order vector v to the owners' Y[jm][:]
+    // this team's vector v to the owners' Y[jm][:]
     auto push_to_owners = [&](const float2 (&v)[E]) {
 #pragma unroll
         for (int e = 0; e < E; e++) {
             if (!valid(e)) continue;
-            const int n = ttid + e * NT;
+            const int n = vi(e);
             const int o = owner(n);
             cluster.map_shared_rank(Yr, o)[jm * SL + (n - slice0[o])] = v[e];
         }
@@ -658,7 +670,7 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
 #pragma unroll
             for (int e = 0; e < E; e++) {
                 if constexpr (kMixed) yv[e] = __half2float(yr16[ttid + e * NT]) * ysc;
-                else yv[e] = valid(e) ? yr[ttid + e * NT] : 0.f;
+                else yv[e] = valid(e) ? yr[ki(e)] : 0.f;
                 if (isfinite(yv[e])) pv[0] += yv[e];
                 else pv[1] += 1.f;
             }
@@ -1041,7 +1053,7 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, (SolverCfg<Xf, G>::BT <=
         if (P.Zd) {
 #pragma unroll
             for (int e = 0; e < E; e++) {
-                const int pat = jm * N + ttid + e * NT;
+                const int pat = jm * N + ki(e);
                 if (valid(e) && pat < P.Nd) P.Zd[(size_t)pat * M + row] = early ? make_float2(0.f, 0.f) : cscale(z[e], tsc);
             }
         }

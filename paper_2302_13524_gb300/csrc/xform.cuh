@@ -477,6 +477,219 @@ struct XfBlueSplit {
     }
 };
 
+// XfComp<TEAMS>: N = A B with A <= TEAMS and B <= 128 (2286 = 18 x 127).  With
+// n = B n1 + n2 and k = k1 + A k2 the DFT is A-point DFTs over n1, twiddles
+// W_N^{n2 k1}, and B-point DFTs over n2, one for each k1:
+//   X[k1 + A k2] = sum_{n2} W_B^{n2 k2} W_N^{n2 k1} sum_{n1} x[B n1 + n2] W_A^{n1 k1}.
+// A half warp owns one k1.  Each of its threads forms the sums over n1 for its
+// n2 = t + 16 r directly (A complex multiply-adds for each of 8 values, read
+// from the masked vector in shared memory, W_A^m from a table), and the half
+// warp does the B-point DFT by Bluestein at L = 256 >= 2B - 1 with 16 points
+// per thread: 16 x 16 passes whose one exchange stays inside it.  A transform
+// therefore has one block barrier in front of the sums (and one behind the
+// last read) where Bluestein of the whole length has one or two for each of its
+// 6 to 9 exchanges, and moves half as much through shared memory, which is what
+// bounds both (about 3,600 against 6,500 wavefronts at N = 2286).  The two
+// halves of a warp read the same vector elements, one wavefront for both; with
+// a whole warp per k1 (8 points per lane, two exchanges) the sums alone read
+// twice as much.
+//
+// Layouts: team = tid / 16, t = tid % 16, register e: the vector's element
+// n = B team + t + 16 e (a team owns a run of B elements), the spectrum's
+// element k = team + A (t + 16 e); valid while t + 16 e < B and team < A.
+// Constants: [ W_256^{r j} (15 x 16) | filter F_256(b) / 256 | chirp c_B (128) |
+// W_A^m (32) | W_N^{n2 k1} c_{n2} in order k1 B + n2 (N) | (A, B) ].  The first
+// NCONST entries go to shared memory.
+constexpr int kCompB = 128, kCompA = 32;  // largest factors
+
+// Teams of the instantiated variant that holds A (0: none).
+__host__ __device__ constexpr int comp_teams(int A)
+{
+    return A < 1 ? 0 : A <= 2 ? 2 : A <= 4 ? 4 : A <= 8 ? 8 : A <= 12 ? 12 : A <= 18 ? 18 : A <= 24 ? 24 : A <= 32 ? 32 : 0;
+}
+
+// The split N = A B: the smallest A that leaves B <= 128, because the direct
+// A-point sums cost A per element; false when N has none up to 32 (a prime
+// factor above 128, or an unlucky product) or when its teams are too many for
+// the length: the cost goes with the teams (each does a 256-point Bluestein
+// whatever its B), plain Bluestein's with its length L.  Gradient of 3000 rows,
+// J = 4: 2, 4, 8, 12, 18, 24, 32 teams take 70, 100, 190, 330, 550, 845, 1340 us;
+// L = 512, 1024, 2048, 4096, the split outputs and 8192 take 74, 163, 333, 770,
+// 940, 1460.  At N = 2286 (18 x 127), J = 4: gradient of 8192 rows 2556 us with
+// the split outputs and their FP64 setup, 2277 without the latter, 1681 so; a
+// retrieval of 2048 rows with early exit 54.1 -> 40.0 ms.
+__host__ __device__ inline bool comp_shape(int N, int *A, int *B)
+{
+    const int most = N <= 256 ? 2 : N <= 512 ? 4 : N <= 1024 ? 12 : N <= 2048 ? 18 : N <= kBlueSplitMaxN ? 24 : 32;
+    for (int a = 1; a <= kCompA; a++)
+        if (N % a == 0 && N / a <= kCompB) {
+            *A = a;
+            *B = N / a;
+            return comp_teams(a) <= most;
+        }
+    return false;
+}
+
+// Where element e of a thread's registers sits in the vector (vidx) and in the
+// spectrum (kidx), and whether it exists: tid + e NT for the register FFTs and
+// Bluestein, the policy's own maps for XfComp.
+template <class Xf, class = void>
+struct PermutedTrait {
+    static constexpr bool value = false;
+};
+template <class Xf>
+struct PermutedTrait<Xf, decltype((void)Xf::kPermuted)> {
+    static constexpr bool value = true;
+};
+template <class Xf>
+__device__ __forceinline__ int xf_vidx(const Xf &xf, int e, int tid)
+{
+    if constexpr (PermutedTrait<Xf>::value) return xf.vidx(e, tid);
+    else return tid + e * Xf::NT;
+}
+template <class Xf>
+__device__ __forceinline__ int xf_kidx(const Xf &xf, int e, int tid)
+{
+    if constexpr (PermutedTrait<Xf>::value) return xf.kidx(e, tid);
+    else return tid + e * Xf::NT;
+}
+template <class Xf>
+__device__ __forceinline__ bool xf_valid(const Xf &xf, int e, int tid, int n)
+{
+    if constexpr (PermutedTrait<Xf>::value) return xf.live(e, tid);
+    else return Xf::valid(e, tid, n);
+}
+
+template <int TEAMS>
+struct XfComp {
+    static constexpr bool kBlue = true;
+    static constexpr bool kPermuted = true;  // index maps instead of tid + e NT
+    static constexpr int kN = 0;
+    static constexpr int NT = 16 * TEAMS, NE = kCompB / 16, EL = 16, L = 256;
+    static constexpr int XPITCH = 17, XLEN = 16 * XPITCH;  // one team's exchange block
+    // the vector (N <= NT NE elements), then the teams' exchange blocks
+    static constexpr int LBUF = NT * NE + TEAMS * XLEN;
+    static constexpr int BUFS = 1;
+    static constexpr int OFF_FILT = 240, OFF_CHIRP = OFF_FILT + L, OFF_WA = OFF_CHIRP + kCompB;
+    static constexpr int NCONST = OFF_WA + kCompA;
+    __host__ __device__ static constexpr int shared_consts(int n) { return NCONST; }
+
+    float2 dm[NE];  // mask at this thread's elements
+    float2 tc[NE];  // W_N^{n2 k1} c_{n2}, k1 = team
+    int A, B;
+
+    __device__ __forceinline__ int vidx(int e, int tid) const { return B * (tid >> 4) + (tid & 15) + 16 * e; }
+    __device__ __forceinline__ int kidx(int e, int tid) const { return (tid >> 4) + A * ((tid & 15) + 16 * e); }
+    __device__ __forceinline__ bool live(int e, int tid) const { return (tid >> 4) < A && (tid & 15) + 16 * e < B; }
+
+    __device__ __forceinline__ void setup(const float2 *__restrict__ mask, const float2 *__restrict__ after, int n,
+                                          int tid)
+    {
+        A = (int)after[n].x;
+        B = (int)after[n].y;
+#pragma unroll
+        for (int e = 0; e < NE; e++) tc[e] = live(e, tid) ? after[vidx(e, tid)] : make_float2(0.f, 0.f);
+        load_mask(mask, nullptr, n, tid);
+    }
+    __device__ __forceinline__ void load_mask(const float2 *__restrict__ mask, const float2 *cst, int n, int tid)
+    {
+#pragma unroll
+        for (int e = 0; e < NE; e++) dm[e] = live(e, tid) ? mask[vidx(e, tid)] : make_float2(0.f, 0.f);
+    }
+    // 256-point FFT of v (index t + 16 e) in the half warp, natural order out
+    template <int SIGN>
+    __device__ __forceinline__ void fft256(float2 (&v)[EL], float2 *xb, const float2 *cst, int t) const
+    {
+        dft_small<16, SIGN>(v);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 16; q++) xb[t * XPITCH + q] = v[q];
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 16; r++) {
+            v[r] = xb[r * XPITCH + t];
+            if (r > 0) {
+                float2 w = cst[(r - 1) * 16 + t];
+                if constexpr (SIGN > 0) w.y = -w.y;
+                v[r] = cmul(v[r], w);
+            }
+        }
+        dft_small<16, SIGN>(v);
+    }
+    // x (n2 = t + 16 e, times tc already) <- its cyclic convolution with the chirp's conjugate
+    __device__ __forceinline__ void conv(float2 (&x)[NE], float2 *xb, const float2 *cst, int t) const
+    {
+        float2 v[EL];
+#pragma unroll
+        for (int e = 0; e < EL; e++) v[e] = e < NE ? x[e < NE ? e : 0] : make_float2(0.f, 0.f);
+        fft256<-1>(v, xb, cst, t);
+#pragma unroll
+        for (int e = 0; e < EL; e++) v[e] = cmul(v[e], cst[OFF_FILT + t + 16 * e]);
+        fft256<+1>(v, xb, cst, t);
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = v[e];
+    }
+    // x[e] <- sum_{m < A} src[B m + n2] W_A^{SIGN-signed m team}, n2 = t + 16 e
+    template <int SIGN>
+    __device__ __forceinline__ void dft_a(float2 (&x)[NE], const float2 *src, const float2 *cst, int tid) const
+    {
+        const int team = tid >> 4, t = tid & 15;
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = make_float2(0.f, 0.f);
+        if (team >= A) return;
+        const float2 *WA = cst + OFF_WA;
+        int q = 0;  // m team mod A
+#pragma unroll 2
+        for (int m = 0; m < A; m++) {
+            float2 w = WA[q];
+            if constexpr (SIGN > 0) w.y = -w.y;
+            const float2 *p = src + B * m + t;
+#pragma unroll
+            for (int e = 0; e < NE; e++) {
+                const float2 v = p[16 * e];  // past B: another element, dropped below
+                x[e].x = fmaf(w.x, v.x, fmaf(-w.y, v.y, x[e].x));
+                x[e].y = fmaf(w.x, v.y, fmaf(w.y, v.x, x[e].y));
+            }
+            q += team;
+            if (q >= A) q -= A;
+        }
+#pragma unroll
+        for (int e = 0; e < NE; e++)
+            if (t + 16 * e >= B) x[e] = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ void fwd(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
+    {
+        const int t = tid & 15;
+#pragma unroll
+        for (int e = 0; e < NE; e++)
+            if (live(e, tid)) buf[vidx(e, tid)] = cmul(x[e], dm[e]);
+        __syncthreads();
+        dft_a<-1>(x, buf, cst, tid);
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = cmul(x[e], tc[e]);
+        conv(x, buf + NT * NE + (tid >> 4) * XLEN, cst, t);
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = live(e, tid) ? cmul(x[e], cst[OFF_CHIRP + t + 16 * e]) : make_float2(0.f, 0.f);
+        __syncthreads();  // the vector is read before anyone writes the next one
+    }
+    __device__ __forceinline__ void adj(float2 (&x)[NE], float2 *buf, const float2 *cst, int tid)
+    {
+        const int t = tid & 15;
+#pragma unroll
+        for (int e = 0; e < NE; e++)
+            x[e] = live(e, tid) ? cmul(cconj(x[e]), cst[OFF_CHIRP + t + 16 * e]) : make_float2(0.f, 0.f);
+        conv(x, buf + NT * NE + (tid >> 4) * XLEN, cst, t);
+#pragma unroll
+        for (int e = 0; e < NE; e++)
+            if (live(e, tid)) buf[vidx(e, tid)] = cconj(cmul(x[e], tc[e]));
+        __syncthreads();
+        dft_a<+1>(x, buf, cst, tid);
+#pragma unroll
+        for (int e = 0; e < NE; e++) x[e] = cmulc(x[e], dm[e]);
+        __syncthreads();
+    }
+};
+
 // ---------------------------------------------------------------------------
 // XfMixed<N>: N a power of two, 64 <= N <= 4096, written N = 16^A 8^B with A
 // as large as possible.  The FP32 transforms of XfPow2<N>, plus a tensor-core
