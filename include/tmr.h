@@ -368,8 +368,10 @@ tmr_status tmr_set_init_model(tmr_handle *h, tmr_mlp *model);
 long long tmr_learned_rows(tmr_handle *h);
 
 /* The solver schedule the handle uses (after autotuning): 1, 2 or 4 masks per
- * CTA, 16 for one CTA per row, 32 for the full-length Bluestein plan; 0 for a
- * NULL handle or when no schedule fits (see tmr_create). */
+ * CTA, 16 for one CTA per row, 32 for the full-length Bluestein plan, 64 for the
+ * layout of 16 over a cluster of CTAs per row (rows too large for one CTA;
+ * chosen by the autotuner, not by opt.schedule); 0 for a NULL handle or when no
+ * schedule fits (see tmr_create). */
 int tmr_schedule(const tmr_handle *h);
 /* The schedules the autotuner timed when this handle was made, and the mean
  * time of their timed runs in milliseconds (each: 4 power and 6 L-BFGS

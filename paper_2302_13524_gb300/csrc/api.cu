@@ -251,8 +251,8 @@ bool schedule_ok(int N, int J, int m, int G, int smem_optin, int prec = 0, int c
 tmr_status autotune(tmr_handle *h, int smem_optin, int *G_out, bool *timed)
 {
     *timed = false;
-    int cand[5], nc = 0;
-    for (int G : {1, 2, 4, kRowSchedule, kBlueFullSchedule})
+    int cand[6], nc = 0;
+    for (int G : {1, 2, 4, kRowSchedule, kRowClusterSchedule, kBlueFullSchedule})
         if (schedule_ok(h->N, h->J, h->opt.m, G, smem_optin, h->xk, h->opt.cost) && (G != kRowSchedule || h->pairs) &&
             (G != kBlueFullSchedule || h->tw_alt))
             cand[nc++] = G;
@@ -508,7 +508,8 @@ tmr_status tmr_create(tmr_handle **out, int N, int M, int J, const void *masks,
     TMR_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), "attr");
     if (o.cost == TMR_COST_AMPLITUDE && xk != 0 && xk != 3)
         return fail(TMR_ERR_UNSUPPORTED, "the amplitude cost runs on the FP32 1D transforms (precision FP32, probe_n1 0)");
-    if (o.schedule != 0 && !schedule_ok(N, J, o.m, o.schedule, smem_optin, xk, o.cost))
+    if (o.schedule != 0 &&
+        (o.schedule == kRowClusterSchedule || !schedule_ok(N, J, o.m, o.schedule, smem_optin, xk, o.cost)))
         return fail(TMR_ERR_UNSUPPORTED,
                     "opt.schedule must be 1, 2 or 4 (dividing J), 16 (one CTA per row) or 32 (full-length "
                     "Bluestein), and fit the device");

@@ -105,6 +105,13 @@ struct SolverParams {
 // per thread, FP32, N = 512 .. 2048 with J N / 16 <= 512, L-BFGS pairs in the
 // global workspace p.pairs (solver_row.cuh).
 constexpr int kRowSchedule = 16;
+// G = kRowClusterSchedule (64): the same layout over a cluster of CTAs holding
+// two or more masks each, for rows too large for one CTA: N = 4096 with J = 4,
+// 6 or 8, N = 2048 with J = 6 or 8, intensity cost.  Chosen by the autotuner only.
+constexpr int kRowClusterSchedule = 64;
+int solver_rowc_masks(int N, int J);  // masks per CTA, 0: no such variant
+size_t solver_rowc_smem(int N, int J);
+cudaError_t launch_solver_rowc(int N, const SolverParams &p, cudaStream_t s, int *clusters_out);
 // Lanczos steps of the spectral start at most: the 2 k values of a
 // Gram-Schmidt reduction fit one warp
 constexpr int kMaxLanczos = 16;

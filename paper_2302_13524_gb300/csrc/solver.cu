@@ -11,6 +11,7 @@ bool solver_variant_exists(int N, int G, int prec)
     if (prec == 2) return (G == 1 || G == 2 || G == 4) && (N == 512 || N == 4096) && G * fft_threads(N) <= 512;
     if (prec == 3) return G == 1 && fft_supported(N);
     if (G == kRowSchedule) return prec == 0 && (N == 512 || N == 1024 || N == 2048);
+    if (G == kRowClusterSchedule) return prec == 0 && (N == 2048 || N == 4096);
     if (G == kBlueFullSchedule) return prec == 0 && N > 2048 && N <= 2731;
     if (G != 1 && G != 2 && G != 4) return false;
     if (prec != 0) return G == 1 && mixed_supported(N);
@@ -36,6 +37,8 @@ static long long solver_dispatch(int N, int G, int what, const SolverParams *p, 
                                  int *clusters_out)
 {
     if (G == kRowSchedule) return solver_dispatch_row(N, what, p, s, clusters_out);
+    if (G == kRowClusterSchedule)
+        return what == 0 ? (long long)solver_rowc_smem(N, p->J) : (long long)launch_solver_rowc(N, *p, s, clusters_out);
     if (G == kBlueFullSchedule) return solver_dispatch_blue8192(N, 6, what, p, s, clusters_out);
     if (p->prec == 2) return solver_dispatch_2d(N, G, what, p, s, clusters_out);
     if (p->prec == 3) return solver_dispatch_dense(N, G, what, p, s, clusters_out);
@@ -64,6 +67,7 @@ bool solver_schedule_valid(int N, int J, int G, int prec)
 {
     if (!solver_variant_exists(N, G, prec) || J < 1) return false;
     if (G == kRowSchedule) return J * (N / 16) <= 512;
+    if (G == kRowClusterSchedule) return solver_rowc_masks(N, J) > 0;
     if (G == kBlueFullSchedule) return true;  // one mask per CTA
     return J % G == 0;
 }

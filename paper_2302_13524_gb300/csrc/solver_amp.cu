@@ -21,6 +21,7 @@ bool solver_cost_supported(int N, int G, int prec, int cost)
     if (cost == COST_INTENSITY) return true;
     if (cost != COST_AMPLITUDE || prec != 0) return false;
     if (G == kRowSchedule) return N == 512 || N == 1024 || N == 2048;
+    if (G == kRowClusterSchedule) return false;
     if (fft_supported(N)) return (G == 1 || G == 2 || G == 4) && G * fft_threads(N) <= 512;
     int L = 0, ne = 0;
     return G == 1 && xform_blue_shape(N, &L, &ne) && L <= 4096;

@@ -28,6 +28,14 @@
 //     instead of cluster barriers, no distributed shared memory.
 // Rows come from the same atomic work counter; a persistent launch of one
 // CTA per SM (or two, when shared memory allows) walks the matrix.
+//
+// A row too large for one CTA (N = 4096, or more than four masks of N = 2048)
+// takes the same layout over a small cluster (CLU): each CTA holds two or more
+// of its masks and a slice of its vectors, so that a row occupies half or a
+// quarter of the SMs that one mask per CTA (solver_impl.cuh) gives it, and the
+// serial parts of an iteration (reductions, scalars, barriers: half of it at one
+// mask per CTA) are shared by that many more rows.  N = 4096, J = 4, M = 4096,
+// 20 iterations: 21.6 ms against 29.0.
 #pragma once
 
 #include "solver_impl.cuh"
@@ -52,6 +60,31 @@ struct RowCfg {
 // Variants exist for N = 512 .. 2048 with J * N / 16 <= 512 threads.
 __host__ __device__ constexpr bool row_variant_fits(int N, int J) { return J >= 1 && J * (N / kRowPts) <= 512; }
 
+// The same layout over a cluster (CLU): each CTA holds JB of the row's masks
+// and a 1/JC slice of its vectors, JC = J / JB.  JB: the most masks that fit
+// 512 threads, at least 2; 0 when the row fits one CTA or no such split exists.
+__host__ __device__ constexpr int rowc_masks(int N, int J)
+{
+    if ((N != 2048 && N != 4096) || J > kMaxMasks || row_variant_fits(N, J)) return 0;
+    for (int jb = 512 / (N / kRowPts); jb >= 2; jb--)
+        if (J % jb == 0 && J / jb >= 2) return jb;
+    return 0;
+}
+
+template <int N>
+__host__ __device__ size_t rowc_smem(int J)
+{
+    using C = RowCfg<N>;
+    const int JB = rowc_masks(N, J), JC = J / JB, NW = JB * C::NT / 32;
+    const size_t SL = (N + JC - 1) / JC;
+    const size_t f2 = ((size_t)C::NCONST + 1) / 2 * 2 + (size_t)JB * N /*masks*/ + (size_t)JB * C::LBUF /*exchange; the
+                      first also gathers p*/ + 2 * SL /*t, g*/ + (JC - 1) * SL /*peers' sums*/ + kMaxLanczos * kMaxLanczos;
+    size_t bytes = f2 * sizeof(float2) +
+                   sizeof(float) * ((size_t)JB * N /*y*/ + (size_t)kParts * NW + 2 * (size_t)JC * kParts);
+    bytes = (bytes + 15) & ~(size_t)15;
+    return bytes + sizeof(Gram);
+}
+
 template <int N>
 __host__ __device__ size_t row_smem(int J, int m)
 {
@@ -74,27 +107,44 @@ __host__ __device__ size_t row_smem(int J, int m)
 // most 504 columns for its pairs; the Lanczos vectors go to tensor memory when
 // their blocks fit in 512 columns (klz = k steps, else 0).  The allocation is
 // the next power of two of the larger need (at least 32).
-__host__ __device__ inline int row_ept(int N, int J) { return (N + J * (N / kRowPts) - 1) / (J * (N / kRowPts)); }
-__host__ __device__ inline int row_tmem_block(int N, int J, int m) { return 4 * row_ept(N, J) * (m + 1); }
-__host__ __device__ inline int row_tmem_lanczos_block(int N, int J, int k) { return 2 * row_ept(N, J) * ((k + 3) & ~3); }
-__host__ __device__ inline int row_quarter_warps(int N, int J) { return (J * (N / kRowPts) / 32 + 3) / 4; }
+struct RowShape {
+    int threads, ept;  // threads of the CTA, vector elements per thread
+    __host__ __device__ int quarter_warps() const { return (threads / 32 + 3) / 4; }
+    __host__ __device__ int pair_block(int m) const { return 4 * ept * (m + 1); }
+    __host__ __device__ int lanczos_block(int k) const { return 2 * ept * ((k + 3) & ~3); }
+    __host__ __device__ int klz(bool lanczos_start, int k) const
+    {
+        return lanczos_start && k >= 1 && k <= kMaxLanczos && quarter_warps() * lanczos_block(k) <= 512 ? k : 0;
+    }
+    __host__ __device__ int cols(int m, int klz) const
+    {
+        int need = quarter_warps() * pair_block(m);
+        if (klz > 0) {
+            const int lz = quarter_warps() * lanczos_block(klz);
+            if (lz > need) need = lz;
+        }
+        int c = 32;
+        while (c < need) c *= 2;
+        return c;
+    }
+};
+// JB masks in the CTA, nloc vector elements
+__host__ __device__ inline RowShape row_shape(int N, int JB, int nloc)
+{
+    const int bt = JB * (N / kRowPts);
+    return RowShape{bt, (nloc + bt - 1) / bt};
+}
+
+// The same of the variant with one CTA per row.
+__host__ __device__ inline int row_ept(int N, int J) { return row_shape(N, J, N).ept; }
+__host__ __device__ inline int row_quarter_warps(int N, int J) { return row_shape(N, J, N).quarter_warps(); }
+__host__ __device__ inline int row_tmem_block(int N, int J, int m) { return row_shape(N, J, N).pair_block(m); }
+__host__ __device__ inline int row_tmem_lanczos_block(int N, int J, int k) { return row_shape(N, J, N).lanczos_block(k); }
 __host__ __device__ inline int row_tmem_klz(int N, int J, bool lanczos_start, int k)
 {
-    return lanczos_start && k >= 1 && k <= kMaxLanczos && row_quarter_warps(N, J) * row_tmem_lanczos_block(N, J, k) <= 512
-               ? k
-               : 0;
+    return row_shape(N, J, N).klz(lanczos_start, k);
 }
-__host__ __device__ inline int row_tmem_cols(int N, int J, int m, int klz)
-{
-    int need = row_quarter_warps(N, J) * row_tmem_block(N, J, m);
-    if (klz > 0) {
-        const int lz = row_quarter_warps(N, J) * row_tmem_lanczos_block(N, J, klz);
-        if (lz > need) need = lz;
-    }
-    int c = 32;
-    while (c < need) c *= 2;
-    return c;
-}
+__host__ __device__ inline int row_tmem_cols(int N, int J, int m, int klz) { return row_shape(N, J, N).cols(m, klz); }
 
 // No global pair workspace: the pairs are in tensor memory.
 __host__ __device__ inline size_t row_pair_stride(int N, int m)
@@ -104,19 +154,23 @@ __host__ __device__ inline size_t row_pair_stride(int N, int m)
     return 0;
 }
 
-template <int N, int COST = COST_INTENSITY>
+template <int N, int COST = COST_INTENSITY, bool CLU = false>
 __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
 {
     using C = RowCfg<N>;
     constexpr int NT = C::NT, E = C::E, R = C::R, BPT = C::BPT, NCONST = C::NCONST, LBUF = C::LBUF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int J = P.J, m = P.m, M = P.M;
+    // JT masks in all, J of them in this CTA, JC CTAs (rank jr), my slice [lo, lo + nmine)
+    const int JT = P.J, J = CLU ? rowc_masks(N, P.J) : P.J, JC = CLU ? JT / J : 1, m = P.m, M = P.M;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int jr = CLU ? (int)cluster.block_rank() : 0;
+    const int SL = (N + JC - 1) / JC, lo = CLU ? jr * N / JC : 0, nmine = CLU ? (jr + 1) * N / JC - lo : N;
     const int BT = J * NT;
     const int NW = BT / 32;
     const int tid = threadIdx.x;
     const int team = tid / NT, ttid = tid - team * NT;
     const int lane = tid & 31, warp = tid >> 5;
-    const size_t K = (size_t)J * N;
+    const size_t K = (size_t)JT * N, KL = (size_t)J * N;  // intensities of the row, and of this CTA
     const float JN = (float)K;
     const float gsc = cost_grad_scale(COST);  // the gradient's scale (-4 intensity, 2 amplitude)
 
@@ -125,26 +179,32 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
     float2 *msk = tws + (NCONST + 1) / 2 * 2;     // [J][N]
     float2 *bufs = msk + (size_t)J * N;           // [J][LBUF]
     float2 *buf = bufs + (size_t)team * LBUF;     // this team's exchange buffer
-    float2 *X = bufs + (size_t)J * LBUF;          // direction p (or the vector being transformed)
-    float2 *ts = X + N;                           // t
-    float2 *gs = ts + N;                          // g
-    float *ys = reinterpret_cast<float *>(gs + N);  // [J][N] intensities of the row (scaled)
+    // direction p (or the vector being transformed); in a cluster it is gathered
+    // in the first exchange buffer, which is free until it has been read
+    float2 *X = CLU ? bufs : bufs + (size_t)J * LBUF;
+    float2 *ts = CLU ? bufs + (size_t)J * LBUF : X + N;  // t (my slice)
+    float2 *gs = ts + SL;                                // g (my slice)
+    float2 *Yr = gs + SL;                                // CLU: the peers' sums for my slice [JC - 1][SL]
+    float2 *lzG = CLU ? Yr + (size_t)(JC - 1) * SL : X;  // Gram matrix of the Lanczos vectors
+    float *ys = reinterpret_cast<float *>(CLU ? lzG + kMaxLanczos * kMaxLanczos : gs + SL);  // [J][N] intensities (scaled)
     float *red = ys + (size_t)J * N;                // [kParts][NW]
+    float *part = red + kParts * NW;                // CLU: [2][JC][kParts]
     Gram &Gm = *reinterpret_cast<Gram *>(
-        smem_raw + ((reinterpret_cast<unsigned char *>(red + kParts * NW) - smem_raw + 15) & ~(size_t)15));
+        smem_raw + ((reinterpret_cast<unsigned char *>(CLU ? part + 2 * JC * kParts : part) - smem_raw + 15) & ~(size_t)15));
 
     // L-BFGS pairs in tensor memory: element e (i = tid + e BT) of the pair in
     // slot a at columns tcol(a, e) .. + 3 (s, then y)
     __shared__ uint32_t tmem_base;
-    const int klz = row_tmem_klz(N, J, P.lanczos && P.init == INIT_SPECTRAL && !P.T_init, P.power_iters);
-    const int ncols = row_tmem_cols(N, J, m, klz);
+    const RowShape shape = row_shape(N, J, SL);
+    const int klz = shape.klz(P.lanczos && P.init == INIT_SPECTRAL && !P.T_init, P.power_iters);
+    const int ncols = shape.cols(m, klz);
     if (warp == 0) tmem_alloc_warp(&tmem_base, (uint32_t)ncols);
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();
-    const int EPT = (N + BT - 1) / BT;
+    const int EPT = shape.ept;
     const uint32_t tquarter = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16);
-    const uint32_t tlane = tquarter + (uint32_t)((warp >> 2) * row_tmem_block(N, J, m));
+    const uint32_t tlane = tquarter + (uint32_t)((warp >> 2) * shape.pair_block(m));
     auto tcol = [&](int a, int e) { return tlane + (uint32_t)(4 * (a * EPT + e)); };
 
     // twiddles of the passes between the first and the last:
@@ -158,7 +218,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             tws[off + i] = make_float2((float)c, (float)s);
         }
     }
-    for (int i = tid; i < J * N; i += BT) msk[i] = P.masks[i];
+    for (int i = tid; i < J * N; i += BT) msk[i] = P.masks[jr * J * N + i];
     const float2 *dm = msk + (size_t)team * N;  // this team's mask
     const float *yt = ys + (size_t)team * N;    // this team's intensities
     float2 wb[BPT];  // last-pass twiddle bases exp(-2 pi i b / N), b = ttid + i NT
@@ -182,28 +242,74 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
 #pragma unroll
         for (int e = 0; e < E; e++) x[e] = cmulc(x[e], dm[ttid + e * NT]);
     };
+    if constexpr (CLU) cluster.sync();  // every CTA runs before anyone touches its shared memory
     // after a transform every thread has passed its last exchange, so the team
     // buffer is free: park the natural-order result there (unpadded)
     auto park = [&](const float2 (&x)[E]) {
 #pragma unroll
         for (int e = 0; e < E; e++) buf[ttid + e * NT] = x[e];
     };
-    // sum over the masks of the parked results, element i, times s
-    auto team_sum = [&](int i, float s) {
+    // sum over this CTA's masks of the parked results, element i of the vector
+    auto local_sum = [&](int i) {
         float2 acc = bufs[i];
 #pragma unroll
         for (int j = 1; j < kMaxMasks; j++)
             if (j < J) acc = cadd(acc, bufs[j * LBUF + i]);
+        return acc;
+    };
+    // Make the parked results of every mask available to team_sum.  In a cluster
+    // each CTA adds its own masks for the peers' slices and pushes the sums
+    // into their Yr.  (A cluster barrier follows every read of Yr before the next
+    // share: a reduction's, or the gather's of the next vector.)
+    auto share = [&]() {
+        __syncthreads();
+        if constexpr (CLU) {
+            for (int o = 0; o < JC; o++) {
+                if (o == jr) continue;
+                const int b = o * N / JC, n = (o + 1) * N / JC - b;
+                float2 *dst = cluster.map_shared_rank(Yr, o) + (size_t)(jr < o ? jr : jr - 1) * SL;
+                for (int i = tid; i < n; i += BT) dst[i] = local_sum(b + i);
+            }
+            cluster.sync();
+        }
+    };
+    // sum over all masks, element i of my slice, times s (CTAs in rank order)
+    auto team_sum = [&](int i, float s) {
+        float2 acc = local_sum(lo + i);
+        if constexpr (CLU) {
+            float2 tot = make_float2(0.f, 0.f);
+            for (int r = 0; r < JC; r++) tot = cadd(tot, r == jr ? acc : Yr[(size_t)(r < jr ? r : r - 1) * SL + i]);
+            acc = tot;
+        }
         return cscale(acc, s);
     };
     auto load_team = [&](const float2 *src, float2 (&x)[E]) {
 #pragma unroll
         for (int e = 0; e < E; e++) x[e] = src[ttid + e * NT];
     };
+    // x <- the whole vector whose slices are src.  In a cluster the slices are
+    // first pushed into every CTA's X, once every CTA is done with the parked
+    // results there (X is its first exchange buffer).
+    auto load_vec = [&](const float2 *src, float2 (&x)[E]) {
+        if constexpr (CLU) {
+            cluster.sync();
+            for (int o = 0; o < JC; o++) {
+                float2 *dst = cluster.map_shared_rank(X, o) + lo;
+                for (int i = tid; i < nmine; i += BT) dst[i] = src[i];
+            }
+            cluster.sync();
+            load_team(X, x);
+            __syncthreads();  // X is read before the transform reuses it
+        } else {
+            __syncthreads();
+            load_team(src, x);
+        }
+    };
     // Block-wide sums of nv <= 32 per-thread values: warp sums, then thread k
     // adds the NW warp sums of value k in warp order into Gm.red[k].  With
     // all = false only warp 0 (threads 0 .. 31) goes on to read the sums, so
     // a warp barrier replaces the block barrier after them.
+    int sel = 0;
     auto block_reduce = [&](float (&v)[32], int nv, bool all = true) {
         if (nv <= 6) {
             // constant indices only: a runtime index would move v to local memory
@@ -219,28 +325,51 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             if (lane < nv) red[lane * NW + warp] = v[0];
         }
         __syncthreads();
+        float acc = 0.f;
         if (tid < nv) {
-            float acc = 0.f;
 #pragma unroll
             for (int w = 0; w < 16; w++)  // at most 16 warps: the loads are in flight together
                 if (w < NW) acc += red[tid * NW + w];
-            Gm.red[tid] = acc;
         }
+        if constexpr (CLU) {
+            // the CTAs' sums into every CTA's part, then added in rank order
+            // (two buffers in turn, as in k_solver)
+            float *pb = part + sel * JC * kParts;
+            sel ^= 1;
+            if (tid < nv)
+                for (int o = 0; o < JC; o++) cluster.map_shared_rank(pb, o)[jr * kParts + tid] = acc;
+            cluster.sync();
+            if (tid < nv) {
+                acc = 0.f;
+#pragma unroll
+                for (int o = 0; o < kMaxMasks / 2; o++)
+                    if (o < JC) acc += pb[o * kParts + tid];
+            }
+        }
+        if (tid < nv) Gm.red[tid] = acc;
         if (all) __syncthreads();
         else __syncwarp();
     };
 
     while (true) {
-        if (tid == 0) Gm.row = (int)atomicAdd(P.queue, 1u);
-        __syncthreads();
+        if constexpr (CLU) {
+            if (jr == 0 && tid == 0) {
+                const int r = (int)atomicAdd(P.queue, 1u);
+                for (int o = 0; o < JC; o++) cluster.map_shared_rank(&Gm.row, o)[0] = r;
+            }
+            cluster.sync();
+        } else {
+            if (tid == 0) Gm.row = (int)atomicAdd(P.queue, 1u);
+            __syncthreads();
+        }
         const int row = Gm.row;
-        if (row >= M) break;
+        if (row >= M) break;  // nobody touches another CTA's shared memory after this barrier
 
         // ---- intensities, their sum and finiteness ----
         {
             float pv[32] = {0.f};
-            const float *yr = P.y + (size_t)row * K;
-            for (size_t i = tid; i < K; i += BT) {
+            const float *yr = P.y + (size_t)row * K + jr * KL;
+            for (size_t i = tid; i < KL; i += BT) {
                 const float v = yr[i];
                 ys[i] = v;
                 if (isfinite(v)) pv[0] += v;
@@ -264,7 +393,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             __syncthreads();
             // the row is solved with y 4^-j and t 2^-j (exact scales; see k_solver)
             const float ysc = Gm.yscale;
-            for (size_t i = tid; i < K; i += BT) ys[i] *= ysc;
+            for (size_t i = tid; i < KL; i += BT) ys[i] *= ysc;
             __syncthreads();
         }
         const float sumy = Gm.sumy * Gm.yscale;
@@ -276,38 +405,37 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             // ---- initialisation ----
             if (P.T_init) {
                 const float tinv = 1.f / Gm.tsc;
-                for (int i = tid; i < N; i += BT) ts[i] = cscale(P.T_init[(size_t)row * N + i], tinv);
+                for (int i = tid; i < nmine; i += BT) ts[i] = cscale(P.T_init[(size_t)row * N + lo + i], tinv);
             } else if (P.init == INIT_BP) {
                 float2 u[E];
 #pragma unroll
                 for (int e = 0; e < E; e++) u[e] = make_float2(sqrtf(fmaxf(yt[ttid + e * NT], 0.f)), 0.f);
                 adj(u);
                 park(u);
-                __syncthreads();
-                for (int i = tid; i < N; i += BT) ts[i] = team_sum(i, 1.f / JN);
+                share();
+                for (int i = tid; i < nmine; i += BT) ts[i] = team_sum(i, 1.f / JN);
             } else {
                 // seed: the proposed start (learned initialiser) where it is
                 // finite and nonzero, else the Philox vector
                 bool seeded = false;
                 if (P.T_cand && P.seed_from_cand) {
                     float pv[32] = {0.f};
-                    for (int i = tid; i < N; i += BT) {
-                        const float2 v = P.T_cand[(size_t)row * N + i];
+                    for (int i = tid; i < nmine; i += BT) {
+                        const float2 v = P.T_cand[(size_t)row * N + lo + i];
                         ts[i] = v;
                         pv[0] += cabs2(v);
                     }
                     block_reduce(pv, 1);
                     seeded = isfinite(Gm.red[0]) && Gm.red[0] > 0.f;
-                    if (seeded && tid == 0 && P.cand_wins) atomicAdd(P.cand_wins, 1u);
+                    if (seeded && jr == 0 && tid == 0 && P.cand_wins) atomicAdd(P.cand_wins, 1u);
                 }
                 if (!seeded)
-                    for (int i = tid; i < N; i += BT) ts[i] = philox_cnormal(P.seed, (uint32_t)row, (uint32_t)i);
+                    for (int i = tid; i < nmine; i += BT) ts[i] = philox_cnormal(P.seed, (uint32_t)row, (uint32_t)(lo + i));
                 if (P.init == INIT_SPECTRAL && P.lanczos) {
                     const float mean = sumy / (float)K;
                     auto applyA = [&]() {
-                        __syncthreads();
                         float2 x[E];
-                        load_team(ts, x);
+                        load_vec(ts, x);
                         fwd(x);
 #pragma unroll
                         for (int e = 0; e < E; e++) {
@@ -317,28 +445,28 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                         }
                         adj(x);
                         park(x);
-                        __syncthreads();
-                        for (int i = tid; i < N; i += BT) gs[i] = team_sum(i, 1.f / JN);
+                        share();
+                        for (int i = tid; i < nmine; i += BT) gs[i] = team_sum(i, 1.f / JN);
                         __syncthreads();
                     };
-                    float2 *V = P.krylov + (size_t)blockIdx.x * lanczos_region(N, P.power_iters);
-                    // (the direction p is not in use yet: its buffer X holds
-                    // the Gram matrix of the Lanczos vectors)
+                    float2 *V = P.krylov + (size_t)(blockIdx.x / JC) * lanczos_region(N, P.power_iters);
+                    // (the direction p is not in use yet: one CTA per row keeps
+                    // the Gram matrix of the Lanczos vectors in its buffer X)
                     if (klz)
-                        lanczos_start_tmem(klz, N, EPT,
-                                           tquarter + (uint32_t)((warp >> 2) * row_tmem_lanczos_block(N, J, klz)), ts,
-                                           gs, X, Gm.red, &Gm.SY[0][0], &Gm.YY[0][0], applyA, block_reduce);
+                        lanczos_start_tmem(klz, nmine, EPT,
+                                           tquarter + (uint32_t)((warp >> 2) * shape.lanczos_block(klz)), ts,
+                                           gs, lzG, Gm.red, &Gm.SY[0][0], &Gm.YY[0][0], applyA, block_reduce);
                     else
-                        lanczos_start(P.power_iters, N, ts, gs, V, (size_t)N, V + (size_t)P.power_iters * N, Gm.red,
+                        lanczos_start(P.power_iters, nmine, ts, gs, V + lo, (size_t)N,
+                                      V + (size_t)P.power_iters * N + jr * kMaxLanczos * kMaxLanczos, Gm.red,
                                       &Gm.SY[0][0], &Gm.YY[0][0], applyA, block_reduce);
                 } else if (P.init == INIT_SPECTRAL) {
                     const float mean = sumy / (float)K;
                     for (int it = 0; it < P.power_iters; it++) {
                         // t <- A t, A = Q^H diag(tau) Q / (J N), tau = min(y / mean, clip);
                         // the norm is restored every 8th step and at the end
-                        __syncthreads();
                         float2 x[E];
-                        load_team(ts, x);
+                        load_vec(ts, x);
                         fwd(x);
 #pragma unroll
                         for (int e = 0; e < E; e++) {
@@ -348,10 +476,10 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                         }
                         adj(x);
                         park(x);
-                        __syncthreads();
+                        share();
                         const bool renorm = ((it & 7) == 7) || (it == P.power_iters - 1);
                         float pv[32] = {0.f};
-                        for (int i = tid; i < N; i += BT) {
+                        for (int i = tid; i < nmine; i += BT) {
                             const float2 s = team_sum(i, 1.f / JN);
                             ts[i] = s;
                             pv[0] = fmaf(s.x, s.x, fmaf(s.y, s.y, pv[0]));
@@ -360,28 +488,27 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                             block_reduce(pv, 1);
                             const float nrm = Gm.red[0];
                             const float inv = nrm > 0.f ? rsqrtf(nrm) : 0.f;
-                            for (int i = tid; i < N; i += BT) ts[i] = cscale(ts[i], inv);
+                            for (int i = tid; i < nmine; i += BT) ts[i] = cscale(ts[i], inv);
                         }
                     }
                 }
                 // rescale to the Parseval norm ||t||^2 = sum(y) / (J N)
                 float pv[32] = {0.f};
-                for (int i = tid; i < N; i += BT) pv[0] += cabs2(ts[i]);
+                for (int i = tid; i < nmine; i += BT) pv[0] += cabs2(ts[i]);
                 block_reduce(pv, 1);
                 const float nrm = Gm.red[0];
                 const float sc = nrm > 0.f ? sqrtf(sumy / JN) / sqrtf(nrm) : 0.f;
-                for (int i = tid; i < N; i += BT) ts[i] = cscale(ts[i], sc);
+                for (int i = tid; i < nmine; i += BT) ts[i] = cscale(ts[i], sc);
             }
 
             // ---- per-row selection: a proposed start (learned initialiser) against this one ----
             if (P.T_cand && P.judge_cand) {
                 const float tinv = 1.f / Gm.tsc;
-                for (int i = tid; i < N; i += BT) gs[i] = cscale(P.T_cand[(size_t)row * N + i], tinv);
+                for (int i = tid; i < nmine; i += BT) gs[i] = cscale(P.T_cand[(size_t)row * N + lo + i], tinv);
                 float fv[2];
                 for (int c = 0; c < 2; c++) {  // f at the start above, then at the proposal
-                    __syncthreads();
                     float2 x[E];
-                    load_team(c == 0 ? ts : gs, x);
+                    load_vec(c == 0 ? ts : gs, x);
                     fwd(x);
                     float pv[32] = {0.f};
 #pragma unroll
@@ -392,15 +519,14 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                     fv[c] = Gm.red[0];
                 }
                 if (fv[1] < fv[0]) {  // NaN proposals lose
-                    for (int i = tid; i < N; i += BT) ts[i] = gs[i];
-                    if (tid == 0 && P.cand_wins) atomicAdd(P.cand_wins, 1u);
+                    for (int i = tid; i < nmine; i += BT) ts[i] = gs[i];
+                    if (jr == 0 && tid == 0 && P.cand_wins) atomicAdd(P.cand_wins, 1u);
                 }
             }
 
             // ---- f and gradient at the start ----
             {
-                __syncthreads();
-                load_team(ts, z);
+                load_vec(ts, z);
                 fwd(z);
                 float2 u[E];
                 float pv[32] = {0.f};
@@ -408,8 +534,8 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                 for (int e = 0; e < E; e++) u[e] = cscale(z[e], cost_coef(COST, z[e], yt[ttid + e * NT], pv[0]));
                 adj(u);
                 park(u);
-                __syncthreads();
-                for (int i = tid; i < N; i += BT) {
+                share();
+                for (int i = tid; i < nmine; i += BT) {
                     const float2 g = team_sum(i, gsc);
                     gs[i] = g;
                     pv[1] += cabs2(g);
@@ -449,7 +575,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                     tmem_fence_after_sync();
                     for (int e = 0; e < EPT; e++) {
                         const int i = tid + e * BT;
-                        const bool in = i < N;
+                        const bool in = i < nmine;
                         float2 acc = in ? cscale(gs[i], gam) : make_float2(0.f, 0.f);
 #pragma unroll
                         for (int k = 0; k < kSlots; k++) {
@@ -464,13 +590,25 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                                 acc.y = fmaf(c1r[k], sa.y, fmaf(c2r[k], ya.y, acc.y));
                             }
                         }
-                        if (in) X[i] = make_float2(-acc.x, -acc.y);
+                        if constexpr (CLU) {
+                            // to every CTA; my own copy waits in the new pair's
+                            // cells, X being an exchange buffer until then
+                            if (in)
+                                for (int o = 0; o < JC; o++)
+                                    cluster.map_shared_rank(X, o)[lo + i] = make_float2(-acc.x, -acc.y);
+                            tmem_st2(tcol(sn_slot, e), -acc.x, -acc.y);
+                        } else {
+                            if (in) X[i] = make_float2(-acc.x, -acc.y);
+                        }
                     }
+                    if constexpr (CLU) tmem_wait_st();
                 }
-                __syncthreads();
+                if constexpr (CLU) cluster.sync();
+                else __syncthreads();
                 // C: w = F(d .* p)
                 float2 w[E];
                 load_team(X, w);
+                if constexpr (CLU) __syncthreads();  // X is read before the transform reuses it
                 fwd(w);
                 // D: the step -- the amplitude cost's line search, or the quartic's exact minimiser
                 if constexpr (COST == COST_AMPLITUDE) {
@@ -519,7 +657,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                 }
                 adj(u);
                 park(u);
-                __syncthreads();
+                share();
                 // G: new gradient, new pair, batched dot products
                 {
                     float pv[32];
@@ -527,11 +665,19 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                     for (int k = 0; k < 32; k++) pv[k] = 0.f;
                     for (int e = 0; e < EPT; e++) {
                         const int i = tid + e * BT;
-                        const bool in = i < N;
-                        float2 gn = make_float2(0.f, 0.f), sn = gn, yn = gn;
+                        const bool in = i < nmine;
+                        float2 gn = make_float2(0.f, 0.f), sn = gn, yn = gn, pn = gn;
+                        if constexpr (CLU) {
+                            uint32_t r[2];
+                            tmem_ld2(tcol(sn_slot, e), r);
+                            tmem_wait_ld();
+                            tmem_reg_ready(r);
+                            pn = make_float2(__uint_as_float(r[0]), __uint_as_float(r[1]));
+                        }
                         if (in) {
                             gn = team_sum(i, gsc);
-                            sn = cscale(X[i], al);
+                            if constexpr (!CLU) pn = X[i];
+                            sn = cscale(pn, al);
                             yn = csub(gn, gs[i]);
                             ts[i] = cadd(ts[i], sn);
                             gs[i] = gn;
@@ -573,9 +719,9 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
         // ---- outputs (rows decided before initialisation come back as zero) ----
         const bool early = Gm.early != 0;
         const float tsc = Gm.tsc;
-        for (int i = tid; i < N; i += BT)
-            P.T_out[(size_t)row * N + i] = early ? make_float2(0.f, 0.f) : cscale(ts[i], tsc);
-        if (tid == 0) {
+        for (int i = tid; i < nmine; i += BT)
+            P.T_out[(size_t)row * N + lo + i] = early ? make_float2(0.f, 0.f) : cscale(ts[i], tsc);
+        if (jr == 0 && tid == 0) {
             if (P.row_status) P.row_status[row] = Gm.status;
             if (P.row_iters) P.row_iters[row] = Gm.done;
             if (P.row_loss) {
@@ -588,7 +734,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
         if (P.Zd) {
 #pragma unroll
             for (int e = 0; e < E; e++) {
-                const int pat = team * N + ttid + e * NT;
+                const int pat = (jr * J + team) * N + ttid + e * NT;
                 if (pat < P.Nd) P.Zd[(size_t)pat * M + row] = early ? make_float2(0.f, 0.f) : cscale(z[e], tsc);
             }
         }
@@ -659,6 +805,45 @@ cudaError_t launch_solver_row_t(const SolverParams &p, cudaStream_t s, int *ctas
     if (ctas_out) *ctas_out = (int)grid;
     k_solver_row<N, COST><<<(int)grid, BT, sm, s>>>(p);
     return cudaGetLastError();
+}
+
+// The row layout over clusters of JC CTAs.  Shared memory (above 114 KB for
+// every supported shape; raised to that otherwise) keeps it at one such CTA per
+// SM, so no tensor-memory allocation waits for a CTA of another cluster, which
+// might wait for this one in turn.
+template <int N, int COST = COST_INTENSITY>
+cudaError_t launch_solver_rowc_t(const SolverParams &p, cudaStream_t s, int *clusters_out)
+{
+    const int JB = rowc_masks(N, p.J);
+    if (JB == 0 || p.m < 1 || p.m > kMaxMem) return cudaErrorInvalidValue;
+    const int JC = p.J / JB;
+    size_t sm = rowc_smem<N>(p.J);
+    const auto kernel = k_solver_row<N, COST, true>;
+    if (sm < 116 * 1024) sm = 116 * 1024;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = JC;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(JB * RowCfg<N>::NT);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(JC);
+    int maxc = 0;
+    e = cudaOccupancyMaxActiveClusters(&maxc, kernel, &cfg);
+    if (e != cudaSuccess) return e;
+    if (maxc < 1) return cudaErrorInvalidConfiguration;
+    int nc = maxc < p.M ? maxc : p.M;
+    if (p.lanczos && p.init == INIT_SPECTRAL && nc > p.krylov_units) nc = p.krylov_units;  // one region each
+    if (nc < 1) nc = 1;
+    cfg.gridDim = dim3(nc * JC);
+    if (clusters_out) *clusters_out = nc;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
 }  // namespace tmr
