@@ -138,10 +138,25 @@ __device__ __forceinline__ void dft_small(float2 (&x)[R])
     }
 }
 
+// The barrier of a transform's exchanges: of the whole block, or of the T threads
+// (whole warps) that share the transform, named by id >= 1.
+struct BlockBarrier {
+    __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+template <int T>
+struct TeamBarrier {
+    int id;
+    __device__ __forceinline__ void operator()() const
+    {
+        if constexpr (T == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(T) : "memory");
+    }
+};
+
 // One Stockham pass (see file comment).  buf: shared, fft_buf_len(N) float2.
 // TRAIL = false drops the barrier after the read-back (ping-pong buffers, below).
-template <int N, int T, int R, int NS, int TWOFF, int SIGN, bool LAST, bool TRAIL = true>
-__device__ __forceinline__ void fft_pass(float2 (&v)[N / T], float2 *buf, const float2 *tw, int tid)
+template <int N, int T, int R, int NS, int TWOFF, int SIGN, bool LAST, bool TRAIL = true, class Bar = BlockBarrier>
+__device__ __forceinline__ void fft_pass(float2 (&v)[N / T], float2 *buf, const float2 *tw, int tid, Bar bar = {})
 {
     constexpr int E = N / T, BPT = E / R;
     static_assert(BPT * R == E, "radix must divide the points per thread");
@@ -171,10 +186,10 @@ __device__ __forceinline__ void fft_pass(float2 (&v)[N / T], float2 *buf, const 
         }
     }
     if constexpr (!LAST) {
-        __syncthreads();
+        bar();
 #pragma unroll
         for (int e = 0; e < E; e++) v[e] = buf[fft_pad(tid + e * T)];
-        if constexpr (TRAIL) __syncthreads();
+        if constexpr (TRAIL) bar();
     }
 }
 
@@ -278,14 +293,14 @@ __device__ __forceinline__ void block_fft_rb(float2 (&v)[N / T], float2 *buf, co
 // (BPT = E / R butterflies each).  The last pass takes its twiddles from
 // per-thread bases as above, one per butterfly: butterfly i of thread tid is
 // b = tid + i T, and wb[i] = exp(-2 pi i b / N).
-template <int N, int T, int R, int SIGN, int p>
+template <int N, int T, int R, int SIGN, int p, class Bar = BlockBarrier>
 __device__ __forceinline__ void fft_passes_rbx(float2 (&v)[N / T], float2 *buf, const float2 *tw,
-                                               const float2 (&wb)[N / T / R], int tid)
+                                               const float2 (&wb)[N / T / R], int tid, Bar bar = {})
 {
     using Pl = FftPlan<N, N / T, R>;
     if constexpr (p < Pl::P - 1) {
-        fft_pass<N, T, Pl::radix(p), Pl::ns(p), Pl::tw_off(p), SIGN, false>(v, buf, tw, tid);
-        fft_passes_rbx<N, T, R, SIGN, p + 1>(v, buf, tw, wb, tid);
+        fft_pass<N, T, Pl::radix(p), Pl::ns(p), Pl::tw_off(p), SIGN, false>(v, buf, tw, tid, bar);
+        fft_passes_rbx<N, T, R, SIGN, p + 1>(v, buf, tw, wb, tid, bar);
     } else if constexpr (p == Pl::P - 1) {
         constexpr int BPT = N / T / R;
         static_assert(Pl::radix(p) == R, "last pass must use the full radix");
@@ -302,11 +317,11 @@ __device__ __forceinline__ void fft_passes_rbx(float2 (&v)[N / T], float2 *buf, 
     }
 }
 
-template <int N, int T, int R, int SIGN>
+template <int N, int T, int R, int SIGN, class Bar = BlockBarrier>
 __device__ __forceinline__ void block_fft_rbx(float2 (&v)[N / T], float2 *buf, const float2 *tw,
-                                              const float2 (&wb)[N / T / R], int tid)
+                                              const float2 (&wb)[N / T / R], int tid, Bar bar = {})
 {
-    fft_passes_rbx<N, T, R, SIGN, 0>(v, buf, tw, wb, tid);
+    fft_passes_rbx<N, T, R, SIGN, 0>(v, buf, tw, wb, tid, bar);
 }
 
 

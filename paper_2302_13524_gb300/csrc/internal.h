@@ -110,7 +110,7 @@ constexpr int kRowSchedule = 16;
 // 6 or 8, N = 2048 with J = 6 or 8, intensity cost.  Chosen by the autotuner only.
 constexpr int kRowClusterSchedule = 64;
 int solver_rowc_masks(int N, int J);  // masks per CTA, 0: no such variant
-size_t solver_rowc_smem(int N, int J);
+size_t solver_rowc_smem(int N, int J, int m);  // more than any SM has where the row's state does not fit
 cudaError_t launch_solver_rowc(int N, const SolverParams &p, cudaStream_t s, int *clusters_out);
 // Lanczos steps of the spectral start at most: the 2 k values of a
 // Gram-Schmidt reduction fit one warp
@@ -130,6 +130,7 @@ long long solver_dispatch_blue8192(int N, int ne, int what, const SolverParams *
 // 2048), clusters with G = 1, 2, 4 for powers of two, and G = 1 for the
 // Bluestein lengths with L <= 4096 (other N: none).
 cudaError_t launch_solver_row_amp(int N, const SolverParams &p, cudaStream_t s, int *ctas_out);
+cudaError_t launch_solver_row_regs(int N, const SolverParams &p, cudaStream_t s, int *ctas_out);
 cudaError_t launch_solver_amp(int N, int G, const SolverParams &p, cudaStream_t s, int *clusters_out);
 bool solver_cost_supported(int N, int G, int prec, int cost);
 bool solver_variant_exists(int N, int G, int prec = 0);

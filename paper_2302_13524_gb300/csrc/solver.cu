@@ -38,7 +38,7 @@ static long long solver_dispatch(int N, int G, int what, const SolverParams *p, 
 {
     if (G == kRowSchedule) return solver_dispatch_row(N, what, p, s, clusters_out);
     if (G == kRowClusterSchedule)
-        return what == 0 ? (long long)solver_rowc_smem(N, p->J) : (long long)launch_solver_rowc(N, *p, s, clusters_out);
+        return what == 0 ? (long long)solver_rowc_smem(N, p->J, p->m) : (long long)launch_solver_rowc(N, *p, s, clusters_out);
     if (G == kBlueFullSchedule) return solver_dispatch_blue8192(N, 6, what, p, s, clusters_out);
     if (p->prec == 2) return solver_dispatch_2d(N, G, what, p, s, clusters_out);
     if (p->prec == 3) return solver_dispatch_dense(N, G, what, p, s, clusters_out);

@@ -30,7 +30,8 @@ static int row_max_ctas_t(int J, int m)
     // the largest tensor-memory need of the schedule (a 16-step Lanczos start)
     // bounds the resident CTAs of every launch
     const int klz = row_tmem_klz(N, J, true, kMaxLanczos);
-    if (row_launch_shape<N, COST_INTENSITY>(J, m, klz, &sm, &occ) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+    if (row_launch_shape<N, COST_INTENSITY, true>(J, m, row_tmem_cols(N, J, m, klz), &sm, &occ) != cudaSuccess ||
+        cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -116,9 +116,10 @@ struct RowShape {
     {
         return lanczos_start && k >= 1 && k <= kMaxLanczos && quarter_warps() * lanczos_block(k) <= 512 ? k : 0;
     }
-    __host__ __device__ int cols(int m, int klz) const
+    // z: the row's fields take 2 kRowPts columns more of each warp, after the pairs
+    __host__ __device__ int cols(int m, int klz, bool z = false) const
     {
-        int need = quarter_warps() * pair_block(m);
+        int need = quarter_warps() * (pair_block(m) + (z ? 2 * kRowPts : 0));
         if (klz > 0) {
             const int lz = quarter_warps() * lanczos_block(klz);
             if (lz > need) need = lz;
@@ -128,6 +129,15 @@ struct RowShape {
         return c;
     }
 };
+// Whether the fields z fit beside the pairs without taking residency: as many
+// CTAs share an SM as its registers (512 threads) and the pairs alone allow.
+__host__ __device__ inline bool row_fields_fit(const RowShape &s, int m, int klz)
+{
+    const int with = s.cols(m, klz, true), without = s.cols(m, klz), by_regs = 512 / s.threads;
+    if (with > 512) return false;
+    const int a = 512 / with, b = 512 / without;
+    return a >= b || a >= by_regs;
+}
 // JB masks in the CTA, nloc vector elements
 __host__ __device__ inline RowShape row_shape(int N, int JB, int nloc)
 {
@@ -154,7 +164,12 @@ __host__ __device__ inline size_t row_pair_stride(int N, int m)
     return 0;
 }
 
-template <int N, int COST = COST_INTENSITY, bool CLU = false>
+// ZT: between a step's update and the next step's line search the fields z wait
+// in tensor memory.  32 registers a thread are then free for both transforms and
+// for the sweeps over the pairs, which keep three loads in flight instead of
+// spilling or waiting for each: 8192 rows, 20 iterations, J = 4, N = 2048 15.17 ->
+// 14.46 ms, N = 1024 10.65 -> 9.39; 4096 rows of N = 4096 (CLU) 21.6 -> 19.6.
+template <int N, int COST = COST_INTENSITY, bool CLU = false, bool ZT = true>
 __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
 {
     using C = RowCfg<N>;
@@ -197,7 +212,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
     __shared__ uint32_t tmem_base;
     const RowShape shape = row_shape(N, J, SL);
     const int klz = shape.klz(P.lanczos && P.init == INIT_SPECTRAL && !P.T_init, P.power_iters);
-    const int ncols = shape.cols(m, klz);
+    const int ncols = shape.cols(m, klz, ZT);
     if (warp == 0) tmem_alloc_warp(&tmem_base, (uint32_t)ncols);
     tmem_fence_before_sync();
     __syncthreads();
@@ -206,6 +221,41 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
     const uint32_t tquarter = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16);
     const uint32_t tlane = tquarter + (uint32_t)((warp >> 2) * shape.pair_block(m));
     auto tcol = [&](int a, int e) { return tlane + (uint32_t)(4 * (a * EPT + e)); };
+    const uint32_t tfields =
+        tquarter + (uint32_t)(shape.quarter_warps() * shape.pair_block(m) + (warp >> 2) * 2 * kRowPts);
+    auto put_fields = [&](const float2 (&z)[E]) {
+        if constexpr (ZT) tmem_st32(tfields, z);
+    };
+    auto get_fields = [&](float2 (&z)[E]) {
+        if constexpr (ZT) {
+            tmem_wait_st();
+            tmem_ld32(tfields, z);
+            tmem_wait_ld();
+            tmem_reg_ready(z);
+        }
+    };
+
+    // f(k, s, y) for element e of the np pairs by age, three loads in flight (six
+    // measure the same).  Loads past np repeat one: under a condition their
+    // registers would stay taken around the whole loop.
+    auto for_pairs = [&](int np, int e, auto &&f) {
+        constexpr int Q = 3;
+#pragma unroll
+        for (int k0 = 0; k0 < kMaxMem; k0 += Q) {
+            if (k0 >= np) break;
+            uint32_t r[Q][4];
+#pragma unroll
+            for (int q = 0; q < Q; q++) tmem_ld4(tcol(Gm.slot[k0 + q < np ? k0 + q : k0], e), r[q]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                tmem_reg_ready(r[q]);
+                if (k0 + q < np)
+                    f(k0 + q, make_float2(__uint_as_float(r[q][0]), __uint_as_float(r[q][1])),
+                      make_float2(__uint_as_float(r[q][2]), __uint_as_float(r[q][3])));
+            }
+        }
+    };
 
     // twiddles of the passes between the first and the last:
     // tw_p[(r - 1) Ns + j] = exp(-2 pi i r j / (Ns R)) at tw_off(p)
@@ -230,15 +280,18 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
     }
     __syncthreads();
 
-    // x <- F(d .* x) and x <- conj(d) .* F^H x for this team's mask; every team
-    // runs the same passes, so the block barriers inside line up
+    // x <- F(d .* x) and x <- conj(d) .* F^H x for this team's mask.  Only the
+    // team's own warps meet inside, so that one team's exchange can run beside
+    // another's butterflies (N = 2048, J = 4: 14.74 ms a launch of 20 iterations
+    // against 14.97 with block barriers).
+    const TeamBarrier<NT> team_bar{1 + team};
     auto fwd = [&](float2 (&x)[E]) {
 #pragma unroll
         for (int e = 0; e < E; e++) x[e] = cmul(x[e], dm[ttid + e * NT]);
-        block_fft_rbx<N, NT, R, -1>(x, buf, tws, wb, ttid);
+        block_fft_rbx<N, NT, R, -1>(x, buf, tws, wb, ttid, team_bar);
     };
     auto adj = [&](float2 (&x)[E]) {
-        block_fft_rbx<N, NT, R, +1>(x, buf, tws, wb, ttid);
+        block_fft_rbx<N, NT, R, +1>(x, buf, tws, wb, ttid, team_bar);
 #pragma unroll
         for (int e = 0; e < E; e++) x[e] = cmulc(x[e], dm[ttid + e * NT]);
     };
@@ -528,6 +581,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             {
                 load_vec(ts, z);
                 fwd(z);
+                put_fields(z);
                 float2 u[E];
                 float pv[32] = {0.f};
 #pragma unroll
@@ -557,39 +611,23 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             // ---- L-BFGS iterations ----
             for (int it = 0; it < P.iters && !Gm.stop; it++) {
                 const int np = Gm.np;
-                int so[kSlots];  // slots by age
-#pragma unroll
-                for (int k = 0; k < kSlots; k++) so[k] = Gm.slot[k <= np ? k : 0];
-                const int sn_slot = so[np < kSlots ? np : 0];  // the free slot (age np) of the new pair
+                const int sn_slot = Gm.slot[np];  // the free slot (age np) of the new pair
                 // A: direction p = -(gamma g + sum c1 s + sum c2 y) into X
                 {
                     const float gam = Gm.gamma;
-                    float c1r[kSlots], c2r[kSlots];
-#pragma unroll
-                    for (int k = 0; k < kSlots; k++) {
-                        c1r[k] = k < np ? Gm.c1[k] : 0.f;
-                        c2r[k] = k < np ? Gm.c2[k] : 0.f;
-                    }
                     // every thread runs all EPT steps (the tensor-memory loads
                     // are warp-wide); steps past N only load
                     tmem_fence_after_sync();
+#pragma unroll 1
                     for (int e = 0; e < EPT; e++) {
                         const int i = tid + e * BT;
                         const bool in = i < nmine;
                         float2 acc = in ? cscale(gs[i], gam) : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int k = 0; k < kSlots; k++) {
-                            if (k < np) {
-                                uint32_t r[4];
-                                tmem_ld4(tcol(so[k], e), r);
-                                tmem_wait_ld();
-                                tmem_reg_ready(r);
-                                const float2 sa = make_float2(__uint_as_float(r[0]), __uint_as_float(r[1]));
-                                const float2 ya = make_float2(__uint_as_float(r[2]), __uint_as_float(r[3]));
-                                acc.x = fmaf(c1r[k], sa.x, fmaf(c2r[k], ya.x, acc.x));
-                                acc.y = fmaf(c1r[k], sa.y, fmaf(c2r[k], ya.y, acc.y));
-                            }
-                        }
+                        for_pairs(np, e, [&](int k, float2 sa, float2 ya) {
+                            const float c1 = Gm.c1[k], c2 = Gm.c2[k];
+                            acc.x = fmaf(c1, sa.x, fmaf(c2, ya.x, acc.x));
+                            acc.y = fmaf(c1, sa.y, fmaf(c2, ya.y, acc.y));
+                        });
                         if constexpr (CLU) {
                             // to every CTA; my own copy waits in the new pair's
                             // cells, X being an exchange buffer until then
@@ -610,6 +648,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                 load_team(X, w);
                 if constexpr (CLU) __syncthreads();  // X is read before the transform reuses it
                 fwd(w);
+                get_fields(z);
                 // D: the step -- the amplitude cost's line search, or the quartic's exact minimiser
                 if constexpr (COST == COST_AMPLITUDE) {
                     const float al = amp_line_search(
@@ -655,6 +694,7 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                     z[e] = make_float2(fmaf(al, w[e].x, z[e].x), fmaf(al, w[e].y, z[e].y));
                     u[e] = cscale(z[e], cost_coef(COST, z[e], yt[ttid + e * NT], fpart));
                 }
+                put_fields(z);
                 adj(u);
                 park(u);
                 share();
@@ -663,6 +703,8 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                     float pv[32];
 #pragma unroll
                     for (int k = 0; k < 32; k++) pv[k] = 0.f;
+                    float dn[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
                     for (int e = 0; e < EPT; e++) {
                         const int i = tid + e * BT;
                         const bool in = i < nmine;
@@ -683,31 +725,28 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
                             gs[i] = gn;
                         }
                         tmem_st4(tcol(sn_slot, e), sn.x, sn.y, yn.x, yn.y);
-#pragma unroll
-                        for (int k = 0; k < kSlots; k++) {
-                            if (k < np) {  // live pairs by age
-                                uint32_t r[4];
-                                tmem_ld4(tcol(so[k], e), r);
-                                tmem_wait_ld();
-                                tmem_reg_ready(r);
-                                const float2 sa = make_float2(__uint_as_float(r[0]), __uint_as_float(r[1]));
-                                const float2 ya = make_float2(__uint_as_float(r[2]), __uint_as_float(r[3]));
-                                pv[4 * k + 0] += cdotr(sa, yn);
-                                pv[4 * k + 1] += cdotr(ya, yn);
-                                pv[4 * k + 2] += cdotr(sa, gn);
-                                pv[4 * k + 3] += cdotr(ya, gn);
-                            } else if (k == np) {  // the new pair (age np)
-                                pv[4 * k + 0] += cdotr(sn, yn);
-                                pv[4 * k + 1] += cdotr(yn, yn);
-                                pv[4 * k + 2] += cdotr(sn, gn);
-                                pv[4 * k + 3] += cdotr(yn, gn);
-                            }
-                        }
+                        for_pairs(np, e, [&](int k, float2 sa, float2 ya) {
+                            pv[4 * k + 0] += cdotr(sa, yn);  // live pairs by age
+                            pv[4 * k + 1] += cdotr(ya, yn);
+                            pv[4 * k + 2] += cdotr(sa, gn);
+                            pv[4 * k + 3] += cdotr(ya, gn);
+                        });
+                        // the new pair (age np), added to its place after the loop
+                        dn[0] += cdotr(sn, yn);
+                        dn[1] += cdotr(yn, yn);
+                        dn[2] += cdotr(sn, gn);
+                        dn[3] += cdotr(yn, gn);
                         pv[kIdxSS] += cabs2(sn);
                         pv[kIdxGG] += cabs2(gn);
                     }
                     tmem_wait_st();  // the new pair is read back from the next iteration on
                     tmem_fence_before_sync();
+#pragma unroll
+                    for (int k = 0; k < kSlots; k++)
+                        if (k == np) {
+#pragma unroll
+                            for (int q = 0; q < 4; q++) pv[4 * k + q] = dn[q];
+                        }
                     pv[kIdxF] = fpart;
                     block_reduce(pv, kParts, false);
                     if (warp == 0) lbfgs_gram_update(Gm, lane, m, it, P.iters, P.tol);
@@ -732,10 +771,16 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
             }
         }
         if (P.Zd) {
+            if (early) {
+#pragma unroll
+                for (int e = 0; e < E; e++) z[e] = make_float2(0.f, 0.f);
+            } else {
+                get_fields(z);
+            }
 #pragma unroll
             for (int e = 0; e < E; e++) {
                 const int pat = (jr * J + team) * N + ttid + e * NT;
-                if (pat < P.Nd) P.Zd[(size_t)pat * M + row] = early ? make_float2(0.f, 0.f) : cscale(z[e], tsc);
+                if (pat < P.Nd) P.Zd[(size_t)pat * M + row] = cscale(z[e], tsc);
             }
         }
         __syncthreads();
@@ -749,17 +794,18 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
 }
 
 // Shared memory and resident CTAs per SM of a launch.  Every CTA holds
-// row_tmem_cols columns of the SM's 512 for its whole life, so at most
+// RowShape::cols columns of the SM's 512 for its whole life, so at most
 // 512 / cols CTAs may share an SM; where registers and shared memory would
 // let more in, the shared-memory request is raised until they do not, and no
 // allocation has to wait for the columns of another CTA of the same launch.
 // (A concurrent launch on another stream that holds tensor memory can delay
 // an allocation until its CTAs on that SM exit; they never wait on this one.)
-template <int N, int COST>
-cudaError_t row_launch_shape(int J, int m, int klz, size_t *smem_out, int *per_sm_out)
+template <int N, int COST, bool ZT>
+cudaError_t row_launch_shape(int J, int m, int cols, size_t *smem_out, int *per_sm_out)
 {
     const int BT = J * RowCfg<N>::NT;
-    const int cap = 512 / row_tmem_cols(N, J, m, klz);
+    const int cap = 512 / cols;
+    const auto kernel = k_solver_row<N, COST, false, ZT>;
     size_t sm = row_smem<N>(J, m);
     int dev = 0, occ = 0, sm_per_mp = 0, optin = 0;
     cudaError_t e;
@@ -769,10 +815,10 @@ cudaError_t row_launch_shape(int J, int m, int klz, size_t *smem_out, int *per_s
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
     for (int pass = 0; pass < 2; pass++) {
         if (sm > (size_t)optin) return cudaErrorInvalidConfiguration;
-        if ((e = cudaFuncSetAttribute(k_solver_row<N, COST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) !=
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) !=
             cudaSuccess)
             return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_solver_row<N, COST>, BT, sm)) != cudaSuccess)
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, BT, sm)) != cudaSuccess)
             return e;
         if (occ < 1) return cudaErrorInvalidConfiguration;
         if (occ <= cap) break;
@@ -785,15 +831,15 @@ cudaError_t row_launch_shape(int J, int m, int klz, size_t *smem_out, int *per_s
     return cudaSuccess;
 }
 
-template <int N, int COST = COST_INTENSITY>
-cudaError_t launch_solver_row_t(const SolverParams &p, cudaStream_t s, int *ctas_out)
+template <int N, int COST, bool ZT>
+cudaError_t launch_solver_row_zt(const SolverParams &p, cudaStream_t s, int *ctas_out)
 {
     if (!row_variant_fits(N, p.J) || p.m < 1 || p.m > kMaxMem) return cudaErrorInvalidValue;
     const int BT = p.J * RowCfg<N>::NT;
     size_t sm = 0;
     int occ = 0, dev = 0, nsm = 0;
     const int klz = row_tmem_klz(N, p.J, p.lanczos && p.init == INIT_SPECTRAL && !p.T_init, p.power_iters);
-    cudaError_t e = row_launch_shape<N, COST>(p.J, p.m, klz, &sm, &occ);
+    cudaError_t e = row_launch_shape<N, COST, ZT>(p.J, p.m, row_shape(N, p.J, N).cols(p.m, klz, ZT), &sm, &occ);
     if (e != cudaSuccess) return e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -803,8 +849,19 @@ cudaError_t launch_solver_row_t(const SolverParams &p, cudaStream_t s, int *ctas
     if (p.lanczos && p.init == INIT_SPECTRAL && grid > p.krylov_units) grid = p.krylov_units;
     if (grid < 1) grid = 1;
     if (ctas_out) *ctas_out = (int)grid;
-    k_solver_row<N, COST><<<(int)grid, BT, sm, s>>>(p);
+    k_solver_row<N, COST, false, ZT><<<(int)grid, BT, sm, s>>>(p);
     return cudaGetLastError();
+}
+
+// The fields in tensor memory where they fit beside the pairs, else in registers
+// (solver_row_regs.cu).
+template <int N, int COST = COST_INTENSITY>
+cudaError_t launch_solver_row_t(const SolverParams &p, cudaStream_t s, int *ctas_out)
+{
+    if (!row_variant_fits(N, p.J) || p.m < 1 || p.m > kMaxMem) return cudaErrorInvalidValue;
+    const int klz = row_tmem_klz(N, p.J, p.lanczos && p.init == INIT_SPECTRAL && !p.T_init, p.power_iters);
+    if (!row_fields_fit(row_shape(N, p.J, N), p.m, klz)) return launch_solver_row_regs(N, p, s, ctas_out);
+    return launch_solver_row_zt<N, COST, true>(p, s, ctas_out);
 }
 
 // The row layout over clusters of JC CTAs.  Shared memory (above 114 KB for
@@ -817,6 +874,7 @@ cudaError_t launch_solver_rowc_t(const SolverParams &p, cudaStream_t s, int *clu
     const int JB = rowc_masks(N, p.J);
     if (JB == 0 || p.m < 1 || p.m > kMaxMem) return cudaErrorInvalidValue;
     const int JC = p.J / JB;
+    if (!row_fields_fit(row_shape(N, JB, (N + JC - 1) / JC), p.m, 0)) return cudaErrorInvalidValue;
     size_t sm = rowc_smem<N>(p.J);
     const auto kernel = k_solver_row<N, COST, true>;
     if (sm < 116 * 1024) sm = 116 * 1024;

@@ -6,9 +6,13 @@ namespace tmr {
 
 int solver_rowc_masks(int N, int J) { return J >= 1 && J <= kMaxMasks ? rowc_masks(N, J) : 0; }
 
-size_t solver_rowc_smem(int N, int J)
+size_t solver_rowc_smem(int N, int J, int m)
 {
-    if (!solver_rowc_masks(N, J)) return 0;
+    const int JB = solver_rowc_masks(N, J);
+    if (!JB) return 0;
+    const int JC = J / JB;
+    // N = 4096, J = 4, m = 6: the pairs leave the fields no room in tensor memory
+    if (!row_fields_fit(row_shape(N, JB, (N + JC - 1) / JC), m, 0)) return (size_t)1 << 30;
     return N == 2048 ? rowc_smem<2048>(J) : rowc_smem<4096>(J);
 }
 

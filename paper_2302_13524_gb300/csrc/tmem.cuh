@@ -74,12 +74,41 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, float a, float b)
                  : "memory");
 }
 
+// Whole warp: 16 complex values from / to 32 consecutive columns of each thread's lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float2 (&z)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=f"(z[0].x), "=f"(z[0].y), "=f"(z[1].x), "=f"(z[1].y), "=f"(z[2].x), "=f"(z[2].y), "=f"(z[3].x), "=f"(z[3].y),
+          "=f"(z[4].x), "=f"(z[4].y), "=f"(z[5].x), "=f"(z[5].y), "=f"(z[6].x), "=f"(z[6].y), "=f"(z[7].x), "=f"(z[7].y),
+          "=f"(z[8].x), "=f"(z[8].y), "=f"(z[9].x), "=f"(z[9].y), "=f"(z[10].x), "=f"(z[10].y), "=f"(z[11].x), "=f"(z[11].y),
+          "=f"(z[12].x), "=f"(z[12].y), "=f"(z[13].x), "=f"(z[13].y), "=f"(z[14].x), "=f"(z[14].y), "=f"(z[15].x), "=f"(z[15].y)
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float2 (&z)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+          "f"(z[0].x), "f"(z[0].y), "f"(z[1].x), "f"(z[1].y), "f"(z[2].x), "f"(z[2].y), "f"(z[3].x), "f"(z[3].y),
+          "f"(z[4].x), "f"(z[4].y), "f"(z[5].x), "f"(z[5].y), "f"(z[6].x), "f"(z[6].y), "f"(z[7].x), "f"(z[7].y),
+          "f"(z[8].x), "f"(z[8].y), "f"(z[9].x), "f"(z[9].y), "f"(z[10].x), "f"(z[10].y), "f"(z[11].x), "f"(z[11].y),
+          "f"(z[12].x), "f"(z[12].y), "f"(z[13].x), "f"(z[13].y), "f"(z[14].x), "f"(z[14].y), "f"(z[15].x), "f"(z[15].y)
+        : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // After tmem_wait_ld: ties the loaded registers to the wait, so that no use of
 // them is scheduled before it (volatile asm statements keep their order).
 __device__ __forceinline__ void tmem_reg_ready(uint32_t (&r)[2]) { asm volatile("" : "+r"(r[0]), "+r"(r[1])); }
+__device__ __forceinline__ void tmem_reg_ready(float2 (&z)[16])
+{
+#pragma unroll
+    for (int i = 0; i < 16; i++) asm volatile("" : "+f"(z[i].x), "+f"(z[i].y));
+}
 __device__ __forceinline__ void tmem_reg_ready(uint32_t (&r)[4])
 {
     asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]));
