@@ -285,8 +285,9 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
     }
 }
 
+// (MNA and MNB: the weight gradients, see plan())
 template <int BN, bool MNA, bool MNB>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(128, MNA && MNB ? 4 : 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
               int K, int stages, int ldc, const __grid_constant__ GemmEpilogue E, int *err)
 {
@@ -484,8 +485,11 @@ namespace {
 // of K alone; 64 tiles of 128 x 32 share that walk.  (32 columns at least, 64
 // where B is MN-major.)  When there are more tiles than SMs, two CTAs share an
 // SM, three where K is short, so that one's epilogue overlaps another's loads;
-// else the stages fill the SM.
-void plan(int M, int N, int K, bool mnb, int nsm, int *bn, int *stages)
+// else the stages fill the SM.  A weight update's time is its epilogue's traffic
+// (26 bytes a weight): 64 columns and four CTAs an SM (128 registers) leave no
+// short last wave and keep more of it in flight.  256 rows into 8192 x 1024 x
+// 1024 x 4096: 245 -> 222 us the training step.
+void plan(int M, int N, int K, bool mnb, bool update, int nsm, int *bn, int *stages)
 {
     const long long mt = (M + kBM - 1) / kBM;
     long long best = 0, tiles = 0;
@@ -497,8 +501,12 @@ void plan(int M, int N, int K, bool mnb, int nsm, int *bn, int *stages)
             *bn = w;
         }
     }
+    if (update && *bn == 128) {
+        *bn = 64;
+        tiles = mt * ((N + 63) / 64);
+    }
     const int ktiles = (K + kBK - 1) / kBK, per = kTileA + tile_b(*bn);
-    int st = (tiles <= nsm ? 200 * 1024 : ktiles <= 8 ? 70 * 1024 : 104 * 1024) / per;
+    int st = (tiles <= nsm ? 200 * 1024 : update ? 50 * 1024 : ktiles <= 8 ? 70 * 1024 : 104 * 1024) / per;
     if (st > kMaxStages) st = kMaxStages;
     if (st > ktiles) st = ktiles;
     *stages = st < 2 ? 2 : st;
@@ -527,7 +535,7 @@ cudaError_t gemm_tc(int M, int N, int K, const GemmOperand &A, const GemmOperand
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    plan(M, N, K, !B.k_contiguous, nsm, &bn, &stages);
+    plan(M, N, K, !B.k_contiguous, E.kind == GEMM_ADAM, nsm, &bn, &stages);
     GemmEpilogue ep = E;
     // 16-byte accesses: every matrix (8 for the BF16 one) and row aligned for
     // them, and no row ending inside a group of four columns
