@@ -837,7 +837,8 @@ def main():
     # 138.84 MB and wrote 42.29 MB; traffic grows with the rows, so a full
     # 8192-row launch moves twice that.
     kname = (f"k_solver_row<{N}> (one CTA per row)" if sched == 16
-             else f"k_solver<{'XfPow2' if N & (N - 1) == 0 else 'XfBlue'}, {sched}> (cluster of {J // max(sched, 1)} CTAs)")
+             else f"k_solver_row<{N}> (a cluster of CTAs per row)" if sched == 64
+             else f"k_solver<{'XfPow2' if N & (N - 1) == 0 else 'XfComp or XfBlue'}, {sched}> (cluster of {J // max(sched, 1)} CTAs)")
     traffic, tbasis = None, "no capture of this kernel and workload"
     if (args.workload == "plain" and sched == 16 and args.precision == "fp32" and args.lanczos
             and args.power_iters == 16):
@@ -991,6 +992,7 @@ def main():
                            "l2": f"inputs larger than L2 (y is {M * J * N * 4 >> 20} MB)",
                            "parallelism": f"{world} independent TMs, one per GPU"},
                 "schedule": {"code": sched, "layout": "one CTA per row (16 points per thread)" if sched == 16
+                             else "a cluster of CTAs per row (16 points per thread)" if sched == 64
                              else f"{sched} masks per CTA, cluster of {J // max(sched, 1)} CTAs per row",
                              "autotuned": not args.schedule, "cuda_graph": True},
                 "fidelity": {"mean": float(fid.mean()), "p1": float(np.percentile(fid, 1)),
@@ -998,11 +1000,11 @@ def main():
                              "matrix_after_phase_fit": mfid},
                 "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk,
                 "to_fidelity_0.99": to099,
-                # kernels per timed step: k_solver, k_fields, k_row_energy,
-                # k_phase_fit, k_apply_phase (+ k_pack_f16 in mixed precision;
+                # kernels per timed step: k_solver, k_fields, k_phase_fit,
+                # k_apply_phase (+ k_pack_f16 in mixed precision;
                 # + k_prep_rows, k_prep_energy, k_prep_select, k_prep_zero and
                 # k_half_sample for the camera workload)
-                "gpu_launches": ((6 if args.precision == "mixed" else 5) + (5 if cam else 0)) * args.steps}
+                "gpu_launches": ((5 if args.precision == "mixed" else 4) + (5 if cam else 0)) * args.steps}
         if batching is not None:
             line["batching"] = batching
         if arms is not None:

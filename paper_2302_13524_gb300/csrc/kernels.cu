@@ -482,9 +482,9 @@ static cudaError_t dispatch_xf(int N, int prec, bool wide, F &&f)
 // in a transform's setup (two FP64 lanes a cycle and SM: it took most of a
 // short row), its bases come from the table.  Bound by shared-memory wavefronts
 // and issue slots of the transforms, not by HBM.  J = 4, one call before ->
-// after: forward N = 4096, M = 16384 1896 -> 628 us (1.7 GB moved: 2.6 TB/s);
-// gradient N = 2048, M = 8192 435 -> 288; forward N = 64, M = 128 5.1 -> 4.6
-// (launch).
+// after (the packed additions of fft.cuh included): forward N = 4096, M = 16384
+// 1896 -> 609 us (1.6 GB moved: 2.6 TB/s); gradient N = 2048, M = 8192 435 -> 266;
+// forward N = 64, M = 128 5.1 -> 4.7 (launch).
 //
 // CTAs per SM aimed at, as threads per SM, swept for the two kernels (forward,
 // gradient): register FFTs of 8 points 1024 and 640 (64 and 96 registers a

@@ -516,8 +516,8 @@ __host__ __device__ constexpr int comp_teams(int A)
 // J = 4: 2, 4, 8, 12, 18, 24, 32 teams take 70, 100, 190, 330, 550, 845, 1340 us;
 // L = 512, 1024, 2048, 4096, the split outputs and 8192 take 74, 163, 333, 770,
 // 940, 1460.  At N = 2286 (18 x 127), J = 4: gradient of 8192 rows 2556 us with
-// the split outputs and their FP64 setup, 2227 without the latter, 1681 so; a
-// retrieval of 2048 rows with early exit 54.1 -> 40.0 ms.
+// the split outputs and their FP64 setup, 2227 without the latter, 1681 so (1610
+// with packed additions); a retrieval of 2048 rows with early exit 54.1 -> 39.7 ms.
 __host__ __device__ inline bool comp_shape(int N, int *A, int *B)
 {
     const int most = N <= 256 ? 2 : N <= 512 ? 4 : N <= 1024 ? 12 : N <= 2048 ? 18 : N <= kBlueSplitMaxN ? 24 : 32;
