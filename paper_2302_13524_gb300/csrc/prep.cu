@@ -218,6 +218,7 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads)
         for (int p = tid; p < n; p += kSelThreads) key_s[p] = key[p];
         key = key_s;  // each thread reads back its own
     }
+    cluster.sync();  // every CTA of the cluster runs before anyone touches its shared memory
     // S8[j] <- the cluster's sum (or, with `largest`, maximum) of acc[j]; the two
     // part buffers alternate, so that a slow CTA may still read the last one
     int sel = 0;
