@@ -339,17 +339,19 @@ static __device__ void lbfgs_gram_update(Gram &Gm, int lane, int m, int it, int 
     const bool drop = accept && np + 1 > m;
     const int np2 = np + (accept ? 1 : 0) - (drop ? 1 : 0);
     if (accept && lane == 0) Gm.rD[ns] = 1.f / sy;
+    int moved = 0;
     if (drop) {
         const int s0 = sl[0];
 #pragma unroll
         for (int i = 0; i < kSlots; i++) sl[i] = i < m ? sl[i + 1] : s0;  // the m + 1 slots in use rotate
-        if (lane < kSlots && lane <= m) Gm.slot[lane] = lane < m ? Gm.slot[lane + 1] : s0;
+        moved = lane < m ? Gm.slot[lane + 1] : s0;
     }
     // status, when a row stops here: numeric trouble before convergence
     const float rel = fabsf(fold - fnew) / fmaxf(fold, 1e-30f);
     const bool numeric = !isfinite(fnew) || !isfinite(gg);
     const bool conv = (tol > 0.0 && rel < (float)tol) || (it + 1 < iters && (fnew == 0.f || gg == 0.f));
-    __syncwarp();
+    __syncwarp();  // every lane has read the slots, np and f that are written now
+    if (drop && lane <= m) Gm.slot[lane] = moved;
     if (lane == 0) {
         Gm.np = np2;
         Gm.gg = gg;
@@ -370,7 +372,7 @@ static __device__ void lbfgs_gram_update(Gram &Gm, int lane, int m, int it, int 
     bool ok = false;
     if (np2 > 0) {
         const int off = drop ? 1 : 0;
-        const int sn = Gm.slot[np2 - 1];  // the youngest pair
+        const int sn = accept ? ns : Gm.slot[np2 - 1];  // the youngest pair
         // three phases, each loading what it needs (a __syncwarp keeps the
         // compiler from holding both matrices in registers at once)
         float acc[kMaxMem], rd[kMaxMem], SY[kMaxMem][kMaxMem];
