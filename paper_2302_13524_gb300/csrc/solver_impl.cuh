@@ -82,9 +82,8 @@ constexpr int kIdxSS = 4 * kSlots, kIdxGG = 4 * kSlots + 1, kIdxF = 4 * kSlots +
 // moves nothing), and slot[np] is the free slot that receives the next pair.
 constexpr int kGramPitch = 8;  // kSlots rounded up: rows and coefficient vectors are 16-byte aligned
 struct __align__(16) Gram {
-    float SY[kSlots][kGramPitch];  // s_i^T y_j at [slot of i][slot of j], i no younger than j
+    float SY[kSlots][kGramPitch];  // s_i^T y_j at [slot of i][slot of j], i no younger than j; last column: 1 / s_i^T y_i
     float YY[kSlots][kGramPitch];  // y_i^T y_j
-    float rD[kGramPitch];          // 1 / s_i^T y_i by slot
     float c1[kGramPitch], c2[kGramPitch];  // direction coefficients by age (c2 includes gamma)
     float red[kParts];  // the last cluster-wide sums
     int slot[kGramPitch];
@@ -93,6 +92,12 @@ struct __align__(16) Gram {
     int np;
     int status, done, stop, early, row;
 };
+// What a row's state counts for it: which (N, J, m) fit an SM hangs on this
+// figure, and problems of several lengths fill the shared memory to the last 16
+// bytes, so it stays as it is, and k_solver has no static shared memory beside
+// its dynamic request.
+constexpr size_t kGramBytes = 740;
+static_assert(sizeof(Gram) <= kGramBytes, "the scalars take shared memory from problems that fit");
 
 // Global minimiser of phi(a) = c0 + c1 a + c2 a^2 + c3 a^3 + c4 a^4 (c4 > 0)
 // over the real line.  phi' = g(a) = c1 + 2 c2 a + 3 c3 a^2 + 4 c4 a^3 rises at
@@ -338,7 +343,7 @@ static __device__ void lbfgs_gram_update(Gram &Gm, int lane, int m, int it, int 
     const bool accept = sy > 1e-10f * sqrtf(tot[kIdxSS]) * sqrtf(yy) && sy > 0.f;
     const bool drop = accept && np + 1 > m;
     const int np2 = np + (accept ? 1 : 0) - (drop ? 1 : 0);
-    if (accept && lane == 0) Gm.rD[ns] = 1.f / sy;
+    if (accept && lane == 0) Gm.SY[ns][kSlots] = 1.f / sy;
     int moved = 0;
     if (drop) {
         const int s0 = sl[0];
@@ -380,7 +385,7 @@ static __device__ void lbfgs_gram_update(Gram &Gm, int lane, int m, int it, int 
         for (int i = 0; i < kMaxMem; i++) {
             const bool in = i < np2;
             acc[i] = in ? -tot[4 * (i + off) + 2] : 0.f;
-            rd[i] = in ? Gm.rD[sl[i]] : 0.f;
+            rd[i] = in ? Gm.SY[sl[i]][kSlots] : 0.f;
 #pragma unroll
             for (int j = i; j < kMaxMem; j++) SY[i][j] = j < np2 ? Gm.SY[sl[i]][sl[j]] : 0.f;
         }
@@ -498,7 +503,7 @@ __host__ __device__ size_t solver_smem(int N, int J, int m)
     size_t bytes = f2 * sizeof(float2) + 2 * (size_t)(m + 1) * SL * sizeof(SolverHist<Xf>) /*pairs*/;
     bytes += sizeof(float) * ((size_t)kParts * C::NW + 2 * (size_t)JC * kParts);
     bytes = (bytes + 15) & ~(size_t)15;
-    return bytes + sizeof(Gram);
+    return bytes + kGramBytes;
 }
 
 // CTAs per SM to leave registers for: 128 a thread for the composite lengths,
@@ -566,19 +571,13 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, solver_min_ctas<Xf, G>()
         for (int e = 0; e < E; e++) x[e] = valid(e) ? X[vi(e)] : make_float2(0.f, 0.f);
     };
     const int sl_shift = (even && (SL & (SL - 1)) == 0) ? __ffs(SL) - 1 : -1;
-    // the CTA that owns element n; for uneven slices by counting the slice
-    // starts at or below n (a 64-bit division here cost more than the
-    // exchange itself: 4000 cycles an iteration at N = 2286)
-    __shared__ int slice0[kMaxMasks];  // first element of each CTA's slice
-    auto owner = [&](int n) {
-        if (sl_shift >= 0) return n >> sl_shift;
-        int o = 0;
-#pragma unroll
-        for (int r = 1; r < kMaxMasks; r++) o += r < JC && n >= slice0[r];
-        return o;
-    };
-    if (tid < JC) slice0[tid] = (tid * N) / JC;
-    __syncthreads();
+    // the CTA that owns element n and its slice's first element; for uneven
+    // slices, which start at floor(o N / JC), o = floor(((n + 1) JC - 1) / N), both
+    // by FP32 products with a half added, exact for these sizes (a 64-bit division
+    // here cost more than the exchange itself: 4000 cycles an iteration at N = 2286)
+    const float jc_n = (float)JC / (float)N, n_jc = (float)N / (float)JC, half_jc = 0.5f / (float)JC;
+    auto owner = [&](int n) { return sl_shift >= 0 ? n >> sl_shift : (int)(((float)n + 1.f - half_jc) * jc_n); };
+    auto slice0 = [&](int o) { return sl_shift >= 0 ? o << sl_shift : (int)((float)o * n_jc + half_jc); };
     cluster.sync();  // every CTA of the cluster runs before anyone touches its shared memory
 
     // Cluster-wide sums of nv <= 32 per-thread values (v padded with zeros):
@@ -638,7 +637,7 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, solver_min_ctas<Xf, G>()
             if (!valid(e)) continue;
             const int n = vi(e);
             const int o = owner(n);
-            cluster.map_shared_rank(Yr, o)[jm * SL + (n - slice0[o])] = v[e];
+            cluster.map_shared_rank(Yr, o)[jm * SL + (n - slice0(o))] = v[e];
         }
     };
     // element i of my slice of sum_j Y[j], times s

@@ -82,7 +82,7 @@ __host__ __device__ size_t rowc_smem(int J)
     size_t bytes = f2 * sizeof(float2) +
                    sizeof(float) * ((size_t)JB * N /*y*/ + (size_t)kParts * NW + 2 * (size_t)JC * kParts);
     bytes = (bytes + 15) & ~(size_t)15;
-    return bytes + sizeof(Gram);
+    return bytes + kGramBytes;
 }
 
 template <int N>
@@ -95,7 +95,7 @@ __host__ __device__ size_t row_smem(int J, int m)
                 (size_t)J * C::LBUF /*team exchange buffers*/ + 3 * (size_t)N /*p, t, g*/;
     size_t bytes = f2 * sizeof(float2) + sizeof(float) * ((size_t)J * N /*y*/ + (size_t)kParts * (NW > 0 ? NW : 1));
     bytes = (bytes + 15) & ~(size_t)15;
-    return bytes + sizeof(Gram);
+    return bytes + kGramBytes;
 }
 
 // Tensor-memory columns of one CTA.  Thread tid owns elements tid + e BT,
