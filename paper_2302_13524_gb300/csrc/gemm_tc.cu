@@ -52,9 +52,16 @@ constexpr int kBM = 128, kBK = 64, kMaxStages = 10;
 constexpr int kTileA = kBM * kBK * 2;  // bytes per stage
 __host__ __device__ constexpr int tile_b(int bn) { return bn * kBK * 2; }
 constexpr long long kSpinLimit = 1LL << 22;  // polls of a barrier wait (about 0.1 - 1 s)
-size_t smem_bytes(int bn, int stages)
+constexpr int kStageBytes = 200 * 1024;      // of all stages together, at most
+constexpr size_t smem_bytes(int bn, int stages)
 {
     return 1024 /*alignment slack*/ + (size_t)stages * (kTileA + tile_b(bn)) + 256;
+}
+// the most a plan of this tile width asks for
+constexpr size_t smem_most(int bn)
+{
+    const int st = kStageBytes / (kTileA + tile_b(bn));
+    return smem_bytes(bn, st < kMaxStages ? st : kMaxStages);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
@@ -506,7 +513,7 @@ void plan(int M, int N, int K, bool mnb, bool update, int nsm, int *bn, int *sta
         tiles = mt * ((N + 63) / 64);
     }
     const int ktiles = (K + kBK - 1) / kBK, per = kTileA + tile_b(*bn);
-    int st = (tiles <= nsm ? 200 * 1024 : update ? 50 * 1024 : ktiles <= 8 ? 70 * 1024 : 104 * 1024) / per;
+    int st = (tiles <= nsm ? kStageBytes : update ? 50 * 1024 : ktiles <= 8 ? 70 * 1024 : 104 * 1024) / per;
     if (st > kMaxStages) st = kMaxStages;
     if (st > ktiles) st = ktiles;
     *stages = st < 2 ? 2 : st;
@@ -517,8 +524,10 @@ cudaError_t launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, i
                    const GemmEpilogue &E, int *err, cudaStream_t s)
 {
     const size_t sm = smem_bytes(BN, stages);
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_gemm_tc<BN, MNA, MNB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // the limit belongs to the kernel, not to this launch: always the same value,
+    // or another thread's shape could lower it between here and the launch
+    const cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<BN, MNA, MNB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem_most(BN));
     if (e != cudaSuccess) return e;
     dim3 grid((N + BN - 1) / BN, (M + kBM - 1) / kBM);
     k_gemm_tc<BN, MNA, MNB><<<grid, 128, sm, s>>>(ma, mb, M, N, K, stages, ldc, E, err);
