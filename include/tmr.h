@@ -148,6 +148,9 @@ typedef struct {
                                32 = for 2048 < N <= 2731, one mask per CTA with the
                                full-length Bluestein plan (FFTs of L = 8192) instead
                                of the split outputs at L = 4096 of schedule 1;
+                               64 = the layout of 16 over a cluster of CTAs per row
+                               (FP32, intensity cost, N = 4096 with J = 4, 6 or 8 or
+                               N = 2048 with J = 6 or 8);
                                0 = chosen by the autotuner (default)                 */
     const char *tune_cache; /* JSON file caching autotuned schedules per device, N, J,
                                m; NULL = this process only                           */
@@ -369,9 +372,9 @@ long long tmr_learned_rows(tmr_handle *h);
 
 /* The solver schedule the handle uses (after autotuning): 1, 2 or 4 masks per
  * CTA, 16 for one CTA per row, 32 for the full-length Bluestein plan, 64 for the
- * layout of 16 over a cluster of CTAs per row (rows too large for one CTA;
- * chosen by the autotuner, not by opt.schedule); 0 for a NULL handle or when no
- * schedule fits (see tmr_create). */
+ * layout of 16 over a cluster of CTAs per row (rows too large for one CTA); 0 for
+ * a NULL handle or when no schedule fits (see tmr_create).  Every other code it
+ * returns can be given back as opt.schedule for the same problem. */
 int tmr_schedule(const tmr_handle *h);
 /* The schedules the autotuner timed when this handle was made, and the mean
  * time of their timed runs in milliseconds (each: 4 power and 6 L-BFGS

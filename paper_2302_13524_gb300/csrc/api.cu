@@ -508,11 +508,10 @@ tmr_status tmr_create(tmr_handle **out, int N, int M, int J, const void *masks,
     TMR_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), "attr");
     if (o.cost == TMR_COST_AMPLITUDE && xk != 0 && xk != 3)
         return fail(TMR_ERR_UNSUPPORTED, "the amplitude cost runs on the FP32 1D transforms (precision FP32, probe_n1 0)");
-    if (o.schedule != 0 &&
-        (o.schedule == kRowClusterSchedule || !schedule_ok(N, J, o.m, o.schedule, smem_optin, xk, o.cost)))
+    if (o.schedule != 0 && !schedule_ok(N, J, o.m, o.schedule, smem_optin, xk, o.cost))
         return fail(TMR_ERR_UNSUPPORTED,
-                    "opt.schedule must be 1, 2 or 4 (dividing J), 16 (one CTA per row) or 32 (full-length "
-                    "Bluestein), and fit the device");
+                    "opt.schedule must be 1, 2 or 4 (dividing J), 16 (one CTA per row), 64 (that layout over a "
+                    "cluster) or 32 (full-length Bluestein), and fit the device");
 
     tmr_handle *h = new tmr_handle();
     h->N = N;

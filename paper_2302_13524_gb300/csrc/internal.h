@@ -107,7 +107,7 @@ struct SolverParams {
 constexpr int kRowSchedule = 16;
 // G = kRowClusterSchedule (64): the same layout over a cluster of CTAs holding
 // two or more masks each, for rows too large for one CTA: N = 4096 with J = 4,
-// 6 or 8, N = 2048 with J = 6 or 8, intensity cost.  Chosen by the autotuner only.
+// 6 or 8, N = 2048 with J = 6 or 8, intensity cost.
 constexpr int kRowClusterSchedule = 64;
 int solver_rowc_masks(int N, int J);  // masks per CTA, 0: no such variant
 size_t solver_rowc_smem(int N, int J, int m);  // more than any SM has where the row's state does not fit

@@ -105,7 +105,7 @@ class Retriever:
 
     @property
     def schedule(self) -> int:
-        """Masks per CTA of the solver schedule in use (0: none fits)."""
+        """Code of the solver schedule in use, as for the option of that name (0: none fits)."""
         return _lib.tmr_schedule(self.h)
 
     def close(self):
