@@ -1,7 +1,7 @@
 // gemm_tc.cu -- BF16 x BF16 -> FP32 GEMM on the fifth-generation tensor cores
 // (tcgen05.mma, accumulators in tensor memory), fed by TMA.  It computes the
 // products of the learned initialiser's network (mlp.cu) where the shapes
-// allow (row lengths a multiple of 8 elements, 16-byte aligned rows).
+// allow (at least 128 x 128 x 64, 16-byte aligned rows).
 //
 //   C[M][N] (FP32, row stride ldc) = sum_k A(m, k) B(n, k).  Each operand is
 //   stored either K-contiguous (A [M][K], B [N][K]) or K-strided (A [K][M],
@@ -228,6 +228,7 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
     for (int r0 = lane >> 3; r0 < 32; r0 += 16) {
         float4 x[4];
         size_t o[4];
+        __nv_bfloat16 *h[4];
         bool in[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) {
@@ -235,6 +236,7 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
             x[i] = make_float4(p[0], p[1], p[2], p[3]);
             in[i] = row0 + r0 + 4 * i < M;
             o[i] = (size_t)(row0 + r0 + 4 * i) * ldc + col;
+            h[i] = E.H + (size_t)(row0 + r0 + 4 * i) * E.ldh + col;
         }
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
         switch (E.kind) {
@@ -246,7 +248,7 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
                 if (!in[i]) continue;
                 st4<V>(E.C + o[i], z, n);
                 if (E.kind == GEMM_BIAS_GELU)
-                    st4<V>(E.H + o[i], make_float4(gelu_f(z.x), gelu_f(z.y), gelu_f(z.z), gelu_f(z.w)), n);
+                    st4<V>(h[i], make_float4(gelu_f(z.x), gelu_f(z.y), gelu_f(z.z), gelu_f(z.w)), n);
             }
             break;
         case GEMM_GELU_BACK: {
@@ -256,7 +258,7 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
 #pragma unroll
             for (int i = 0; i < 4; i++)
                 if (in[i])
-                    st4<V>(E.H + o[i],
+                    st4<V>(h[i],
                            make_float4(x[i].x * gelu_grad_f(z[i].x), x[i].y * gelu_grad_f(z[i].y),
                                        x[i].z * gelu_grad_f(z[i].z), x[i].w * gelu_grad_f(z[i].w)),
                            n);
@@ -280,7 +282,7 @@ __device__ __forceinline__ void epilogue_block(const GemmEpilogue &E, const floa
                 st4<V>(E.w + o[i], w[i], n);
                 st4<V>(E.m + o[i], m[i], n);
                 st4<V>(E.v + o[i], v[i], n);
-                st4<V>(E.H + o[i], w[i], n);
+                st4<V>(h[i], w[i], n);
             }
             break;
         }
@@ -476,9 +478,9 @@ bool make_map(CUtensorMap *map, const __nv_bfloat16 *ptr, int rows, int cols, in
 bool gemm_tc_supported(int M, int N, int K, const GemmOperand &A, const GemmOperand &B)
 {
     if (M < kBM || N < 128 || K < kBK) return false;
-    // 16-byte rows and strides: the contiguous dimension and the row stride of each operand
+    // rows that start on 16-byte boundaries (their length may be any: TMA fills what is past it)
     const int ca = A.k_contiguous ? K : M, cb = B.k_contiguous ? K : N;
-    if (ca % 8 || cb % 8 || A.ld % 8 || B.ld % 8 || A.ld < ca || B.ld < cb) return false;
+    if (A.ld % 8 || B.ld % 8 || A.ld < ca || B.ld < cb) return false;
     if ((reinterpret_cast<uintptr_t>(A.p) & 15) || (reinterpret_cast<uintptr_t>(B.p) & 15)) return false;
     return encode_fn() != nullptr;
 }
@@ -548,7 +550,7 @@ cudaError_t gemm_tc(int M, int N, int K, const GemmOperand &A, const GemmOperand
     GemmEpilogue ep = E;
     // 16-byte accesses: every matrix (8 for the BF16 one) and row aligned for
     // them, and no row ending inside a group of four columns
-    ep.wide = N % 4 == 0 && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(E.H) & 7) == 0;
+    ep.wide = N % 4 == 0 && ldc % 4 == 0 && ep.ldh % 4 == 0 && (reinterpret_cast<uintptr_t>(E.H) & 7) == 0;
     for (const float *p : {(const float *)E.C, E.bias, E.Z, (const float *)E.w, (const float *)E.m, (const float *)E.v})
         ep.wide = ep.wide && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
     CUtensorMap ma, mb;
@@ -582,7 +584,7 @@ extern "C" tmr_status tmr_gemm_bf16(int M, int N, int K, const void *A, int lda,
     const tmr::GemmOperand oa{(const __nv_bfloat16 *)A, lda, true}, ob{(const __nv_bfloat16 *)B, ldb, true};
     tmr::GemmEpilogue ep{};
     ep.C = C;
-    if (!tmr::gemm_tc_supported(M, N, K, oa, ob)) {
+    if (K % 8 || !tmr::gemm_tc_supported(M, N, K, oa, ob)) {
         tmr::set_last_error("tmr_gemm_bf16: needs M, N >= 128, K >= 64, K, lda, ldb multiples of 8, 16-byte alignment");
         return TMR_ERR_UNSUPPORTED;
     }

@@ -162,15 +162,16 @@ cudaError_t launch_fill_synthetic(float *y, size_t n, unsigned seed, cudaStream_
 // ---- BF16 tensor-core GEMM (gemm_tc.cu) ---------------------------------------
 // C[M][N] (FP32, row stride ldc) = sum_k A(m, k) B(n, k), then an elementwise
 // step.  An operand is BF16 with rows of stride ld elements: [M or N][K]
-// (k_contiguous) or [K][M or N].  Needs M, N >= 128, K >= 64, the contiguous
-// dimension and ld of each multiples of 8 and 16-byte aligned pointers; *err
-// (device) is raised when a barrier wait ran out.
+// (k_contiguous) or [K][M or N].  Needs M, N >= 128, K >= 64, 16-byte aligned
+// pointers and rows (ld a multiple of 8, no shorter than the row); *err (device)
+// is raised when a barrier wait ran out.
 struct GemmOperand {
     const __nv_bfloat16 *p;
     int ld;
     bool k_contiguous;
 };
-// What becomes of the product x at (row, col); every matrix has row stride ldc.
+// What becomes of the product x at (row, col); every matrix has row stride ldc,
+// the BF16 one ldh.
 //   GEMM_STORE      C = x
 //   GEMM_BIAS       C = x + bias[col]
 //   GEMM_BIAS_GELU  C = x + bias[col], H = GELU(C)
@@ -182,6 +183,7 @@ struct GemmEpilogue {
     float *C = nullptr;
     const float *bias = nullptr, *Z = nullptr;
     __nv_bfloat16 *H = nullptr;
+    int ldh = 0;
     float *w = nullptr, *m = nullptr, *v = nullptr;
     float lr = 0.f, c1 = 1.f, c2 = 1.f;  // step size and bias corrections
     bool wide = false;  // set by gemm_tc: 16-byte accesses are aligned

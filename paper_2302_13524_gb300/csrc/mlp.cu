@@ -10,7 +10,9 @@
 // products X W^T, the input gradients dZ W and the weight gradients dZ^T H run
 // on the tensor cores with the layer's elementwise step as their epilogue
 // (gemm_tc.cu); this file's mma.sync kernel, through generic element strides,
-// takes the shapes that does not.
+// takes the shapes that does not.  Rows of the BF16 matrices are padded to 16
+// bytes (row_ld), which is what the tensor-core path asks of its operands, so that
+// layers of any width take it.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -29,6 +31,10 @@ namespace tmr {
 // B(k, n) = B[k sbk + n sbn] in BF16.  64 x 64 tile per CTA, 4 warps of 32 x 32,
 // K in steps of 32 through shared memory; out-of-range elements read as zero.
 constexpr int GB_M = 64, GB_N = 64, GB_K = 32, GB_PAD = 8;
+
+// Row stride of a BF16 matrix with n columns: 16-byte aligned rows.  The padding
+// is zeroed where the matrix is allocated and never written.
+__host__ __device__ constexpr int row_ld(int n) { return (n + 7) & ~7; }
 
 __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi)
 {
@@ -120,14 +126,34 @@ static void gemm_sync(int M, int N, int K, const __nv_bfloat16 *A, long long sam
     k_gemm_bf16<<<grid, 128, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, N);
 }
 
-// Z += b (per column); H = GELU(Z) in BF16 (gelu != 0) or Z itself copied to out.
-__global__ void k_bias_act(int B, int N, float *Z, const float *b, __nv_bfloat16 *H, int gelu)
+// A thread's elements of a matrix of n columns, row after row, without a division
+// for each (64-bit ones take longer than the element's work).
+struct RowWalk {
+    size_t i, r, step, dr;
+    int n, c, dc;
+    __device__ RowWalk(int cols)
+    {
+        n = cols;
+        i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+        step = (size_t)gridDim.x * blockDim.x;
+        r = i / n, c = (int)(i - r * n);
+        dr = step / n, dc = (int)(step - dr * n);
+    }
+    __device__ void next()
+    {
+        i += step, r += dr, c += dc;
+        if (c >= n) c -= n, r++;
+    }
+};
+
+// Z += b (per column); H (row stride ldh) = GELU(Z) in BF16 (gelu != 0) or Z itself copied to out.
+__global__ void k_bias_act(int B, int N, float *Z, const float *b, __nv_bfloat16 *H, int ldh, int gelu)
 {
     const size_t total = (size_t)B * N;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const float z = Z[i] + b[i % N];
-        Z[i] = z;
-        if (H) H[i] = __float2bfloat16(gelu ? gelu_f(z) : z);
+    for (RowWalk w(N); w.i < total; w.next()) {
+        const float z = Z[w.i] + b[w.c];
+        Z[w.i] = z;
+        if (H) H[w.r * ldh + w.c] = __float2bfloat16(gelu ? gelu_f(z) : z);
     }
 }
 
@@ -141,6 +167,7 @@ __global__ void __launch_bounds__(256) k_loss_rows(int B, int N, int phase, cons
 {
     const size_t o = (size_t)blockIdx.x * N;
     const float *y = Y + o, *t = T + o;
+    __nv_bfloat16 *dy = dY + (size_t)blockIdx.x * row_ld(N);
     __shared__ float red[64], res[2];
     const float sc = 2.f / (float)((size_t)B * N);
     float acc = 0.f;
@@ -163,15 +190,15 @@ __global__ void __launch_bounds__(256) k_loss_rows(int B, int N, int phase, cons
             const float e0 = y[k] - (tr * rr - ti * ri), e1 = y[n + k] - (tr * ri + ti * rr);
             acc = fmaf(e0, e0, acc);
             acc = fmaf(e1, e1, acc);
-            dY[o + k] = __float2bfloat16(sc * e0);
-            dY[o + n + k] = __float2bfloat16(sc * e1);
+            dy[k] = __float2bfloat16(sc * e0);
+            dy[n + k] = __float2bfloat16(sc * e1);
         }
     } else {
 #pragma unroll 4
         for (int k = threadIdx.x; k < N; k += blockDim.x) {
             const float e = y[k] - t[k];
             acc = fmaf(e, e, acc);
-            dY[o + k] = __float2bfloat16(sc * e);
+            dy[k] = __float2bfloat16(sc * e);
         }
     }
     __syncthreads();  // res is read before red and res are used again
@@ -192,15 +219,16 @@ __global__ void __launch_bounds__(256) k_loss_finish(int nparts, const float *pa
     if (threadIdx.x == 0) *loss = (float)(out[0] / total);
 }
 
-// dZ = dH .* GELU'(Z) -> BF16
-__global__ void k_gelu_back(size_t n, const float *dH, const float *Z, __nv_bfloat16 *dZ)
+// dZ = dH .* GELU'(Z) -> BF16 (row stride ldz)
+__global__ void k_gelu_back(int B, int N, const float *dH, const float *Z, __nv_bfloat16 *dZ, int ldz)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dZ[i] = __float2bfloat16(dH[i] * gelu_grad_f(Z[i]));
+    const size_t n = (size_t)B * N;
+    for (RowWalk w(N); w.i < n; w.next())
+        dZ[w.r * ldz + w.c] = __float2bfloat16(dH[w.i] * gelu_grad_f(Z[w.i]));
 }
 
 // Bias gradients of the three layers in one launch: g[c] = sum_r dZ[r][c] (dZ
-// BF16 [B][N]), and with adam != 0 the biases' Adam update instead of storing
+// BF16, rows of N), and with adam != 0 the biases' Adam update instead of storing
 // it.  A block of 32 x 8 threads takes 32 columns of one layer, thread (c, r)
 // the rows r, r + 8, ...  (One thread per column, walking all rows, used 16
 // blocks of the chip for 20 us a layer.)
@@ -208,7 +236,6 @@ struct BiasLayer {
     const __nv_bfloat16 *dZ;
     int N, block0;  // columns; first block of the layer
     float *g, *w, *m, *v;
-    __nv_bfloat16 *wb;
 };
 struct BiasLayers {
     BiasLayer l[3];
@@ -222,7 +249,7 @@ __global__ void __launch_bounds__(256) k_bias_grad(int B, const __grid_constant_
     float s = 0.f;
     if (c < L.N) {
 #pragma unroll 8
-        for (int r = threadIdx.y; r < B; r += 8) s += __bfloat162float(L.dZ[(size_t)r * L.N + c]);
+        for (int r = threadIdx.y; r < B; r += 8) s += __bfloat162float(L.dZ[(size_t)r * row_ld(L.N) + c]);
     }
     red[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
@@ -238,7 +265,6 @@ __global__ void __launch_bounds__(256) k_bias_grad(int B, const __grid_constant_
     L.w[c] = w;
     L.m[c] = m;
     L.v[c] = v;
-    L.wb[c] = __float2bfloat16(w);
 }
 
 // x -> BF16, four values a thread and step where both are aligned for it
@@ -259,21 +285,30 @@ __global__ void k_to_bf16(size_t n, const float *x, __nv_bfloat16 *y)
     }
     for (size_t i = done + t0; i < n; i += step) y[i] = __float2bfloat16(x[i]);
 }
-
-__global__ void k_adam(size_t n, float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, float lr,
-                       float c1, float c2)
+// the same of rows of n values into rows of stride ld
+__global__ void k_rows_to_bf16(int rows, int n, const float *x, __nv_bfloat16 *y, int ld)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t total = (size_t)rows * n;
+    for (RowWalk w(n); w.i < total; w.next()) y[w.r * ld + w.c] = __float2bfloat16(x[w.i]);
+}
+
+// wb: the weights' BF16 copy, row stride ldw
+__global__ void k_adam(int rows, int cols, float *w, const float *g, float *m, float *v, __nv_bfloat16 *wb, int ldw,
+                       float lr, float c1, float c2)
+{
+    const size_t n = (size_t)rows * cols;
+    for (RowWalk k(cols); k.i < n; k.next()) {
+        const size_t i = k.i;
         float wi = w[i], mi = m[i], vi = v[i];
         adam_update(wi, g[i], mi, vi, lr, c1, c2);
         m[i] = mi;
         v[i] = vi;
         w[i] = wi;
-        wb[i] = __float2bfloat16(wi);
+        wb[k.r * ldw + k.c] = __float2bfloat16(wi);
     }
 }
 
-// y = normalised sqrt intensities: x[r][i] = sqrt(max(y, 0)) / sqrt(mean_i y[r][i]) (BF16)
+// y = normalised sqrt intensities: x[r][i] = sqrt(max(y, 0)) / sqrt(mean_i y[r][i]) (BF16, padded rows)
 __global__ void k_features(int K, const float *y, __nv_bfloat16 *x)
 {
     const int r = blockIdx.x;
@@ -285,7 +320,7 @@ __global__ void k_features(int K, const float *y, __nv_bfloat16 *x)
     block_sum<1>(v, red, out);
     const float inv = out[0] > 0.f ? rsqrtf(out[0] / (float)K) : 0.f;
     for (int i = threadIdx.x; i < K; i += blockDim.x)
-        x[(size_t)r * K + i] = __float2bfloat16(sqrtf(fmaxf(yr[i], 0.f)) * inv);
+        x[(size_t)r * row_ld(K) + i] = __float2bfloat16(sqrtf(fmaxf(yr[i], 0.f)) * inv);
 }
 
 // candidate start: t[n] = (out[n] + i out[N + n]) scaled to ||t||^2 = sum(y) / (J N)
@@ -312,10 +347,11 @@ using namespace tmr;
 struct tmr_mlp {
     int n_in, h1, h2, n_out;
     size_t np;  // parameters
-    size_t off[6];
+    size_t off[6];   // each layer's weights and biases among them
+    size_t woff[3];  // the layers' weights in wb
     cudaStream_t stream;
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr;
-    __nv_bfloat16 *wb = nullptr;
+    __nv_bfloat16 *wb = nullptr;  // the weights in BF16, padded rows
     long long step = 0;
     // batch scratch
     int cap = 0;
@@ -354,9 +390,9 @@ void gemm(tmr_mlp *m, int M, int N, int K, const GemmOperand &A, const GemmOpera
     const int nb = ew_blocks(n);
     switch (E.kind) {
     case GEMM_BIAS:
-    case GEMM_BIAS_GELU: k_bias_act<<<nb, 256, 0, s>>>(M, N, E.C, E.bias, E.H, E.kind == GEMM_BIAS_GELU); break;
-    case GEMM_GELU_BACK: k_gelu_back<<<nb, 256, 0, s>>>(n, E.C, E.Z, E.H); break;
-    case GEMM_ADAM: k_adam<<<nb, 256, 0, s>>>(n, E.w, E.C, E.m, E.v, E.H, E.lr, E.c1, E.c2); break;
+    case GEMM_BIAS_GELU: k_bias_act<<<nb, 256, 0, s>>>(M, N, E.C, E.bias, E.H, E.ldh, E.kind == GEMM_BIAS_GELU); break;
+    case GEMM_GELU_BACK: k_gelu_back<<<nb, 256, 0, s>>>(M, N, E.C, E.Z, E.H, E.ldh); break;
+    case GEMM_ADAM: k_adam<<<nb, 256, 0, s>>>(M, N, E.w, E.C, E.m, E.v, E.H, E.ldh, E.lr, E.c1, E.c2); break;
     default: break;
     }
 }
@@ -365,6 +401,14 @@ int ew_blocks(size_t n)
 {
     size_t b = (n + 255) / 256;
     return (int)(b > 152 * 8 ? 152 * 8 : (b < 1 ? 1 : b));
+}
+
+// rows x n values to BF16, padded rows
+void to_bf16(int rows, int n, const float *x, __nv_bfloat16 *y, cudaStream_t s)
+{
+    const size_t total = (size_t)rows * n;
+    if (row_ld(n) == n) k_to_bf16<<<ew_blocks(total), 256, 0, s>>>(total, x, y);
+    else k_rows_to_bf16<<<ew_blocks(total), 256, 0, s>>>(rows, n, x, y, row_ld(n));
 }
 
 tmr_status ensure_batch(tmr_mlp *m, int B)
@@ -378,20 +422,21 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
             cudaFree(*b);
             *b = nullptr;
         }
-    const size_t big = (size_t)B * (m->n_in > m->n_out ? m->n_in : m->n_out);
-    const size_t hid = (size_t)B * (m->h1 > m->h2 ? m->h1 : m->h2);
-    const size_t hmax = big > hid ? big : hid;
-    bool ok = cudaMalloc(&m->xb, sizeof(__nv_bfloat16) * (size_t)B * m->n_in) == cudaSuccess &&
-              cudaMalloc(&m->h1b, sizeof(__nv_bfloat16) * (size_t)B * m->h1) == cudaSuccess &&
-              cudaMalloc(&m->h2b, sizeof(__nv_bfloat16) * (size_t)B * m->h2) == cudaSuccess &&
-              cudaMalloc(&m->dzb, sizeof(__nv_bfloat16) * hmax) == cudaSuccess &&
-              cudaMalloc(&m->dz2b, sizeof(__nv_bfloat16) * hmax) == cudaSuccess &&
-              cudaMalloc(&m->dyb, sizeof(__nv_bfloat16) * (size_t)B * m->n_out) == cudaSuccess &&
-              cudaMalloc(&m->z1, sizeof(float) * (size_t)B * m->h1) == cudaSuccess &&
-              cudaMalloc(&m->z2, sizeof(float) * (size_t)B * m->h2) == cudaSuccess &&
-              cudaMalloc(&m->y, sizeof(float) * (size_t)B * m->n_out) == cudaSuccess &&
-              cudaMalloc(&m->dh, sizeof(float) * hmax) == cudaSuccess &&
-              cudaMalloc(&m->part, sizeof(float) * (size_t)B) == cudaSuccess;
+    const int hid = m->h1 > m->h2 ? m->h1 : m->h2, io = m->n_in > m->n_out ? m->n_in : m->n_out;
+    const int hmax = io > hid ? io : hid;
+    const size_t rows = (size_t)B;
+    auto padded = [&](__nv_bfloat16 **p, int width) {
+        const size_t bytes = sizeof(__nv_bfloat16) * rows * row_ld(width);
+        return cudaMalloc(p, bytes) == cudaSuccess && cudaMemsetAsync(*p, 0, bytes, m->stream) == cudaSuccess;
+    };
+    bool ok = padded(&m->xb, m->n_in) && padded(&m->h1b, m->h1) && padded(&m->h2b, m->h2) && padded(&m->dzb, m->h1) &&
+              padded(&m->dz2b, m->h2) && padded(&m->dyb, m->n_out) &&
+              cudaMalloc(&m->z1, sizeof(float) * rows * m->h1) == cudaSuccess &&
+              cudaMalloc(&m->z2, sizeof(float) * rows * m->h2) == cudaSuccess &&
+              cudaMalloc(&m->y, sizeof(float) * rows * m->n_out) == cudaSuccess &&
+              cudaMalloc(&m->dh, sizeof(float) * rows * hmax) == cudaSuccess &&
+              cudaMalloc(&m->part, sizeof(float) * rows) == cudaSuccess &&
+              cudaStreamSynchronize(m->stream) == cudaSuccess;  // mlp_propose goes on on another stream
     if (!ok) {
         cudaGetLastError();
         return mfail(TMR_ERR_OOM, "MLP batch buffers");
@@ -400,24 +445,26 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
     return TMR_OK;
 }
 
-GemmEpilogue bias_step(float *z, const float *bias, __nv_bfloat16 *h)
+GemmEpilogue bias_step(float *z, const float *bias, __nv_bfloat16 *h, int ldh)
 {
     GemmEpilogue E;
     E.kind = h ? GEMM_BIAS_GELU : GEMM_BIAS;
     E.C = z;
     E.bias = bias;
     E.H = h;
+    E.ldh = ldh;
     return E;
 }
 
 // forward from BF16 features m->xb into y (FP32 [B][out]); keeps Z1, Z2, H1, H2
 void forward_core(tmr_mlp *m, int B, float *y)
 {
-    const __nv_bfloat16 *W1 = m->wb + m->off[0], *W2 = m->wb + m->off[2], *W3 = m->wb + m->off[4];
+    const __nv_bfloat16 *W1 = m->wb + m->woff[0], *W2 = m->wb + m->woff[1], *W3 = m->wb + m->woff[2];
     const float *b1 = m->w + m->off[1], *b2 = m->w + m->off[3], *b3 = m->w + m->off[5];
-    gemm(m, B, m->h1, m->n_in, {m->xb, m->n_in, true}, {W1, m->n_in, true}, bias_step(m->z1, b1, m->h1b));
-    gemm(m, B, m->h2, m->h1, {m->h1b, m->h1, true}, {W2, m->h1, true}, bias_step(m->z2, b2, m->h2b));
-    gemm(m, B, m->n_out, m->h2, {m->h2b, m->h2, true}, {W3, m->h2, true}, bias_step(y, b3, nullptr));
+    const int li = row_ld(m->n_in), l1 = row_ld(m->h1), l2 = row_ld(m->h2);
+    gemm(m, B, m->h1, m->n_in, {m->xb, li, true}, {W1, li, true}, bias_step(m->z1, b1, m->h1b, l1));
+    gemm(m, B, m->h2, m->h1, {m->h1b, l1, true}, {W2, l1, true}, bias_step(m->z2, b2, m->h2b, l2));
+    gemm(m, B, m->n_out, m->h2, {m->h2b, l2, true}, {W3, l2, true}, bias_step(y, b3, nullptr, 0));
 }
 
 // One Adam step's size and bias corrections
@@ -430,20 +477,23 @@ struct AdamStep {
 void backward_core(tmr_mlp *m, int B, const float *T, float *loss, float *g, const AdamStep *step)
 {
     cudaStream_t s = m->stream;
-    const __nv_bfloat16 *W2 = m->wb + m->off[2], *W3 = m->wb + m->off[4];
+    const __nv_bfloat16 *W2 = m->wb + m->woff[1], *W3 = m->wb + m->woff[2];
+    const int li = row_ld(m->n_in), l1 = row_ld(m->h1), l2 = row_ld(m->h2), lo = row_ld(m->n_out);
     k_loss_rows<<<B, 256, 0, s>>>(B, m->n_out, m->loss_kind == TMR_LOSS_PHASE, m->y, T, m->dyb, m->part);
     k_loss_finish<<<1, 256, 0, s>>>(B, m->part, (float)((size_t)B * m->n_out), loss);
     // dZ = (dZ_next W) .* GELU'(Z)
-    auto back = [&](const float *z, __nv_bfloat16 *dz) {
+    auto back = [&](const float *z, __nv_bfloat16 *dz, int ldz) {
         GemmEpilogue E;
         E.kind = GEMM_GELU_BACK;
         E.C = m->dh;
         E.Z = z;
         E.H = dz;
+        E.ldh = ldz;
         return E;
     };
-    // dW = dZ^T H: the gradient, or the update of the weights at offset o
-    auto weights = [&](size_t o) {
+    // dW = dZ^T H: the gradient, or the update of the layer's weights
+    auto weights = [&](int layer, int ldw) {
+        const size_t o = m->off[2 * layer];
         GemmEpilogue E;
         E.C = g + o;
         if (step) {
@@ -451,7 +501,8 @@ void backward_core(tmr_mlp *m, int B, const float *T, float *loss, float *g, con
             E.w = m->w + o;
             E.m = m->m + o;
             E.v = m->v + o;
-            E.H = m->wb + o;
+            E.H = m->wb + m->woff[layer];
+            E.ldh = ldw;
             E.lr = step->lr;
             E.c1 = step->c1;
             E.c2 = step->c2;
@@ -459,18 +510,18 @@ void backward_core(tmr_mlp *m, int B, const float *T, float *loss, float *g, con
         return E;
     };
     // every dZ is made before the weights it was made with change
-    gemm(m, B, m->h2, m->n_out, {m->dyb, m->n_out, true}, {W3, m->h2, false}, back(m->z2, m->dz2b));
-    gemm(m, m->n_out, m->h2, B, {m->dyb, m->n_out, false}, {m->h2b, m->h2, false}, weights(m->off[4]));
-    gemm(m, B, m->h1, m->h2, {m->dz2b, m->h2, true}, {W2, m->h1, false}, back(m->z1, m->dzb));
-    gemm(m, m->h2, m->h1, B, {m->dz2b, m->h2, false}, {m->h1b, m->h1, false}, weights(m->off[2]));
-    gemm(m, m->h1, m->n_in, B, {m->dzb, m->h1, false}, {m->xb, m->n_in, false}, weights(m->off[0]));
+    gemm(m, B, m->h2, m->n_out, {m->dyb, lo, true}, {W3, l2, false}, back(m->z2, m->dz2b, l2));
+    gemm(m, m->n_out, m->h2, B, {m->dyb, lo, false}, {m->h2b, l2, false}, weights(2, l2));
+    gemm(m, B, m->h1, m->h2, {m->dz2b, l2, true}, {W2, l1, false}, back(m->z1, m->dzb, l1));
+    gemm(m, m->h2, m->h1, B, {m->dz2b, l2, false}, {m->h1b, l1, false}, weights(1, l1));
+    gemm(m, m->h1, m->n_in, B, {m->dzb, l1, false}, {m->xb, li, false}, weights(0, li));
     BiasLayers L;
     const __nv_bfloat16 *dz[3] = {m->dzb, m->dz2b, m->dyb};
     const int width[3] = {m->h1, m->h2, m->n_out};
     int blocks = 0;
     for (int i = 0; i < 3; i++) {
         const size_t o = m->off[2 * i + 1];
-        L.l[i] = {dz[i], width[i], blocks, g + o, m->w + o, m->m + o, m->v + o, m->wb + o};
+        L.l[i] = {dz[i], width[i], blocks, g + o, m->w + o, m->m + o, m->v + o};
         blocks += (width[i] + 31) / 32;
     }
     k_bias_grad<<<blocks, dim3(32, 8), 0, s>>>(B, L, step != nullptr, step ? step->lr : 0.f, step ? step->c1 : 1.f,
@@ -518,11 +569,18 @@ tmr_status tmr_mlp_create(tmr_mlp **out, int n_in, int n_h1, int n_h2, int n_out
         o += sz[i];
     }
     m->np = o;
+    size_t nwb = 0;
+    const int fan[3][2] = {{n_h1, n_in}, {n_h2, n_h1}, {n_out, n_h2}};
+    for (int l = 0; l < 3; l++) {
+        m->woff[l] = nwb;
+        nwb += (size_t)fan[l][0] * row_ld(fan[l][1]);
+    }
     const bool ok = cudaMalloc(&m->w, sizeof(float) * o) == cudaSuccess &&
                     cudaMalloc(&m->m, sizeof(float) * o) == cudaSuccess &&
                     cudaMalloc(&m->v, sizeof(float) * o) == cudaSuccess &&
                     cudaMalloc(&m->g, sizeof(float) * o) == cudaSuccess &&
-                    cudaMalloc(&m->wb, sizeof(__nv_bfloat16) * o) == cudaSuccess &&
+                    cudaMalloc(&m->wb, sizeof(__nv_bfloat16) * nwb) == cudaSuccess &&
+                    cudaMemsetAsync(m->wb, 0, sizeof(__nv_bfloat16) * nwb, m->stream) == cudaSuccess &&
                     cudaMalloc(&m->lossd, sizeof(float) * 4) == cudaSuccess &&
                     cudaMalloc(&m->tc_err, sizeof(int)) == cudaSuccess &&
                     cudaMemset(m->tc_err, 0, sizeof(int)) == cudaSuccess;
@@ -563,7 +621,9 @@ tmr_status tmr_mlp_set_params(tmr_mlp *m, const float *params)
         cudaMemsetAsync(m->m, 0, sizeof(float) * m->np, m->stream) != cudaSuccess ||
         cudaMemsetAsync(m->v, 0, sizeof(float) * m->np, m->stream) != cudaSuccess)
         return mfail(TMR_ERR_CUDA, "set params");
-    k_to_bf16<<<ew_blocks(m->np), 256, 0, m->stream>>>(m->np, m->w, m->wb);
+    to_bf16(m->h1, m->n_in, m->w + m->off[0], m->wb + m->woff[0], m->stream);
+    to_bf16(m->h2, m->h1, m->w + m->off[2], m->wb + m->woff[1], m->stream);
+    to_bf16(m->n_out, m->h2, m->w + m->off[4], m->wb + m->woff[2], m->stream);
     m->step = 0;
     if (cudaStreamSynchronize(m->stream) != cudaSuccess) return mfail(TMR_ERR_CUDA, "set params sync");
     return TMR_OK;
@@ -589,7 +649,7 @@ tmr_status tmr_mlp_forward(tmr_mlp *m, const float *X, int B, float *Y)
     if (!dev_ptr(X) || !dev_ptr(Y)) return mfail(TMR_ERR_INVALID_ARG, "X and Y must be device memory");
     tmr_status st = ensure_batch(m, B);
     if (st != TMR_OK) return st;
-    k_to_bf16<<<ew_blocks((size_t)B * m->n_in), 256, 0, m->stream>>>((size_t)B * m->n_in, X, m->xb);
+    to_bf16(B, m->n_in, X, m->xb, m->stream);
     forward_core(m, B, Y);
     return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "forward kernels");
 }
@@ -605,7 +665,7 @@ static tmr_status mlp_batch(tmr_mlp *m, const float *X, const float *T, int B, f
         return mfail(TMR_ERR_INVALID_ARG, "arrays must be device memory");
     tmr_status st = ensure_batch(m, B);
     if (st != TMR_OK) return st;
-    k_to_bf16<<<ew_blocks((size_t)B * m->n_in), 256, 0, m->stream>>>((size_t)B * m->n_in, X, m->xb);
+    to_bf16(B, m->n_in, X, m->xb, m->stream);
     forward_core(m, B, m->y);
     backward_core(m, B, T, loss ? loss : m->lossd, grad ? grad : m->g, step);
     return cudaGetLastError() == cudaSuccess ? TMR_OK : mfail(TMR_ERR_CUDA, "network kernels");
