@@ -32,11 +32,10 @@ __device__ __forceinline__ float cost_coef(int cost, float2 z, float y, float &f
 __host__ __device__ __forceinline__ float cost_grad_scale(int cost) { return cost == COST_AMPLITUDE ? 2.f : -4.f; }
 
 // Half the first and second derivatives of phi(al) = sum (a - |z + al w|)^2
-// for one element, added to d1 and d2 (a term with |u| = 0 adds |w|^2 to d2
+// for one element (a = sqrt(y)), added to d1 and d2 (a term with |u| = 0 adds |w|^2 to d2
 // only, as in the gradient).
-__device__ __forceinline__ void amp_derivs(float2 z, float2 w, float y, float al, float &d1, float &d2)
+__device__ __forceinline__ void amp_derivs(float2 z, float2 w, float a, float al, float &d1, float &d2)
 {
-    const float a = sqrtf(fmaxf(y, 0.f));
     const float2 u = make_float2(fmaf(al, w.x, z.x), fmaf(al, w.y, z.y));
     const float m2 = cabs2(u), m = sqrtf(m2);
     const float cr = u.x * w.x + u.y * w.y, ci = u.x * w.y - u.y * w.x;  // conj(u) w
@@ -68,12 +67,15 @@ __device__ float amp_line_search(const float2 (&z)[E], const float2 (&w)[E], YAt
     float pv[32];
 #pragma unroll
     for (int q = 0; q < 32; q++) pv[q] = 0.f;
+    float a[E];  // held over the passes: the root is a quarter of a pass's work
 #pragma unroll
-    for (int e = 0; e < E; e++)
+    for (int e = 0; e < E; e++) {
+        a[e] = valid(e) ? sqrtf(fmaxf(yat(e), 0.f)) : 0.f;
         if (valid(e)) {
-            amp_derivs(z[e], w[e], yat(e), 0.f, pv[0], pv[1]);
-            amp_derivs(z[e], w[e], yat(e), 1.f, pv[2], pv[3]);
+            amp_derivs(z[e], w[e], a[e], 0.f, pv[0], pv[1]);
+            amp_derivs(z[e], w[e], a[e], 1.f, pv[2], pv[3]);
         }
+    }
     reduce(pv, 4);
     // thread 0's state, kept in registers of thread 0 only
     float lo = 0.f, hi = 0.f, x = 1.f, d1lo = red[0], d2lo = red[1], d1 = red[2], d2 = red[3];
@@ -130,7 +132,7 @@ __device__ float amp_line_search(const float2 (&z)[E], const float2 (&w)[E], YAt
         for (int q = 0; q < 2; q++) pv[q] = 0.f;
 #pragma unroll
         for (int e = 0; e < E; e++)
-            if (valid(e)) amp_derivs(z[e], w[e], yat(e), al, pv[0], pv[1]);
+            if (valid(e)) amp_derivs(z[e], w[e], a[e], al, pv[0], pv[1]);
         reduce(pv, 2);
         d1 = red[0];
         d2 = red[1];

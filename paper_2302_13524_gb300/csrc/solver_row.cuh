@@ -380,9 +380,17 @@ __global__ void __launch_bounds__(512, 1) k_solver_row(SolverParams P)
         __syncthreads();
         float acc = 0.f;
         if (tid < nv) {
+            // at most 16 warps, the loads in flight together; the amplitude cost's line
+            // search, which holds its fields through a dozen reductions an
+            // iteration, has registers for four at a time
+            constexpr int U = COST == COST_AMPLITUDE ? 4 : 16;
 #pragma unroll
-            for (int w = 0; w < 16; w++)  // at most 16 warps: the loads are in flight together
-                if (w < NW) acc += red[tid * NW + w];
+            for (int w0 = 0; w0 < 16; w0 += U) {
+                if (w0 >= NW) break;
+#pragma unroll
+                for (int w = w0; w < w0 + U; w++)
+                    if (w < NW) acc += red[tid * NW + w];
+            }
         }
         if constexpr (CLU) {
             // the CTAs' sums into every CTA's part, then added in rank order
