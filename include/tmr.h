@@ -228,10 +228,11 @@ void tmr_default_options(tmr_options *opt);
 
 /* Create a handle for M rows of length N probed with J masks.  With
  * opt->schedule == 0 the first handle for a (device, N, J, m) times every
- * solver schedule that fits (G masks per CTA with a cluster of J/G CTAs per
- * row, and one CTA per row) on synthetic rows and keeps the fastest; the
- * choice is cached in memory and, when opt->tune_cache names a file, in that
- * JSON file.
+ * solver schedule that fits (see opt->schedule) on synthetic rows and keeps the
+ * fastest; the choice is cached in memory and, when opt->tune_cache names a
+ * file, in that JSON file.  Where schedule 64 is one of them, handles of so few
+ * rows that M J is at most twice the number of SMs are timed at their own M and
+ * cached by it.
  *   masks      complex64 [J][N], |d| = 1 (not checked), copied.
  *   defocus_op NULL: no phase-offset fit; else copied (H copied).
  *   opt        NULL: defaults.
@@ -378,7 +379,7 @@ long long tmr_learned_rows(tmr_handle *h);
 int tmr_schedule(const tmr_handle *h);
 /* The schedules the autotuner timed when this handle was made, and the mean
  * time of their timed runs in milliseconds (each: 4 power and 6 L-BFGS
- * iterations on 608 synthetic rows): writes up to cap entries, returns their
+ * iterations on 608 synthetic rows, or on M where tmr_create says so): writes up to cap entries, returns their
  * number (0 when the schedule was given, cached, or the only one). */
 int tmr_autotune_report(const tmr_handle *h, int *codes, float *ms, int cap);
 

@@ -246,9 +246,20 @@ bool schedule_ok(int N, int J, int m, int G, int smem_optin, int prec = 0, int c
     return b > 0 && b <= (size_t)smem_optin;
 }
 
-// Time every valid schedule on synthetic rows (spectral start, a few power
+// Rows that the autotuner times its candidates on: 608, four for each SM, or the
+// handle's own where the row layout over a cluster is a candidate and they are too
+// few to fill the chip twice at one mask per CTA.  That layout gives a row half
+// or a quarter of the SMs, which pays by the rows that run beside it (N = 4096, J =
+// 4, 10 iterations: up to 30 rows 142 us at one mask per CTA and 206 so; 37 rows, in
+// two waves there, 267 and 205).
+int tune_rows(int M, int J, int nsm, bool cluster_layout)
+{
+    return cluster_layout && (long long)M * J <= 2LL * nsm ? (M > 0 ? M : 1) : 608;
+}
+
+// Time every valid schedule on R synthetic rows (spectral start, a few power
 // and L-BFGS iterations) and return the fastest.
-tmr_status autotune(tmr_handle *h, int smem_optin, int *G_out, bool *timed)
+tmr_status autotune(tmr_handle *h, int smem_optin, int R, int *G_out, bool *timed)
 {
     *timed = false;
     int cand[6], nc = 0;
@@ -265,7 +276,6 @@ tmr_status autotune(tmr_handle *h, int smem_optin, int *G_out, bool *timed)
         *timed = true;
         return TMR_OK;
     }
-    const int R = 608;
     const size_t K = (size_t)h->J * h->N;
     // the timing rows are temporary device memory of the handle: under a
     // workspace_limit they must fit in what is left, else the first
@@ -642,7 +652,11 @@ tmr_status tmr_create(tmr_handle **out, int N, int M, int J, const void *masks,
     if (o.schedule != 0) {
         h->G = o.schedule;
     } else {
-        const std::string key = tune_key(dev, N, J, o.m, h->xk, o.cost);
+        int nsm = 0;
+        TMR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev), "attr");
+        const int R = tune_rows(M, J, nsm, schedule_ok(N, J, o.m, kRowClusterSchedule, smem_optin, h->xk, o.cost));
+        std::string key = tune_key(dev, N, J, o.m, h->xk, o.cost);
+        if (R != 608) key += "|rows" + std::to_string(R);  // a choice of its own
         int G = 0;
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -658,7 +672,7 @@ tmr_status tmr_create(tmr_handle **out, int N, int M, int J, const void *masks,
         }
         bool timed = true;  // a cached choice was timed when it was made
         if (!G) {
-            TRY(autotune(h, smem_optin, &G, &timed));
+            TRY(autotune(h, smem_optin, R, &G, &timed));
             if (timed) {
                 std::lock_guard<std::mutex> lk(g_tune_mu);
                 g_tune_mem[key] = G;
