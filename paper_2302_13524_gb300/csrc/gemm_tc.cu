@@ -6,7 +6,8 @@
 //   C[M][N] (FP32, row stride ldc) = sum_k A(m, k) B(n, k).  Each operand is
 //   stored either K-contiguous (A [M][K], B [N][K]) or K-strided (A [K][M],
 //   B [K][N]); both forms feed the tensor cores straight from memory (K-major
-//   or MN-major shared-memory tiles), so no operand is transposed first.
+//   or MN-major shared-memory tiles), so no operand is transposed first.  (A
+//   K-strided with B K-contiguous, which no product of the network has, is left out.)
 //
 // One CTA computes one 128 x BN tile of C with 4 warps:
 //   warp 0, one lane: TMA producer.  Each k-step of 64 elements loads a
@@ -478,6 +479,7 @@ bool make_map(CUtensorMap *map, const __nv_bfloat16 *ptr, int rows, int cols, in
 bool gemm_tc_supported(int M, int N, int K, const GemmOperand &A, const GemmOperand &B)
 {
     if (M < kBM || N < 128 || K < kBK) return false;
+    if (!A.k_contiguous && B.k_contiguous) return false;  // no product has this pair of forms
     // rows that start on 16-byte boundaries (their length may be any: TMA fills what is past it)
     const int ca = A.k_contiguous ? K : M, cb = B.k_contiguous ? K : N;
     if (A.ld % 8 || B.ld % 8 || A.ld < ca || B.ld < cb) return false;
@@ -561,8 +563,6 @@ cudaError_t gemm_tc(int M, int N, int K, const GemmOperand &A, const GemmOperand
     if (A.k_contiguous && B.k_contiguous)
         return bn == 128 ? TMR_GEMM(128, false, false) : bn == 64 ? TMR_GEMM(64, false, false) : TMR_GEMM(32, false, false);
     if (A.k_contiguous) return bn == 128 ? TMR_GEMM(128, false, true) : TMR_GEMM(64, false, true);
-    if (B.k_contiguous)
-        return bn == 128 ? TMR_GEMM(128, true, false) : bn == 64 ? TMR_GEMM(64, true, false) : TMR_GEMM(32, true, false);
     return bn == 128 ? TMR_GEMM(128, true, true) : TMR_GEMM(64, true, true);
 #undef TMR_GEMM
 }

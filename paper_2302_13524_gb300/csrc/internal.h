@@ -163,8 +163,8 @@ cudaError_t launch_fill_synthetic(float *y, size_t n, unsigned seed, cudaStream_
 // C[M][N] (FP32, row stride ldc) = sum_k A(m, k) B(n, k), then an elementwise
 // step.  An operand is BF16 with rows of stride ld elements: [M or N][K]
 // (k_contiguous) or [K][M or N].  Needs M, N >= 128, K >= 64, 16-byte aligned
-// pointers and rows (ld a multiple of 8, no shorter than the row); *err (device)
-// is raised when a barrier wait ran out.
+// pointers and rows (ld a multiple of 8, no shorter than the row), and not A
+// K-strided with B K-contiguous; *err (device) is raised when a barrier wait ran out.
 struct GemmOperand {
     const __nv_bfloat16 *p;
     int ld;
