@@ -843,8 +843,11 @@ __global__ void __launch_bounds__(SolverCfg<Xf, G>::BT, solver_min_ctas<Xf, G>()
             }
 
             // ---- f and gradient at t (the start; in a mixed-precision run also the
-            // switch to the FP32 transforms, which restarts the history) ----
-            auto eval_at_t = [&]() {
+            // switch to the FP32 transforms, which restarts the history).  Inlined whatever
+            // its size: as a function of its own it takes the row's registers by
+            // address, and they all live in local memory then (mixed precision,
+            // N = 4096, 304 rows, J = 6, 10 power steps: 3.63 ms instead of 1.75) ----
+            auto eval_at_t = [&]() __attribute__((always_inline)) {
                 __syncthreads();
                 push_slice_to_X(ts);
                 cluster.sync();
