@@ -425,9 +425,13 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
     const int hid = m->h1 > m->h2 ? m->h1 : m->h2, io = m->n_in > m->n_out ? m->n_in : m->n_out;
     const int hmax = io > hid ? io : hid;
     const size_t rows = (size_t)B;
+    bool zeroed = false;
     auto padded = [&](__nv_bfloat16 **p, int width) {
         const size_t bytes = sizeof(__nv_bfloat16) * rows * row_ld(width);
-        return cudaMalloc(p, bytes) == cudaSuccess && cudaMemsetAsync(*p, 0, bytes, m->stream) == cudaSuccess;
+        if (cudaMalloc(p, bytes) != cudaSuccess) return false;
+        if (row_ld(width) == width) return true;
+        zeroed = true;
+        return cudaMemsetAsync(*p, 0, bytes, m->stream) == cudaSuccess;
     };
     bool ok = padded(&m->xb, m->n_in) && padded(&m->h1b, m->h1) && padded(&m->h2b, m->h2) && padded(&m->dzb, m->h1) &&
               padded(&m->dz2b, m->h2) && padded(&m->dyb, m->n_out) &&
@@ -436,7 +440,8 @@ tmr_status ensure_batch(tmr_mlp *m, int B)
               cudaMalloc(&m->y, sizeof(float) * rows * m->n_out) == cudaSuccess &&
               cudaMalloc(&m->dh, sizeof(float) * rows * hmax) == cudaSuccess &&
               cudaMalloc(&m->part, sizeof(float) * rows) == cudaSuccess &&
-              cudaStreamSynchronize(m->stream) == cudaSuccess;  // mlp_propose goes on on another stream
+              // mlp_propose goes on on another stream
+              (!zeroed || cudaStreamSynchronize(m->stream) == cudaSuccess);
     if (!ok) {
         cudaGetLastError();
         return mfail(TMR_ERR_OOM, "MLP batch buffers");
