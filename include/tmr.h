@@ -253,7 +253,10 @@ tmr_status tmr_create(tmr_handle **out, int N, int M, int J, const void *masks,
                       void *stream);
 
 /* Forward model (Eq. optTMsmall2): Y[r][j][k] = |F(d_j .* T[r])[k]|^2.
- *   T complex64 [M][N] in, Y float32 [M][J][N] out. */
+ *   T complex64 [M][N] in, Y float32 [M][J][N] out.
+ * Here and in tmr_grad the transform's layout follows the number of rows in the
+ * call, so a matrix taken in several calls agrees with one call to FP32 rounding,
+ * not bit for bit; repeated calls of the same shape do. */
 tmr_status tmr_forward(tmr_handle *h, const void *T, float *Y);
 
 /* Loss and gradient (Eq. optTMsmall2, Eq. derivative, App. A):

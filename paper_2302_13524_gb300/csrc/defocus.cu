@@ -947,10 +947,10 @@ __device__ void pf_eval(const PhaseFitParams &Pp, const PFWork &W, float2 *g, co
 // the same FP64 L-BFGS scalars (identical sums in identical order), so all
 // take the same decisions.
 //
-// Bound by latency, not by a rate: a fit is a few evaluations in a row, each a
-// chain of about 60 FFT stages of one grid with a block barrier between them,
-// and the CTAs past the Nd patterns only help with the chunk-owned vectors.  So
-// what counts is each stage's instructions: index arithmetic by shifts, neighbouring
+// Bound by latency, not by a rate: a fit is a few evaluations in a row, each for
+// every pattern a chain of passes over one grid with a block barrier between them
+// (13 for the same-grid operator at 128 x 64, 56 for the padded one), by min(Nd,
+// SMs) CTAs.  So what counts is each stage's instructions: index arithmetic by shifts, neighbouring
 // passes of the same axis (last inverse stage, the product, first forward
 // stage) in one, H and full-length twiddle tables in shared memory, and the
 // FP64 scalars, on a pipe of two lanes a cycle, by one warp in registers.

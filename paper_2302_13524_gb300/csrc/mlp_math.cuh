@@ -18,8 +18,8 @@ __device__ __forceinline__ float gelu_grad_f(float x)
 // rounds back to m): in a long training run that made the weight updates, which
 // are bound by memory otherwise, twice as slow (a step of batch 256, 8192 x 1024 x
 // 1024 x 4096, after a thousand steps with its weights read back: 424 us against
-// 284 at the start of the run; 263 now throughout, with the tiles of gemm_tc.cu).  So the operands are kept out of
-// that range without moving the result: below 1e-31, sqrt(v / c2) is less than
+// 284 at the start of the run; 260 now throughout, with the tiles of gemm_tc.cu).
+// So the operands are kept out of that range without moving the result: below 1e-31, sqrt(v / c2) is less than
 // half an ulp of eps, and a small m is scaled by a power of two around the
 // divisions.
 __device__ __forceinline__ void adam_update(float &w, float g, float &m, float &v, float lr, float c1, float c2)

@@ -220,7 +220,7 @@ __device__ __forceinline__ float sqrt_approx(float x)
 // when c4 <= 0 or a root comes out non-finite.
 //
 // One warp runs this between two block barriers of every iteration, so its
-// latency is all that counts, hence no IEEE divisions, cbrtf, acosf or ldexpf in
+// latency is all that counts, hence no IEEE divisions, cbrtf, cosf or ldexpf in
 // the chain.  With the bookkeeping below also in registers: 20 iterations of
 // 4096 rows at N = 4096, J = 4, one mask per CTA, 33.1 -> 29.0 ms.
 static __device__ float quartic_argmin_warp(const float *c, int lane)

@@ -35,7 +35,9 @@
 // quarter of the SMs that one mask per CTA (solver_impl.cuh) gives it, and the
 // serial parts of an iteration (reductions, scalars, barriers: half of it at one
 // mask per CTA) are shared by that many more rows.  N = 4096, J = 4, M = 4096,
-// 20 iterations: 21.6 ms against 29.0 (19.6 with the fields in tensor memory, ZT below).
+// 20 iterations: 21.6 ms against 29.0 (19.4 with the fields in tensor memory, ZT below).
+// For a few rows, which do not fill the chip either way, it is the slower one: see
+// tune_rows in api.cu.
 #pragma once
 
 #include "solver_impl.cuh"

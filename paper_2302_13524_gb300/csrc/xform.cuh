@@ -97,7 +97,7 @@ struct XfPow2 {
 
 // XfPow2W<N>: the same transform with 16 points per thread, N = 512 .. 4096, for
 // the streaming kernels: a first pass of the remaining radix and radix-16
-// passes, two exchanges (one for 512 and less) where XfPow2 has three.  What
+// passes, two exchanges for every length where XfPow2 has three (two at 512).  What
 // bounds those kernels is the shared-memory traffic of the exchanges and the
 // instructions around them.  Its constants stand behind XfPow2's in the table:
 // [ twiddles of the middle pass | bases exp(-2 pi i k t / N), t < NT, for k = 1, 2,
@@ -517,7 +517,11 @@ __host__ __device__ constexpr int comp_teams(int A)
 // L = 512, 1024, 2048, 4096, the split outputs and 8192 take 74, 163, 333, 770,
 // 940, 1460.  At N = 2286 (18 x 127), J = 4: gradient of 8192 rows 2556 us with
 // the split outputs and their FP64 setup, 2227 without the latter, 1681 so (1610
-// with packed additions); a retrieval of 2048 rows with early exit 54.1 -> 39.7 ms.
+// with packed additions); a retrieval of 2048 rows with early exit 54.1 -> 37.9 ms
+// (with the slices' owners by FP32 products).  What the lengths up to 256 lose: a
+// forward call of a few dozen rows, one short wave of single warps, takes 8.2 us
+// against 6.2 with plain Bluestein (J = 1 .. 4, up to 30 rows; 100 rows equal, 400 rows
+// and J = 8 14.4 against 20.5).
 __host__ __device__ inline bool comp_shape(int N, int *A, int *B)
 {
     const int most = N <= 256 ? 2 : N <= 512 ? 4 : N <= 1024 ? 12 : N <= 2048 ? 18 : N <= kBlueSplitMaxN ? 24 : 32;
